@@ -293,7 +293,7 @@ cl_status cl_lbm_solve_krylov(cl_handle h, double tol, int max_iter, long long m
    axial, 1/36 diagonal; 2 w_i on a fixed-concentration face, (1 - r) w_i
    on a catalytic face, 0 on a bounce-back face).  The preconditioner
    P v = v + w_i eps with L eps = sum_i v_i (diagonal-preconditioned
-   conjugate gradients to 1e-2) keeps the number of step applications
+   conjugate gradients to 1e-1) keeps the number of step applications
    small as the box grows (it levels off near 100) and with a spread of
    relaxation times (Knudsen): 15 for the bulk-D 48^3 Pt layer, about 80
    for Knudsen layers of 24^3 and 32^3, where the unpreconditioned solve
@@ -304,8 +304,10 @@ cl_status cl_lbm_solve_krylov(cl_handle h, double tol, int max_iter, long long m
      iterations:       nullable; GMRES iterations (step applications).
      inner_iterations: nullable; conjugate-gradient iterations in all.
    Needs CL_STORAGE_FP32POP, else CL_ERR_STATE.  Allocates 64 f32
-   and 2 FP64 population-sized vectors plus 6 f32 cell fields for the call
-   (through p->alloc if given) and frees them before returning.
+   population vectors over the active cells, 1 f32 and 2 FP64 ones over the
+   box, and their link lists for the call (through p->alloc if given) and
+   frees them before returning.  Its kernels wait on one another with a
+   bound (CL_ERR_TIMEOUT).
    Errors: as cl_lbm_solve_krylov. */
 cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long long max_steps, cl_solve_info* info,
                                   int* iterations, long long* inner_iterations);

@@ -1083,152 +1083,117 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
     const int nblk = kry_blocks();
     constexpr int kM = 30;           // Krylov vectors per GMRES cycle
     constexpr int kMaxCycles = 10;   // cycles per correction
-    constexpr int kCgBatch = 8;      // CG iterations between host reads
     constexpr int kMaxCg = 4000;     // CG iterations per preconditioner application
-    const double kCgTol = 1e-2;      // relative residual of the inner CG solve
+    const double kCgTol = 1e-1;      // relative residual of the inner CG solve (see dsa.cuh)
     int iters = 0;
     long long cg_total = 0;
     {
         Scratch sc(h);
-        float* V[kM + 1];
-        float* Z[kM];
-        for (int k = 0; k <= kM; ++k) CKS(sc.get((void**)&V[k], sizeof(float) * (size_t)L));
-        for (int k = 0; k < kM; ++k) CKS(sc.get((void**)&Z[k], sizeof(float) * (size_t)L));
-        float *wv = nullptr, *e = nullptr, *c = nullptr;
-        CKS(sc.get((void**)&wv, sizeof(float) * (size_t)L));
-        CKS(sc.get((void**)&e, sizeof(float) * (size_t)L));
-        CKS(sc.get((void**)&c, sizeof(float) * (size_t)L));
-        float* cell[6];  // eps, r, z, p, q of the inner CG, and 1/diag(L)
-        for (int k = 0; k < 6; ++k) {
-            CKS(sc.get((void**)&cell[k], sizeof(float) * (size_t)N));
-            CK(cudaMemsetAsync(cell[k], 0, sizeof(float) * (size_t)N, h->s));
+        // the active cells (dsa.cuh); every f32 vector below holds only those
+        const StepArgs a7 = q19 ? StepArgs() : make_args(h);
+        const Q19Args a19 = q19 ? make_args19(h) : Q19Args();
+        const uint16_t* m7 = q19 ? nullptr : h->mask;
+        const uint32_t* m19 = q19 ? h->mask19 : nullptr;
+        DsaCells d;
+        d.q = q19 ? 19 : 7;
+        int* scan = nullptr;
+        const int nscan = dsa_scan_blocks(N);
+        CKS(sc.get((void**)&scan, sizeof(int) * (size_t)(nscan + 1)));
+        CKS(sc.get((void**)&d.inv, sizeof(int) * (size_t)N));
+        CK(launch_dsa_count(m7, m19, N, scan, scan + nscan, h->s));
+        CK(cudaMemcpyAsync(&d.n, scan + nscan, sizeof(int), cudaMemcpyDeviceToHost, h->s));
+        CK(cudaStreamSynchronize(h->s));
+        const size_t n = (size_t)d.n;
+        d.np = (d.n + 31) / 32 * 32;
+        const long long Lc = (long long)d.q * d.np;  // elements of a vector
+        CKS(sc.get((void**)&d.list, sizeof(int) * n));
+        CKS(sc.get((void**)&d.nb, sizeof(int) * n * (d.q - 1)));
+        CKS(sc.get((void**)&d.sink, sizeof(float) * n));
+        CKS(sc.get((void**)&d.dinv, sizeof(float) * n));
+        CKS(sc.get((void**)&d.omega, sizeof(float) * n));
+        CK(launch_dsa_number(m7, m19, N, scan, d.inv, d.list, h->s));
+        CK(q19 ? launch_dsa_links19(d, a19, h->s) : launch_dsa_links7(d, a7, h->s));
+        // V (kM + 1) and Z (kM) of the GMRES cycle, w, e and c: one allocation, pads zero
+        float* vecs = nullptr;
+        CKS(sc.get((void**)&vecs, sizeof(float) * (size_t)Lc * (2 * kM + 4)));
+        CK(cudaMemsetAsync(vecs, 0, sizeof(float) * (size_t)Lc * (2 * kM + 4), h->s));
+        float* V = vecs;
+        float* Z = V + (size_t)Lc * (kM + 1);
+        float *wv = Z + (size_t)Lc * kM, *e = wv + Lc, *c = e + Lc;
+        float* cfull = nullptr;  // the residual in the population layout
+        CKS(sc.get((void**)&cfull, sizeof(float) * (size_t)L));
+        PcgArgs<float> cg;
+        memset(&cg, 0, sizeof(cg));
+        cg.tol2 = kCgTol * kCgTol;
+        cg.max_iters = kMaxCg;
+        CKS(sc.get((void**)&cg.u, sizeof(float) * n));
+        if (dsa_prec_streams(d.n)) {
+            CKS(sc.get((void**)&cg.x, sizeof(float) * n));
+            CKS(sc.get((void**)&cg.r, sizeof(float) * n));
+            CKS(sc.get((void**)&cg.p, sizeof(float) * n));
+            CKS(sc.get((void**)&cg.s, sizeof(float) * n));
+            CKS(sc.get((void**)&cg.w, sizeof(float) * n));
         }
-        float *eps = cell[0], *rc = cell[1], *zc = cell[2], *pc = cell[3], *qc = cell[4], *dinv = cell[5];
-        double *x64 = nullptr, *y64 = nullptr, *part = nullptr, *dH = nullptr, *dnrm = nullptr, *dy = nullptr;
+        cg.meet_blocks = dsa_mgs_blocks();
+        CKS(sc.get(&cg.meet_mem, pcg_meet_bytes(cg.meet_blocks)));
+        CKS(sc.get((void**)&cg.out, sizeof(PcgOut)));
+        double *x64 = nullptr, *y64 = nullptr, *part = nullptr, *dcol = nullptr, *dnrm = nullptr, *dy = nullptr;
         KryScalars* ks = nullptr;
-        CgScalars* cs = nullptr;
         CKS(sc.get((void**)&x64, sizeof(double) * (size_t)L));
         CKS(sc.get((void**)&y64, sizeof(double) * (size_t)L));
         CK(cudaMemsetAsync(y64, 0, sizeof(double) * (size_t)L, h->s));
         CKS(sc.get((void**)&part, sizeof(double) * 2 * (size_t)nblk));
-        CKS(sc.get((void**)&dH, sizeof(double) * (kM + 1) * kM));
+        CKS(sc.get((void**)&dcol, sizeof(double) * (kM + 1)));
         CKS(sc.get((void**)&dnrm, sizeof(double)));
         CKS(sc.get((void**)&dy, sizeof(double) * kM));
         CKS(sc.get((void**)&ks, sizeof(KryScalars)));
-        CKS(sc.get((void**)&cs, sizeof(CgScalars)));
         CK(cudaMemsetAsync(ks, 0, sizeof(KryScalars), h->s));
-        CK(cudaMemsetAsync(cs, 0, sizeof(CgScalars), h->s));
         float* x = h->pop[h->cur];
-        float* u = h->pop[h->cur ^ 1];  // A(.) output; the next step of the march rewrites it
-        DsaArgs da;
-        da.nx = h->nx; da.ny = h->ny; da.nz = h->nz; da.N = N;
-        da.mask = h->mask;
-        da.rfac = reactive_factor(h);
-        da.rsink = (float)reactive_sink_d(h);
-        da.bc_in = h->p.bc_in; da.bc_out = h->p.bc_out;
-        da.kscale = h->kscale;
-        da.k_lu = h->k_lu;
-        Dsa19 d19;
-        d19.px = h->px19;
-        d19.mask = h->mask19;
-        d19.react = h->react19;
-        CK(q19 ? launch_lap_dinv19(da, d19, dinv, nblk, h->s) : launch_lap_dinv(da, dinv, nblk, h->s));
-        auto host_double = [&](const double* dptr, double* out, int n) -> cl_status {
-            CK(cudaMemcpyAsync(out, dptr, sizeof(double) * n, cudaMemcpyDeviceToHost, h->s));
+        auto host_double = [&](const double* dptr, double* out, int cnt) -> cl_status {
+            CK(cudaMemcpyAsync(out, dptr, sizeof(double) * cnt, cudaMemcpyDeviceToHost, h->s));
             CK(cudaStreamSynchronize(h->s));
-            return CL_OK;
-        };
-        // kCgBatch CG iterations on the fixed cell buffers, captured once and
-        // replayed as one CUDA graph (five launches per iteration otherwise
-        // cost more than the iteration's own memory traffic on small boxes)
-        auto enqueue_cg = [&](cudaStream_t st) -> cudaError_t {
-            for (int k = 0; k < kCgBatch; ++k) {
-                const cudaError_t ce = q19 ? launch_cg_iter19(da, d19, dinv, eps, rc, zc, pc, qc, nblk, part, cs, st)
-                                           : launch_cg_iter(da, dinv, eps, rc, zc, pc, qc, nblk, part, cs, st);
-                if (ce != cudaSuccess) return ce;
-            }
-            return cudaSuccess;
-        };
-        cudaGraphExec_t cg_graph = nullptr;
-        struct GraphGuard {
-            cudaGraphExec_t* g;
-            ~GraphGuard() { if (*g) cudaGraphExecDestroy(*g); }
-        } guard{&cg_graph};
-        {
-            cudaStream_t cap = nullptr;
-            cudaGraph_t g = nullptr;
-            bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess;
-            if (ok) ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-            if (ok) {
-                const cudaError_t ce = enqueue_cg(cap);
-                ok = cudaStreamEndCapture(cap, &g) == cudaSuccess && g && ce == cudaSuccess;
-            }
-            if (ok) ok = cudaGraphInstantiate(&cg_graph, g, 0) == cudaSuccess;
-            if (g) cudaGraphDestroy(g);
-            if (cap) cudaStreamDestroy(cap);
-            if (!ok) {
-                cg_graph = nullptr;
-                cudaGetLastError();  // the same kernels then run as plain launches
-            }
-        }
-        // P v = v + w_i eps, L eps = sum_i v_i to kCgTol by diagonal-preconditioned CG
-        auto precondition = [&](const float* v, float* zout) -> cl_status {
-            CK(q19 ? launch_cg_start19(da, d19, v, dinv, eps, rc, zc, pc, nblk, part, cs, h->s)
-                   : launch_cg_start(da, v, dinv, eps, rc, zc, pc, nblk, part, cs, h->s));
-            CgScalars hc;
-            CK(cudaMemcpyAsync(&hc, cs, sizeof(hc), cudaMemcpyDeviceToHost, h->s));
-            CK(cudaStreamSynchronize(h->s));
-            while (!hc.bad && hc.iters < kMaxCg && hc.rr > kCgTol * kCgTol * hc.rr0) {
-                if (cg_graph) CK(cudaGraphLaunch(cg_graph, h->s));
-                else CK(enqueue_cg(h->s));
-                CK(cudaMemcpyAsync(&hc, cs, sizeof(hc), cudaMemcpyDeviceToHost, h->s));
-                CK(cudaStreamSynchronize(h->s));
-            }
-            cg_total += hc.iters;
-            CK(q19 ? launch_prec_out19(N, v, eps, zout, nblk, h->s) : launch_prec_out(N, v, eps, zout, nblk, h->s));
             return CL_OK;
         };
         // flexible GMRES(kM) in f32 on (I - A) e = c from e = 0, to tol_in times |c|
         auto correct = [&](double tol_in) -> cl_status {
-            CK(cudaMemsetAsync(e, 0, sizeof(float) * (size_t)L, h->s));
+            CK(cudaMemsetAsync(e, 0, sizeof(float) * (size_t)Lc, h->s));
             double beta0 = 0.0;
-            CK(launch_dot_dev(c, c, L, nblk, part, dnrm, 1, h->s));
+            CK(launch_dot_dev(c, c, Lc, nblk, part, dnrm, 1, h->s));
             CKS(host_double(dnrm, &beta0, 1));
             if (!(beta0 > 0.0) || !isfinite(beta0)) return CL_OK;
             double H[kM + 1][kM], cs_[kM], sn_[kM], g[kM + 1], col[kM + 1], y[kM];
             for (int cyc = 0; cyc < kMaxCycles && iters < max_iter; ++cyc) {
                 double beta = 0.0;
                 if (cyc == 0) {
-                    CK(launch_scale_dev(V[0], c, dnrm, L, nblk, h->s));
+                    CK(launch_scale_dev(V, c, dnrm, Lc, nblk, h->s));
                     beta = beta0;
                 } else {
-                    CK(step_pop(h, e, u, true));
-                    CK(launch_comb(c, e, u, wv, L, nblk, h->s));  // c - (I - A) e
-                    CK(launch_dot_dev(wv, wv, L, nblk, part, dnrm, 1, h->s));
+                    CK(launch_dsa_apply(d, e, wv, h->s));
+                    CK(launch_sub(c, wv, wv, Lc, nblk, h->s));  // c - (I - A) e
+                    CK(launch_dot_dev(wv, wv, Lc, nblk, part, dnrm, 1, h->s));
                     CKS(host_double(dnrm, &beta, 1));
                     if (!isfinite(beta)) break;
                     if (beta <= tol_in * beta0) break;
-                    CK(launch_scale_dev(V[0], wv, dnrm, L, nblk, h->s));
+                    CK(launch_scale_dev(V, wv, dnrm, Lc, nblk, h->s));
                 }
                 for (int k = 0; k <= kM; ++k) g[k] = 0.0;
                 g[0] = beta;
                 int jend = 0;
                 double resid = beta;
                 for (int j = 0; j < kM && iters < max_iter; ++j) {
-                    CKS(precondition(V[j], Z[j]));
-                    CK(step_pop(h, Z[j], u, true));
-                    CK(launch_comb(Z[j], u, nullptr, wv, L, nblk, h->s));  // (I - A) Z_j
+                    float* zj = Z + (size_t)j * Lc;
+                    CK(launch_dsa_prec(d, V + (size_t)j * Lc, zj, cg, h->s));
+                    CK(launch_dsa_apply(d, zj, wv, h->s));  // (I - A) Z_j
                     ++iters;
-                    // modified Gram-Schmidt, coefficients kept on the device
-                    for (int k = 0; k <= j; ++k) {
-                        double* hk = dH + k + (kM + 1) * j;
-                        CK(launch_dot_dev(V[k], wv, L, nblk, part, hk, 0, h->s));
-                        CK(launch_axpy_dev(wv, V[k], hk, -1.f, L, nblk, h->s));
+                    CK(launch_dsa_mgs(V, Lc, j, wv, Lc, dcol, cg.meet_mem, h->s));
+                    PcgOut po;
+                    CK(cudaMemcpyAsync(&po, cg.out, sizeof(po), cudaMemcpyDeviceToHost, h->s));
+                    CKS(host_double(dcol, col, j + 2));
+                    cg_total += po.iters;
+                    if (po.bad == 3 || col[j + 1] < 0.0) {
+                        set_msg_txt("a wait of the steady solve's blocks for one another ran out");
+                        return CL_ERR_TIMEOUT;
                     }
-                    double* hn = dH + (j + 1) + (kM + 1) * j;
-                    CK(launch_dot_dev(wv, wv, L, nblk, part, hn, 1, h->s));
-                    CK(launch_scale_dev(V[j + 1], wv, hn, L, nblk, h->s));
-                    CKS(host_double(dH + (kM + 1) * j, col, j + 2));
                     // Givens rotations: the earlier ones, then a new one that zeroes col[j + 1]
                     for (int k = 0; k < j; ++k) {
                         const double a = cs_[k] * col[k] + sn_[k] * col[k + 1];
@@ -1256,7 +1221,7 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
                     y[k] = t / H[k][k];
                 }
                 CK(cudaMemcpyAsync(dy, y, sizeof(double) * jend, cudaMemcpyHostToDevice, h->s));
-                for (int k = 0; k < jend; ++k) CK(launch_axpy_dev(e, Z[k], dy + k, 1.f, L, nblk, h->s));
+                CK(launch_dsa_update(e, Z, Lc, jend, dy, Lc, h->s));
                 CK(cudaStreamSynchronize(h->s));  // y lives on the host stack
                 if (resid <= tol_in * beta0) break;
             }
@@ -1270,18 +1235,19 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
         KryScalars hs;
         for (int ref = 0; ref < kMaxRefine; ++ref) {
             CK(step_f64(h, x64, y64));
-            CK(launch_kry_res64(x64, y64, c, L, nblk, part, ks, h->s));
+            CK(launch_kry_res64(x64, y64, cfull, L, nblk, part, ks, h->s));
             CK(cudaMemcpyAsync(&hs, ks, sizeof(hs), cudaMemcpyDeviceToHost, h->s));
             CK(cudaStreamSynchronize(h->s));
             if (!(hs.rr < rr_prev)) {
-                if (ref > 0) CK(launch_kry_add64(x64, e, -1.0, L, nblk, h->s));
+                if (ref > 0) CK(launch_dsa_add64(d, e, -1.0, N, x64, h->s));
                 break;
             }
             if (rr0 < 0.0) rr0 = hs.rr;
             if (hs.rr <= tol2 * rr0 || iters >= max_iter || !(hs.rr < 0.25 * rr_prev)) break;
             rr_prev = hs.rr;
+            CK(launch_dsa_gather(d, cfull, N, c, h->s));
             CKS(correct(kKryInnerTol));
-            CK(launch_kry_add64(x64, e, 1.0, L, nblk, h->s));
+            CK(launch_dsa_add64(d, e, 1.0, N, x64, h->s));
         }
         CK(launch_kry_to32(x64, x, L, nblk, h->s));
     }

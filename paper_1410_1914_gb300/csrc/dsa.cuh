@@ -1,31 +1,62 @@
-// Diffusion preconditioner of the Krylov steady solve on the paper's D3Q19
-// lattice (Eq. 22-24): the D3Q7 kernels' counterparts that depend on the
-// lattice (the Laplacian row, the cell sums of the populations, the
-// equilibrium-shaped correction).  The CG update, direction and scalar
-// kernels are the lattice-independent ones of dsa.cu.
+// The preconditioned Krylov steady solve on the active cells alone.
+//
+// Its vectors hold the active cells only (45 % of a Pt layer's box), plane
+// by plane: population q of active cell i is element q * np + i, np being
+// the cell count rounded up to 32 (the pad stays zero).  nb[(k - 1) * n + i]
+// is the active index of the cell that link k of cell i leads to, or what
+// the link meets instead.
 #pragma once
 
 #include "internal.cuh"
+#include "pcg.cuh"
 
 namespace cl {
 
-// The D3Q19 plain-population layout: padded row pitch px (cells x >= nx hold
-// no active cell), link word and catalytic links per padded cell.
-struct Dsa19 {
-    int px;
-    const uint32_t* __restrict__ mask;   // bit i-1: link toward x + c_i closed; kQ19Active
-    const uint32_t* __restrict__ react;  // bit i-1: that closed link is catalytic
+enum DsaLink { DSA_WALL = -1, DSA_SINK = -2, DSA_FIXED = -3, DSA_NOFLUX = -4 };
+
+struct DsaCells {
+    int q;         // 7 or 19
+    int n, np;     // active cells; plane stride
+    int* list;     // [n] cell index in the population layout (D3Q19: padded rows)
+    int* inv;      // [cells] active index
+    int* nb;       // [(q - 1) * n]
+    float* sink;   // [n] 1 - r of the cell's catalytic links
+    float* dinv;   // [n] 1 / diag(L), 0 where the row is empty
+    float* omega;  // [n]
 };
 
-// dinv = 1 / diag(L) on active cells (0 elsewhere); a.N = padded cells
-cudaError_t launch_lap_dinv19(const DsaArgs& a, const Dsa19& b, float* dinv, int nblk, cudaStream_t s);
-// eps = 0, r = sum_i v_i (v: 19 population planes), z = dinv r, p = z; scalars
-cudaError_t launch_cg_start19(const DsaArgs& a, const Dsa19& b, const float* v, const float* dinv, float* eps,
-                              float* r, float* zc, float* p, int nblk, double* part, CgScalars* cs, cudaStream_t s);
-// one CG iteration on L eps = r0
-cudaError_t launch_cg_iter19(const DsaArgs& a, const Dsa19& b, const float* dinv, float* eps, float* r, float* zc,
-                             float* p, float* q, int nblk, double* part, CgScalars* cs, cudaStream_t s);
-// zout_i = v_i + w_i eps (19 planes)
-cudaError_t launch_prec_out19(long long N, const float* v, const float* eps, float* zout, int nblk, cudaStream_t s);
+// Numbers the active cells in index order: inv, and *count (device).  part:
+// dsa_scan_blocks(cells) ints.
+int dsa_scan_blocks(long long cells);
+cudaError_t launch_dsa_count(const uint16_t* mask7, const uint32_t* mask19, long long cells, int* part, int* count,
+                             cudaStream_t s);
+cudaError_t launch_dsa_number(const uint16_t* mask7, const uint32_t* mask19, long long cells, const int* part,
+                              int* inv, int* list, cudaStream_t s);
+// Links, diagonals, sinks and relaxation rates of the listed cells
+cudaError_t launch_dsa_links7(const DsaCells& d, const StepArgs& a, cudaStream_t s);
+cudaError_t launch_dsa_links19(const DsaCells& d, const Q19Args& a, cudaStream_t s);
+
+// w = (I - A) z, A the step with zero boundary values and no source
+cudaError_t launch_dsa_apply(const DsaCells& d, const float* z, float* w, cudaStream_t s);
+// z = v + w_i eps, L eps = sum_i v_i (conjugate gradients until r.r is tol2 of its start).  The caller asks
+// for 1e-1: on Knudsen and reactive layers of 24^3 to 96^3 that takes 57 to 120 outer iterations against 58
+// to 119 at 1e-2, half the inner ones (6354 against 10570 at 96^3), and gives the same field to 2e-7.
+cudaError_t launch_dsa_prec(const DsaCells& d, const float* v, float* z, PcgArgs<float> a, cudaStream_t s);
+// whether the CG of n cells keeps its vectors in memory (PcgArgs x .. w)
+bool dsa_prec_streams(int n);
+
+// Modified Gram-Schmidt of w against V[0..j] (vectors of L floats, `stride`
+// apart), in one launch: col[k] = V_k.w, w -= col[k] V_k, col[j + 1] = |w|,
+// V[j + 1] = w / |w|.  meet_mem: pcg_meet_bytes(dsa_mgs_blocks()).
+cudaError_t launch_dsa_mgs(float* V, long long stride, int j, float* w, long long L, double* col, void* meet_mem,
+                           cudaStream_t s);
+int dsa_mgs_blocks();
+// e += sum_k y[k] Z_k, k < m
+cudaError_t launch_dsa_update(float* e, const float* Z, long long stride, int m, const double* y, long long L,
+                              cudaStream_t s);
+// c (population layout) -> active cells, and x64 += sign * e (active cells -> population layout)
+cudaError_t launch_dsa_gather(const DsaCells& d, const float* c, long long cells, float* out, cudaStream_t s);
+cudaError_t launch_dsa_add64(const DsaCells& d, const float* e, double sign, long long cells, double* x,
+                             cudaStream_t s);
 
 }  // namespace cl
