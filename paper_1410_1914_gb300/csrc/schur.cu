@@ -28,10 +28,12 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <chrono>
 #include <vector>
 
 #include "device_util.cuh"
+#include "dsa.cuh"
 #include "handle.cuh"
 
 using namespace cl;
@@ -39,453 +41,381 @@ using namespace cl;
 namespace {
 
 constexpr int kSB = 256;          // threads per block
-constexpr int kSBlk = 152 * 4;    // blocks of the cell loops
 constexpr double kWa = 0.125;     // D3Q7 axis weight
 constexpr double kWr = 0.25;      // D3Q7 rest weight
 
-struct SchurArgs {
-    int nx, ny, nz;
-    long long N;
-    const uint16_t* __restrict__ mask;
-    const double* __restrict__ D;       // per-cell diffusivity [m^2/s]
-    double dt_cs2dx2;                   // dt / (cs^2 dx^2): tau = 1/2 + D dt / (cs^2 dx^2) (Eq. 24)
-    double rfac;                        // uniform catalytic factor
-    const double* __restrict__ kscale;  // per-cell factor on k_lu (nullable)
-    double k_lu;
-    const double* __restrict__ src;     // per-cell source per step (nullable)
-    double c_in, c_out;
-    int bc_in, bc_out;
-    // formed once per call (k_schur_setup): omega in FP64, and the finite-volume
-    // operator as the conductances of the +x, +y, +z links and the diagonal (4 N)
-    const double* __restrict__ om64;
-    const double* __restrict__ G;
+// A run of open faces along one axis: len cells from i on, or -len for a
+// closed loop (y, z) of len cells.  p = kL g*_-(first) + hL enters at the
+// first cell, m = kR g*_+(last) + hR at the last; al is the product of the
+// cells' decays 1 - omega, inv = 1 / (1 - kL al kR al) (a loop: 1 / (1 - al)).
+struct Run {
+    int i, len;
+    double al, inv, kL, kR, hL, hR;
 };
 
-// relaxation rate in FP64 from the cell's D (Eq. 24), as the FP64 oracle forms it
-__device__ __forceinline__ double omega_from_D(const SchurArgs& a, long long c) {
-    return 1.0 / (0.5 + a.D[c] * a.dt_cs2dx2);
-}
-__device__ __forceinline__ double cell_omega(const SchurArgs& a, long long c) { return a.om64[c]; }
+struct SchurArgs {
+    int nx, ny, nz, n;
+    const int* __restrict__ list;
+    const int* __restrict__ nb;         // [6][n], DsaLink below 0
+    const double* __restrict__ D;       // per-cell diffusivity [m^2/s] (box)
+    double dt_cs2dx2;                   // dt / (cs^2 dx^2): tau = 1/2 + D dt / (cs^2 dx^2) (Eq. 24)
+    double rfac;                        // uniform catalytic factor
+    const double* __restrict__ kscale;  // per-cell factor on k_lu (box, nullable)
+    double k_lu;
+    const double* __restrict__ src;     // per-cell source per step (box, nullable)
+    double c_in, c_out;
+    // formed once per call
+    double* om64;   // [n] omega in FP64
+    double* G;      // [6][n] conductance of each link (0 where closed)
+    double* dinv;   // [n] 1 / diagonal of the finite-volume operator
+    Run* runs;      // [3][n]
+    int* n_runs;    // [3]
+};
 
-__device__ __forceinline__ double cat_factor(const SchurArgs& a, long long c) {
+__device__ __forceinline__ double cat_factor(const SchurArgs& a, int c) {
     return a.kscale ? cell_rfac(a.k_lu, a.kscale[c]) : a.rfac;
 }
 
-// Returning factor and added amount of the closed face `bit` of cell c on axis ax (dir +1/-1).
-__device__ __forceinline__ void end_rule(const SchurArgs& a, int ax, int dir, long long c, int xcoord, bool homog,
-                                         double& k, double& h) {
-    const uint16_t m = a.mask[c];
-    const int bit = 2 * ax + (dir > 0 ? 0 : 1);
-    h = 0.0;
-    if (ax == 0 && dir < 0 && xcoord == 0) {
-        if (a.bc_in == CL_BC_DIRICHLET) { k = -1.0; h = homog ? 0.0 : 2.0 * kWa * a.c_in; }
-        else k = 1.0;
-        return;
-    }
-    if (ax == 0 && dir > 0 && xcoord == a.nx - 1) {
-        if (a.bc_out == CL_BC_DIRICHLET) { k = -1.0; h = homog ? 0.0 : 2.0 * kWa * a.c_out; }
-        else k = 1.0;
-        return;
-    }
-    k = ((m >> (kReactShift + bit)) & 1u) ? cat_factor(a, c) : 1.0;
-}
-
-// One thread per line of axis ax: the incoming populations of the two
-// directions of that axis from C, added to T; with `pop`, the post-collision
-// populations of those directions are written too (f32 state layout).
-// With `out3` (three cell fields: consumption on catalytic faces, inflow at
-// x = 0, outflow at x = L, lattice units per step) the FP64 fluxes of the
-// runs' ends are added there as well.
-template <int AX>
-__global__ void __launch_bounds__(kSB) k_lines(SchurArgs a, const double* __restrict__ C, double* __restrict__ T,
-                                               int homog, float* __restrict__ pop, double* __restrict__ out3) {
-    const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const long long nlines = AX == 0 ? (long long)ny * nz : (AX == 1 ? (long long)nx * nz : (long long)nx * ny);
-    const int L = AX == 0 ? nx : (AX == 1 ? ny : nz);
-    const long long stride = AX == 0 ? 1 : (AX == 1 ? (long long)nx : (long long)nx * ny);
-    const bool periodic = AX != 0;
-    const int bp = 2 * AX, bm = 2 * AX + 1;  // closed-face bits of the + and - faces
-    const int ip = 1 + 2 * AX, im = 2 + 2 * AX;  // population indices of the two directions
-    for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < nlines;
-         l += (long long)gridDim.x * blockDim.x) {
-        long long base;
-        if (AX == 0) base = l * nx;
-        else if (AX == 1) base = (l % nx) + (l / nx) * (long long)nx * ny;
-        else base = l;
-        auto cell = [&](int k) { return base + (long long)k * stride; };
-        auto act = [&](int k) { return (a.mask[cell(k)] & kActiveBit) != 0; };
-        auto coef = [&](int k, double& dec, double& s) {
-            const long long c = cell(k);
-            const double om = cell_omega(a, c);
-            dec = 1.0 - om;
-            s = om * kWa * C[c] + (homog || !a.src ? 0.0 : kWa * a.src[c]);
-        };
-        // a start: a cell whose - face is closed (the x line always has one at x = 0 if active)
-        int k0 = -1;
-        for (int k = 0; k < L; ++k)
-            if (act(k) && ((a.mask[cell(k)] >> bm) & 1u)) { k0 = k; break; }
-        if (k0 < 0) {
-            // no closed face: either no active cell, or (y, z) a closed loop of active cells
-            if (!periodic || !act(0)) continue;
-            for (int dir = 0; dir < 2; ++dir) {
-                double al = 1.0, be = 0.0;
-                for (int j = 0; j < L; ++j) {
-                    const int k = dir == 0 ? j : L - 1 - j;
-                    double dec, s;
-                    coef(k, dec, s);
-                    al = dec * al;
-                    be = dec * be + s;
-                }
-                double g = be / (1.0 - al);
-                for (int j = 0; j < L; ++j) {
-                    const int k = dir == 0 ? j : L - 1 - j;
-                    const long long c = cell(k);
-                    double dec, s;
-                    coef(k, dec, s);
-                    T[c] += g;
-                    g = dec * g + s;
-                    if (pop) pop[(long long)(dir == 0 ? ip : im) * a.N + c] = (float)g;
-                }
-            }
-            continue;
-        }
-        // walk the line once from k0 (wrapping for y, z), one run of open faces at a time
-        int j = 0;
-        while (j < L) {
-            const int kA = (k0 + j) % L;
-            if (!act(kA)) { ++j; continue; }
-            // the run kA .. kB: open + faces until one is closed
-            int n = 1;
-            while (n < L && !((a.mask[cell((kA + n - 1) % L)] >> bp) & 1u)) ++n;
-            const int kB = (kA + n - 1) % L;
-            // forward: g*_+(B) = alB p + beB; backward: g*_-(A) = alA m + beA
-            double alB = 1.0, beB = 0.0, alA = 1.0, beA = 0.0;
-            for (int t = 0; t < n; ++t) {
-                double dec, s;
-                coef((kA + t) % L, dec, s);
-                alB = dec * alB;
-                beB = dec * beB + s;
-                coef((kA + n - 1 - t) % L, dec, s);
-                alA = dec * alA;
-                beA = dec * beA + s;
-            }
-            double kL, hL, kR, hR;
-            const long long cA = cell(kA), cB = cell(kB);
-            end_rule(a, AX, -1, cA, AX == 0 ? kA : -1, homog, kL, hL);
-            end_rule(a, AX, +1, cB, AX == 0 ? kB : -1, homog, kR, hR);
-            // p = kL g*_-(A) + hL, m = kR g*_+(B) + hR
-            const double p = (kL * alA * (kR * beB + hR) + kL * beA + hL) / (1.0 - kL * alA * kR * alB);
-            const double m = kR * (alB * p + beB) + hR;
-            if (out3) {
-                // what leaves through the run's end faces: g*_-(A) through the - face, g*_+(B) through the + face
-                const double gA = alA * m + beA, gB = alB * p + beB;
-                const bool inlet = AX == 0 && kA == 0, outlet = AX == 0 && kB == a.nx - 1;
-                if (inlet) { if (a.bc_in == CL_BC_DIRICHLET) out3[a.N + cA] += 2.0 * kWa * a.c_in - 2.0 * gA; }
-                else if ((a.mask[cA] >> (kReactShift + bm)) & 1u) out3[cA] += (1.0 - kL) * gA;
-                if (outlet) { if (a.bc_out == CL_BC_DIRICHLET) out3[2 * a.N + cB] += 2.0 * gB - 2.0 * kWa * a.c_out; }
-                else if ((a.mask[cB] >> (kReactShift + bp)) & 1u) out3[cB] += (1.0 - kR) * gB;
-            }
-            double g = p;
-            for (int t = 0; t < n; ++t) {
-                const long long c = cell((kA + t) % L);
-                double dec, s;
-                coef((kA + t) % L, dec, s);
-                T[c] += g;
-                g = dec * g + s;
-                if (pop) pop[(long long)ip * a.N + c] = (float)g;
-            }
-            g = m;
-            for (int t = 0; t < n; ++t) {
-                const long long c = cell((kA + n - 1 - t) % L);
-                double dec, s;
-                coef((kA + n - 1 - t) % L, dec, s);
-                T[c] += g;
-                g = dec * g + s;
-                if (pop) pop[(long long)im * a.N + c] = (float)g;
-            }
-            j += n;
-        }
-    }
-}
-
-// F = (T + w0 S / omega) / (1 - w0) on active cells; with `pop`, the rest population g_0 = w0 (C + S / omega)
-__global__ void k_lines_fin(SchurArgs a, const double* __restrict__ C, const double* __restrict__ T, int homog,
-                            double* __restrict__ F, float* __restrict__ pop) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < a.N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const bool act = (a.mask[c] & kActiveBit) != 0;
-        const double S = (act && !homog && a.src) ? a.src[c] / cell_omega(a, c) : 0.0;
-        F[c] = act ? (T[c] + kWr * S) / (1.0 - kWr) : 0.0;
-        if (pop) pop[c] = act ? (float)(kWr * (C[c] + S)) : 0.f;
-    }
-}
-
 // lattice diffusivity cs^2 (tau - 1/2) = D dt / dx^2
-__device__ __forceinline__ double cell_D(const SchurArgs& a, long long c) {
-    return 0.25 * a.D[c] * a.dt_cs2dx2;
+__device__ __forceinline__ double cell_D(const SchurArgs& a, int c) { return 0.25 * a.D[c] * a.dt_cs2dx2; }
+
+// omega (FP64, from the cell's D as the FP64 oracle forms it) and the finite-volume operator L_D (link conductance
+// 2 D_a D_b / (D_a + D_b); 2 D on a fixed-value face; 2 k D / (2 D + k) on a catalytic face)
+__global__ void __launch_bounds__(kSB) k_schur_setup(SchurArgs a) {
+    for (int i = blockIdx.x * kSB + threadIdx.x; i < a.n; i += gridDim.x * kSB) {
+        const int c = a.list[i];
+        const double Dc = cell_D(a, c);
+        double diag = 0.0;
+        for (int d = 0; d < 6; ++d) {
+            const int to = a.nb[(long long)d * a.n + i];
+            double g = 0.0;
+            if (to >= 0) {
+                const double Dn = cell_D(a, a.list[to]);
+                g = 2.0 * Dc * Dn / (Dc + Dn);
+                diag += g;
+            } else if (to == DSA_FIXED) {
+                diag += 2.0 * Dc;
+            } else if (to == DSA_SINK) {
+                const double k = a.k_lu * (a.kscale ? a.kscale[c] : 1.0);
+                diag += 2.0 * k * Dc / (2.0 * Dc + k);
+            }
+            a.G[(long long)d * a.n + i] = g;
+        }
+        a.om64[i] = 1.0 / (0.5 + a.D[c] * a.dt_cs2dx2);
+        a.dinv[i] = diag > 0.0 ? 1.0 / diag : 0.0;
+    }
 }
 
-// neighbour of c across face d (0 +x, 1 -x, 2 +y, 3 -y, 4 +z, 5 -z), y and z periodic
-__device__ __forceinline__ long long face_nb(const SchurArgs& a, long long c, int d, int y, int z) {
-    const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const long long plane = (long long)nx * ny;
-    if (d == 0) return c + 1;
-    if (d == 1) return c - 1;
-    if (d == 2) return y == ny - 1 ? c - (long long)(ny - 1) * nx : c + nx;
-    if (d == 3) return y == 0 ? c + (long long)(ny - 1) * nx : c - nx;
-    if (d == 4) return z == nz - 1 ? c - (long long)(nz - 1) * plane : c + plane;
-    return z == 0 ? c + (long long)(nz - 1) * plane : c - plane;
+// Returning factor and added amount of closed link `to` of box cell c
+__device__ __forceinline__ void end_rule(const SchurArgs& a, int to, bool minus, int c, double& k, double& h) {
+    h = 0.0;
+    if (to == DSA_FIXED) {  // only the x faces of the box have one
+        k = -1.0;
+        h = 2.0 * kWa * (minus ? a.c_in : a.c_out);
+    } else {
+        k = to == DSA_SINK ? cat_factor(a, c) : 1.0;
+    }
 }
 
-// once per call: omega (FP64) and the finite-volume operator L_D (link conductance
-// 2 D_a D_b / (D_a + D_b); 2 D on a fixed-value face; 2 k D / (2 D + k) on a catalytic
-// face) as G[0..2] = conductances of the +x, +y, +z links (0 where closed), G[3] = the
-// diagonal, and dinv = 1 / diagonal (0 off the active set)
-__global__ void k_schur_setup(SchurArgs a, double* __restrict__ om64, double* __restrict__ G,
-                              double* __restrict__ dinv) {
-    const int nx = a.nx, ny = a.ny;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < a.N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const uint16_t m = a.mask[c];
-        double g[3] = {0.0, 0.0, 0.0}, diag = 0.0;
-        double om = 1.0;
-        if (m & kActiveBit) {
-            om = omega_from_D(a, c);
-            const int x = (int)(c % nx);
-            const long long r = c / nx;
-            const int y = (int)(r % ny), z = (int)(r / ny);
-            const double Dc = cell_D(a, c);
-            for (int d = 0; d < 6; ++d) {
-                if ((m >> d) & 1u) {
-                    if (d == 1 && x == 0) { if (a.bc_in == CL_BC_DIRICHLET) diag += 2.0 * Dc; }
-                    else if (d == 0 && x == nx - 1) { if (a.bc_out == CL_BC_DIRICHLET) diag += 2.0 * Dc; }
-                    else if ((m >> (kReactShift + d)) & 1u) {
-                        const double k = a.k_lu * (a.kscale ? a.kscale[c] : 1.0);
-                        diag += 2.0 * k * Dc / (2.0 * Dc + k);
-                    }
-                    continue;
+// The runs of axis blockIdx.y, in any order (runs do not share cells): each cell whose - face is closed starts one;
+// a y or z line without a closed face is a loop, recorded by its cell of coordinate 0.
+__global__ void __launch_bounds__(kSB) k_schur_runs(SchurArgs a) {
+    const int ax = blockIdx.y;
+    const int* __restrict__ fwd = a.nb + (long long)(2 * ax) * a.n;
+    const int* __restrict__ bwd = a.nb + (long long)(2 * ax + 1) * a.n;
+    for (int i = blockIdx.x * kSB + threadIdx.x; i < a.n; i += gridDim.x * kSB) {
+        Run r;
+        r.i = i;
+        r.al = 1.0 - a.om64[i];
+        if (bwd[i] < 0) {
+            int last = i;
+            r.len = 1;
+            for (int t = fwd[i]; t >= 0; t = fwd[t]) {
+                r.al *= 1.0 - a.om64[t];
+                last = t;
+                ++r.len;
+            }
+            end_rule(a, bwd[i], true, a.list[i], r.kL, r.hL);
+            end_rule(a, fwd[last], false, a.list[last], r.kR, r.hR);
+            r.inv = 1.0 / (1.0 - r.kL * r.al * r.kR * r.al);
+        } else {
+            if (ax == 0) continue;
+            const int c = a.list[i];
+            const int coord = ax == 1 ? (c / a.nx) % a.ny : c / (a.nx * a.ny);
+            if (coord != 0) continue;
+            int len = 1, t = fwd[i];
+            for (; t >= 0 && t != i; t = fwd[t]) {
+                r.al *= 1.0 - a.om64[t];
+                ++len;
+            }
+            if (t != i) continue;  // the line has a closed face
+            r.len = -len;
+            r.inv = 1.0 / (1.0 - r.al);
+            r.kL = r.kR = r.hL = r.hR = 0.0;
+        }
+        a.runs[(long long)ax * a.n + atomicAdd(a.n_runs + ax, 1)] = r;
+    }
+}
+
+// One thread per run: the incoming populations of the two directions of its
+// axis from C into T[axis] (their sum).  OUT: also the post-collision
+// populations (f32 state layout, N cells a plane) and, per run, the amounts
+// consumed on its catalytic ends (flux[axis]), entering at x = 0 (flux[3]) and
+// leaving at x = L (flux[4]), lattice units per step, FP64.
+template <bool OUT>
+__global__ void __launch_bounds__(kSB) k_walk(SchurArgs a, const double* __restrict__ C, double* __restrict__ T,
+                                              int homog, float* __restrict__ pop, long long N,
+                                              double* __restrict__ flux) {
+    const int ax = blockIdx.y, n = a.n;
+    const int* __restrict__ fwd = a.nb + (long long)(2 * ax) * n;
+    const int* __restrict__ bwd = a.nb + (long long)(2 * ax + 1) * n;
+    double* __restrict__ Ta = T + (long long)ax * n;
+    const int nr = a.n_runs[ax];
+    auto coef = [&](int i, double& dec, double& s) {
+        const double om = a.om64[i];
+        dec = 1.0 - om;
+        s = om * kWa * C[i] + (homog || !a.src ? 0.0 : kWa * a.src[a.list[i]]);
+    };
+    for (int q = blockIdx.x * kSB + threadIdx.x; q < nr; q += gridDim.x * kSB) {
+        const Run r = a.runs[(long long)ax * n + q];
+        const bool loop = r.len < 0;
+        const int len = loop ? -r.len : r.len;
+        // forward: g*_+(last) = al p + beB; backward: g*_-(first) = al m + beA
+        double beA = 0.0, beB = 0.0, pre = 1.0;
+        int last = r.i;
+        for (int t = 0, i = r.i; t < len; ++t) {
+            double dec, s;
+            coef(i, dec, s);
+            beB = dec * beB + s;
+            beA += pre * s;
+            pre *= dec;
+            last = i;
+            i = ax == 0 ? i + 1 : fwd[i];
+        }
+        double p, m;
+        if (loop) {
+            // populations arriving at the first cell from behind, and at the last cell from ahead
+            p = beB * r.inv;
+            m = beA * r.inv;
+        } else {
+            const double hL = homog ? 0.0 : r.hL, hR = homog ? 0.0 : r.hR;
+            p = (r.kL * r.al * (r.kR * beB + hR) + r.kL * beA + hL) * r.inv;
+            m = r.kR * (r.al * p + beB) + hR;
+            if (OUT) {
+                // what leaves through the run's end faces: g*_-(first) and g*_+(last)
+                const double gA = r.al * m + beA, gB = r.al * p + beB;
+                const int tA = bwd[r.i], tB = fwd[last];
+                double R = 0.0, jin = 0.0, jout = 0.0;
+                if (tA == DSA_FIXED) jin = 2.0 * kWa * a.c_in - 2.0 * gA;
+                else if (tA == DSA_SINK) R += (1.0 - r.kL) * gA;
+                if (tB == DSA_FIXED) jout = 2.0 * gB - 2.0 * kWa * a.c_out;
+                else if (tB == DSA_SINK) R += (1.0 - r.kR) * gB;
+                flux[(long long)ax * n + r.i] = R;
+                if (ax == 0) {
+                    flux[3LL * n + r.i] = jin;
+                    flux[4LL * n + r.i] = jout;
                 }
-                const double Dn = cell_D(a, face_nb(a, c, d, y, z));
-                const double Gl = 2.0 * Dc * Dn / (Dc + Dn);
-                diag += Gl;
-                if ((d & 1) == 0) g[d >> 1] = Gl;
             }
         }
-        om64[c] = om;
-        for (int k = 0; k < 3; ++k) G[(long long)k * a.N + c] = g[k];
-        G[3 * a.N + c] = diag;
-        dinv[c] = diag > 0.0 ? 1.0 / diag : 0.0;
+        double g = p;
+        for (int t = 0, i = r.i; t < len; ++t) {
+            double dec, s;
+            coef(i, dec, s);
+            Ta[i] = g;
+            g = dec * g + s;
+            if (OUT) pop[(1 + 2 * ax) * N + a.list[i]] = (float)g;
+            i = ax == 0 ? i + 1 : fwd[i];
+        }
+        g = m;
+        for (int t = 0, i = last; t < len; ++t) {
+            double dec, s;
+            coef(i, dec, s);
+            Ta[i] += g;
+            g = dec * g + s;
+            if (OUT) pop[(2 + 2 * ax) * N + a.list[i]] = (float)g;
+            i = ax == 0 ? i - 1 : bwd[i];
+        }
     }
 }
 
-// (L_D p)(c) from the stored conductances
-__device__ __forceinline__ double ld_apply(const SchurArgs& a, long long c, const double* __restrict__ p) {
-    const int nx = a.nx, ny = a.ny;
-    const uint16_t m = a.mask[c];
-    const int y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-    const long long N = a.N;
-    double q = a.G[3 * N + c] * p[c];
-    for (int d = 0; d < 6; ++d) {
-        if ((m >> d) & 1u) continue;
-        const long long nb = face_nb(a, c, d, y, z);
-        const double Gl = (d & 1) == 0 ? a.G[(long long)(d >> 1) * N + c] : a.G[(long long)(d >> 1) * N + nb];
-        q -= Gl * p[nb];
+// F = (T + w0 S / omega) / (1 - w0), T the sum over the axes; out = F, or z - F (minus); OUT: the rest population
+// g_0 = w0 (C + S / omega)
+template <bool OUT>
+__global__ void __launch_bounds__(kSB) k_walk_fin(SchurArgs a, const double* __restrict__ C,
+                                                  const double* __restrict__ T, int homog, int minus,
+                                                  double* __restrict__ out, float* __restrict__ pop) {
+    const int n = a.n;
+    for (int i = blockIdx.x * kSB + threadIdx.x; i < n; i += gridDim.x * kSB) {
+        const double S = (!homog && a.src) ? a.src[a.list[i]] / a.om64[i] : 0.0;
+        const double F = ((T[i] + T[n + i]) + T[2LL * n + i] + kWr * S) / (1.0 - kWr);
+        out[i] = minus ? C[i] - F : F;
+        if (OUT) pop[a.list[i]] = (float)(kWr * (C[i] + S));
     }
-    return q;
 }
 
-struct Cg64 {
-    double rz, alpha, beta, rr, rr0, pq;
-    int iters, bad;
+// The finite-volume operator for the resident conjugate gradients (pcg.cuh): z = L_D^{-1} v
+struct FvOp {
+    int n;
+    const int* __restrict__ nb;
+    const double* __restrict__ G;
+    const double* __restrict__ dinv_;
+    const double* __restrict__ v;
+    double* __restrict__ z;
+    struct Row {
+        int j[6];
+        double g[6];
+    };
+    __device__ __forceinline__ Row load(int i) const {
+        Row r;
+#pragma unroll
+        for (int d = 0; d < 6; ++d) {
+            r.j[d] = nb[(long long)d * n + i];
+            r.g[d] = G[(long long)d * n + i];
+        }
+        return r;
+    }
+    template <class S>
+    __device__ __forceinline__ double off(const Row& r, const double* u) const {
+        double t = 0.0;
+#pragma unroll
+        for (int d = 0; d < 6; ++d)
+            if (r.j[d] >= 0) t = fma(r.g[d], S::ld(u + r.j[d]), t);
+        return t;
+    }
+    __device__ __forceinline__ double rhs(int i) const { return v[i]; }
+    __device__ __forceinline__ double dinv(int i) const { return dinv_[i]; }
+    __device__ __forceinline__ void done(int i, double x) const { z[i] = x; }
 };
 
-// CG start from x = 0: r = b, z = dinv r, p = z; partials r.z, r.r
-__global__ void k_cg_start64(long long N, const double* __restrict__ b, const double* __restrict__ dinv,
-                             double* __restrict__ x, double* __restrict__ r, double* __restrict__ p,
-                             double* __restrict__ part) {
-    double acc[2] = {0.0, 0.0};
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const double rv = b[c], zv = dinv[c] * rv;
-        x[c] = 0.0;
-        r[c] = rv;
-        p[c] = zv;
-        acc[0] += rv * zv;
-        acc[1] += rv * rv;
+constexpr int kCgT64 = 256;
+constexpr int kCgStreamT64 = 512;
+
+bool prec_streams64(int n) { return (n + kCgT64 - 1) / kCgT64 > 8 * device_sms(); }
+
+// Few cells go to one cluster: its barrier costs a third of the grid's meetings.  FP64 runs at 2 lanes per cycle and
+// SM, so past a few hundred cells per SM the arithmetic outweighs that and the whole grid takes over.
+cudaError_t prec64(const FvOp& op, const PcgArgs<double>& a, cudaStream_t s) {
+    const int sms = device_sms(), n = op.n;
+    const auto blocks = [&](int k) { return (n + k * kCgT64 - 1) / (k * kCgT64); };
+    if (blocks(1) <= kPcgMaxCluster)
+        // the whole cluster, however few the cells
+        return pcg_launch_cluster<double, FvOp, 1, kCgT64>(op, a, std::min(kPcgMaxCluster, (n + 31) / 32), s);
+    if (blocks(2) <= kPcgMaxCluster) return pcg_launch_cluster<double, FvOp, 2, kCgT64>(op, a, kPcgMaxCluster, s);
+    if (blocks(1) <= sms) return pcg_launch_grid<double, FvOp, 1, kCgT64>(op, a, std::min(sms, (n + 63) / 64), s);
+    switch (blocks(1) <= 8 * sms ? (blocks(1) + sms - 1) / sms : 0) {
+        case 2: return pcg_launch_grid<double, FvOp, 2, kCgT64>(op, a, sms, s);
+        case 3:
+        case 4: return pcg_launch_grid<double, FvOp, 4, kCgT64>(op, a, sms, s);
+        case 5:
+        case 6:
+        case 7:
+        case 8: return pcg_launch_grid<double, FvOp, 8, kCgT64>(op, a, sms, s);
     }
-    block_sum_store<2>(acc, part + 2 * blockIdx.x);
+    return pcg_launch_grid<double, FvOp, 0, kCgStreamT64>(op, a, sms, s);
 }
 
-// q = L_D p, partial p.q
-__global__ void k_cg_q64(SchurArgs a, const double* __restrict__ p, double* __restrict__ q, double* __restrict__ part,
-                         const Cg64* __restrict__ cs) {
-    if (cs->bad) return;
+// h[j] = V_j . w (one block per vector and chunk of kDotCells cells; part[chunk][j])
+constexpr int kDotCells = 8192;
+__global__ void __launch_bounds__(kSB) k_mdot(const double* __restrict__ V, int n, const double* __restrict__ w,
+                                              double* __restrict__ part) {
+    const int c0 = blockIdx.y * kDotCells, c1 = min(n, c0 + kDotCells);
+    const double* __restrict__ v = V + (long long)blockIdx.x * n;
     double acc[1] = {0.0};
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < a.N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const double out = (a.mask[c] & kActiveBit) ? ld_apply(a, c, p) : 0.0;
-        q[c] = out;
-        acc[0] += p[c] * out;
+    for (int c = c0 + threadIdx.x; c < c1; c += kSB) acc[0] = fma(v[c], w[c], acc[0]);
+    block_sum_store<1>(acc, part + (long long)blockIdx.y * gridDim.x + blockIdx.x);
+}
+
+// w -= sum_j h[j] V_j with h[j] = sum over chunks of part[chunk][j]: blocks of 32 cells, the vectors shared out over
+// 8 warps.  hout gets h (block 0); nrm (nullable): this block's part of |w|^2.
+__global__ void __launch_bounds__(kSB) k_msub(const double* __restrict__ V, int n, int m, int chunks,
+                                              const double* __restrict__ part, double* __restrict__ w,
+                                              double* __restrict__ hout, double* __restrict__ nrm) {
+    __shared__ double sh[kSB / 32][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = blockIdx.x * 32 + lane;
+    double acc = 0.0;
+    for (int j = warp; j < m; j += kSB / 32) {
+        double h = part[j];
+        for (int k = 1; k < chunks; ++k) h += part[(long long)k * m + j];
+        if (c < n) acc = fma(h, V[(long long)j * n + c], acc);
+        if (blockIdx.x == 0 && lane == 0) hout[j] = h;
     }
-    block_sum_store<1>(acc, part + blockIdx.x);
-}
-
-// x += alpha p, r -= alpha q; partials r.z (z = dinv r), r.r
-__global__ void k_cg_upd64(long long N, const double* __restrict__ dinv, const double* __restrict__ p,
-                           const double* __restrict__ q, double* __restrict__ x, double* __restrict__ r,
-                           double* __restrict__ part, const Cg64* __restrict__ cs) {
-    if (cs->bad) return;
-    const double al = cs->alpha;
-    double acc[2] = {0.0, 0.0};
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        x[c] += al * p[c];
-        const double rv = r[c] - al * q[c];
-        r[c] = rv;
-        acc[0] += rv * dinv[c] * rv;
-        acc[1] += rv * rv;
-    }
-    block_sum_store<2>(acc, part + 2 * blockIdx.x);
-}
-
-// p = dinv r + beta p
-__global__ void k_cg_p64(long long N, const double* __restrict__ dinv, const double* __restrict__ r,
-                         double* __restrict__ p, const Cg64* __restrict__ cs) {
-    if (cs->bad) return;
-    const double be = cs->beta;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x)
-        p[c] = dinv[c] * r[c] + be * p[c];
-}
-
-// one block: the CG scalars from the block partials (fixed order)
-// stage 0: start (rz, rr0); 1: alpha = rz / p.q; 2: beta from the new r.z, rr
-__global__ void k_cg_fin64(const double* __restrict__ part, int nblk, int stage, Cg64* cs) {
-    const int nv = stage == 1 ? 1 : 2;
-    double acc[2] = {0.0, 0.0};
-    for (int i = threadIdx.x; i < nblk; i += blockDim.x)
-        for (int k = 0; k < nv; ++k) acc[k] += part[(long long)nv * i + k];
-    __shared__ double out[2];
-    block_sum_store<2>(acc, out);
+    sh[warp][lane] = acc;
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    if (stage == 0) {
-        cs->rz = out[0];
-        cs->rr = cs->rr0 = out[1];
-        cs->iters = 0;
-        cs->bad = (out[1] == 0.0) ? 2 : (isfinite(out[0]) ? 0 : 1);
-    } else if (stage == 1) {
-        if (cs->bad) return;
-        cs->pq = out[0];
-        if (!(out[0] > 0.0) || !isfinite(out[0])) {
-            // p.q = 0 after the residual has vanished is convergence, not a breakdown
-            cs->bad = (isfinite(out[0]) && cs->rr <= 1e-28 * cs->rr0) ? 2 : 1;
-            return;
+    if (warp == 0) {
+        double t = 0.0;
+        for (int k = 0; k < kSB / 32; ++k) t += sh[k][lane];
+        double v = 0.0;
+        if (c < n) {
+            v = w[c] - t;
+            w[c] = v;
         }
-        cs->alpha = cs->rz / out[0];
-    } else {
-        if (cs->bad) return;
-        cs->beta = out[0] / cs->rz;
-        cs->rz = out[0];
-        cs->rr = out[1];
-        cs->iters += 1;
-        if (!isfinite(out[0])) cs->bad = 1;
-    }
-}
-
-// dot products of w with V[0..n) in one pass: part[blk][j]
-__global__ void k_mdot(const double* __restrict__ V, long long N, int n, const double* __restrict__ w,
-                       double* __restrict__ part) {
-    // each block sums its chunk for every j; n <= blockDim.x * kMaxJ handled by the j loop
-    __shared__ double sh[kSB];
-    const long long chunk = (N + gridDim.x - 1) / gridDim.x;
-    const long long c0 = blockIdx.x * chunk, c1 = min(N, c0 + chunk);
-    for (int j = 0; j < n; ++j) {
-        double acc = 0.0;
-        const double* v = V + (long long)j * N;
-        for (long long c = c0 + threadIdx.x; c < c1; c += blockDim.x) acc += v[c] * w[c];
-        sh[threadIdx.x] = acc;
-        __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-            __syncthreads();
+        if (nrm) {
+            v *= v;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) nrm[blockIdx.x] = v;
         }
-        if (threadIdx.x == 0) part[(long long)blockIdx.x * n + j] = sh[0];
-        __syncthreads();
     }
 }
 
-// h[j] = sum over blocks of part[blk][j] (one thread per j, fixed order)
-__global__ void k_mdot_fin(const double* __restrict__ part, int nblk, int n, double* __restrict__ h) {
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        double acc = 0.0;
-        for (int b = 0; b < nblk; ++b) acc += part[(long long)b * n + j];
-        h[j] = acc;
+// parts of |v|^2, 32 cells each
+__global__ void __launch_bounds__(kSB) k_norm_part(const double* __restrict__ v, int n, double* __restrict__ nrm) {
+    const int c = blockIdx.x * kSB + threadIdx.x;
+    double t = c < n ? v[c] * v[c] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0 && (c >> 5) < (n + 31) / 32) nrm[c >> 5] = t;
+}
+
+// *out = sqrt(sum of the parts), one block
+__global__ void __launch_bounds__(kSB) k_norm_fin(const double* __restrict__ nrm, int parts, double* __restrict__ out) {
+    double acc[1] = {0.0};
+    for (int k = threadIdx.x; k < parts; k += kSB) acc[0] += nrm[k];
+    __shared__ double tot[1];
+    block_sum_store<1>(acc, tot);
+    if (threadIdx.x == 0) *out = sqrt(tot[0]);
+}
+
+// y = x / *norm (not touched where the norm is 0)
+__global__ void __launch_bounds__(kSB) k_scale64(int n, const double* __restrict__ norm, const double* __restrict__ x,
+                                                 double* __restrict__ y) {
+    __shared__ double f;
+    if (threadIdx.x == 0) f = *norm > 0.0 ? 1.0 / *norm : 0.0;
+    __syncthreads();
+    if (f == 0.0) return;
+    for (int c = blockIdx.x * kSB + threadIdx.x; c < n; c += gridDim.x * kSB) y[c] = f * x[c];
+}
+
+// x += sum_k y[k] Z_k
+__global__ void __launch_bounds__(kSB) k_comb64(const double* __restrict__ Z, int n, int m,
+                                                const double* __restrict__ y, double* __restrict__ x) {
+    for (int c = blockIdx.x * kSB + threadIdx.x; c < n; c += gridDim.x * kSB) {
+        double t = x[c];
+        for (int k = 0; k < m; ++k) t = fma(y[k], Z[(long long)k * n + c], t);
+        x[c] = t;
     }
 }
 
-// w -= sum_j h[j] V[j]
-__global__ void k_msub(const double* __restrict__ V, long long N, int n, const double* __restrict__ h,
-                       double* __restrict__ w) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        double acc = w[c];
-        for (int j = 0; j < n; ++j) acc -= h[j] * V[(long long)j * N + c];
-        w[c] = acc;
-    }
-}
-
-// y = alpha x (+ y if add)
-__global__ void k_axpy64(long long N, double alpha, const double* __restrict__ x, double* __restrict__ y, int add) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x)
-        y[c] = alpha * x[c] + (add ? y[c] : 0.0);
-}
-
-// out = a - b (out may alias a)
-__global__ void k_sub64(long long N, const double* __restrict__ a, const double* __restrict__ b, double* out) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x)
-        out[c] = a[c] - b[c];
-}
-
-// block partials of the three flux fields (fixed order)
-__global__ void k_sum3(long long N, const double* __restrict__ out3, double* __restrict__ part) {
+// sums over the cells of the three axes' consumption, the inflow and the outflow
+__global__ void __launch_bounds__(1024) k_flux_sum(const double* __restrict__ flux, int n, double* __restrict__ out) {
     double acc[3] = {0.0, 0.0, 0.0};
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        acc[0] += out3[c];
-        acc[1] += out3[N + c];
-        acc[2] += out3[2 * N + c];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        acc[0] += (flux[i] + flux[n + i]) + flux[2LL * n + i];
+        acc[1] += flux[3LL * n + i];
+        acc[2] += flux[4LL * n + i];
     }
-    block_sum_store<3>(acc, part + 3 * blockIdx.x);
-}
-
-__global__ void k_sum3_fin(const double* __restrict__ part, int nblk, double* __restrict__ out) {
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < nblk; i += blockDim.x)
-        for (int k = 0; k < 3; ++k) acc[k] += part[3 * i + k];
     block_sum_store<3>(acc, out);
 }
 
-__global__ void k_norm2(long long N, const double* __restrict__ v, double* __restrict__ part) {
-    double acc[1] = {0.0};
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x)
-        acc[0] += v[c] * v[c];
-    block_sum_store<1>(acc, part + blockIdx.x);
-}
-
-__global__ void k_field_to_f64(long long N, const float* __restrict__ pop, const uint16_t* __restrict__ mask,
-                               const double* __restrict__ src, double* __restrict__ C) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
+// C of the stored state, less the last collision's source
+__global__ void __launch_bounds__(kSB) k_field64(SchurArgs a, long long N, const float* __restrict__ pop,
+                                                 double* __restrict__ C) {
+    for (int i = blockIdx.x * kSB + threadIdx.x; i < a.n; i += gridDim.x * kSB) {
+        const int c = a.list[i];
         double v = 0.0;
-        if (mask[c] & kActiveBit) {
-            for (int i = 0; i < 7; ++i) v += (double)pop[(long long)i * N + c];
-            if (src) v -= src[c];
-        }
-        C[c] = v;
+        for (int q = 0; q < 7; ++q) v += (double)pop[q * N + c];
+        C[i] = a.src ? v - a.src[c] : v;
     }
 }
 
@@ -493,11 +423,12 @@ struct Mem {
     cudaStream_t s;
     std::vector<void*> p;
     explicit Mem(cudaStream_t st) : s(st) {}
-    cudaError_t get(double** out, long long n) {
+    template <class T>
+    cudaError_t get(T** out, long long n) {
         void* v = nullptr;
-        cudaError_t e = cudaMallocAsync(&v, sizeof(double) * (size_t)(n > 0 ? n : 1), s);
+        cudaError_t e = cudaMallocAsync(&v, sizeof(T) * (size_t)(n > 0 ? n : 1), s);
         if (e == cudaSuccess) p.push_back(v);
-        *out = (double*)v;
+        *out = (T*)v;
         return e;
     }
     ~Mem() {
@@ -525,173 +456,163 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
     cudaStream_t s = h->s;
     const long long N = h->N;
     const int m = restart < max_iter ? restart : max_iter;
-    SchurArgs a;
-    a.nx = h->nx; a.ny = h->ny; a.nz = h->nz; a.N = N;
-    a.mask = h->mask;
-    a.D = h->D;
-    a.dt_cs2dx2 = h->dt / (0.25 * h->p.dx_m * h->p.dx_m);
-    a.rfac = reactive_factor_d(h);
-    a.kscale = h->kscale;
-    a.k_lu = h->k_lu;
-    a.src = h->src;
-    a.c_in = h->p.c_in; a.c_out = h->p.c_out;
-    a.bc_in = h->p.bc_in; a.bc_out = h->p.bc_out;
-    const int lb = kSB;
-    auto nb_lines = [&](long long nl) { return (int)((nl + lb - 1) / lb); };
     cl_steady_info inf;
     memset(&inf, 0, sizeof(inf));
     cl_status result = CL_ERR_NOT_CONVERGED;
     {
         Mem mem(s);
-        double *V = nullptr, *Z = nullptr, *x = nullptr, *w = nullptr, *T = nullptr, *part = nullptr, *hv = nullptr;
-        double *dinv = nullptr, *cr = nullptr, *cp = nullptr, *cq = nullptr, *cpart = nullptr;
-        CK(mem.get(&V, (long long)(m + 1) * N));
-        CK(mem.get(&Z, (long long)m * N));
-        CK(mem.get(&x, N));
-        CK(mem.get(&w, N));
-        CK(mem.get(&T, N));
-        CK(mem.get(&part, (long long)kSBlk * (m + 1 > 3 ? m + 1 : 3)));
-        CK(mem.get(&hv, m + 1 > 3 ? m + 1 : 3));
-        CK(mem.get(&dinv, N));
-        CK(mem.get(&cr, N));
-        CK(mem.get(&cp, N));
-        CK(mem.get(&cq, N));
-        CK(mem.get(&cpart, 2 * kSBlk));
-        double *om64 = nullptr, *G = nullptr;
-        CK(mem.get(&om64, N));
-        CK(mem.get(&G, 4 * N));
-        a.om64 = om64;
-        a.G = G;
-        Cg64* cs = nullptr;
-        {
-            void* v = nullptr;
-            CK(cudaMallocAsync(&v, sizeof(Cg64), s));
-            mem.p.push_back(v);
-            cs = (Cg64*)v;
+        // the active cells and their links (dsa.cuh)
+        DsaCells d;
+        d.q = 7;
+        int* scan = nullptr;
+        const int nscan = dsa_scan_blocks(N);
+        CK(mem.get(&scan, nscan + 1));
+        CK(mem.get(&d.inv, N));
+        CK(launch_dsa_count(h->mask, nullptr, N, scan, scan + nscan, s));
+        CK(cudaMemcpyAsync(&d.n, scan + nscan, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        const int n = d.n;
+        d.np = n;
+        CK(mem.get(&d.list, n));
+        CK(mem.get(&d.nb, 6LL * n));
+        CK(mem.get(&d.sink, n));
+        CK(mem.get(&d.dinv, n));
+        CK(mem.get(&d.omega, n));
+        CK(launch_dsa_number(h->mask, nullptr, N, scan, d.inv, d.list, s));
+        StepArgs sa;
+        memset(&sa, 0, sizeof(sa));
+        sa.nx = h->nx; sa.ny = h->ny; sa.nz = h->nz; sa.N = N;
+        sa.mask = h->mask;
+        sa.omega = h->omega;
+        sa.rsink = (float)reactive_sink_d(h);
+        sa.kscale = h->kscale;
+        sa.k_lu = h->k_lu;
+        sa.bc_in = h->p.bc_in; sa.bc_out = h->p.bc_out;
+        CK(launch_dsa_links7(d, sa, s));
+        SchurArgs a;
+        a.nx = h->nx; a.ny = h->ny; a.nz = h->nz; a.n = n;
+        a.list = d.list;
+        a.nb = d.nb;
+        a.D = h->D;
+        a.dt_cs2dx2 = h->dt / (0.25 * h->p.dx_m * h->p.dx_m);
+        a.rfac = reactive_factor_d(h);
+        a.kscale = h->kscale;
+        a.k_lu = h->k_lu;
+        a.src = h->src;
+        a.c_in = h->p.c_in; a.c_out = h->p.c_out;
+        CK(mem.get(&a.om64, n));
+        CK(mem.get(&a.G, 6LL * n));
+        CK(mem.get(&a.dinv, n));
+        CK(mem.get(&a.runs, 3LL * n));
+        CK(mem.get(&a.n_runs, 3));
+        CK(cudaMemsetAsync(a.n_runs, 0, 3 * sizeof(int), s));
+        const int nb = std::min((n + kSB - 1) / kSB, 152 * 8);
+        k_schur_setup<<<nb, kSB, 0, s>>>(a);
+        k_schur_runs<<<dim3(nb, 3), kSB, 0, s>>>(a);
+        CK(cudaGetLastError());
+        double *V = nullptr, *Z = nullptr, *x = nullptr, *w = nullptr, *T = nullptr, *part = nullptr, *nrm = nullptr;
+        double *hv = nullptr, *dy = nullptr;
+        const int chunks = (n + kDotCells - 1) / kDotCells, parts = (n + 31) / 32;
+        CK(mem.get(&V, (long long)(m + 1) * n));
+        CK(mem.get(&Z, (long long)m * n));
+        CK(mem.get(&x, n));
+        CK(mem.get(&w, n));
+        CK(mem.get(&T, 3LL * n));
+        CK(mem.get(&part, (long long)chunks * (m + 1)));
+        CK(mem.get(&nrm, parts));
+        CK(mem.get(&hv, 2LL * (m + 1) + 3));  // the two passes' coefficients, a norm, spare
+        CK(mem.get(&dy, m));
+        double* dnorm = hv + 2 * (size_t)(m + 1);
+        // z = L_D^{-1} v to cg_tol (diagonal-preconditioned CG, FP64)
+        PcgArgs<double> cg;
+        memset(&cg, 0, sizeof(cg));
+        cg.n = n;
+        cg.tol2 = cg_tol * cg_tol;
+        cg.max_iters = 100000;
+        CK(mem.get(&cg.u, n));
+        if (prec_streams64(n)) {
+            CK(mem.get(&cg.x, n));
+            CK(mem.get(&cg.r, n));
+            CK(mem.get(&cg.p, n));
+            CK(mem.get(&cg.s, n));
+            CK(mem.get(&cg.w, n));
         }
-        // F(C) into out (affine: homog = 0; linear part: homog = 1); pop: write the state
-        auto apply_F = [&](const double* C, int homog, double* out, float* pop, double* out3 = nullptr) -> cl_status {
-            CK(cudaMemsetAsync(T, 0, sizeof(double) * (size_t)N, s));
-            k_lines<0><<<nb_lines((long long)a.ny * a.nz), lb, 0, s>>>(a, C, T, homog, pop, out3);
-            k_lines<1><<<nb_lines((long long)a.nx * a.nz), lb, 0, s>>>(a, C, T, homog, pop, out3);
-            k_lines<2><<<nb_lines((long long)a.nx * a.ny), lb, 0, s>>>(a, C, T, homog, pop, out3);
-            k_lines_fin<<<kSBlk, kSB, 0, s>>>(a, C, T, homog, out, pop);
+        cg.meet_blocks = device_sms();
+        char* meet_mem = nullptr;
+        CK(mem.get(&meet_mem, (long long)pcg_meet_bytes(cg.meet_blocks)));
+        cg.meet_mem = meet_mem;
+        CK(mem.get(&cg.out, 1));
+        FvOp op;
+        op.n = n;
+        op.nb = d.nb;
+        op.G = a.G;
+        op.dinv_ = a.dinv;
+        // F(C) (affine: homog = 0; linear part: homog = 1) or C - F(C) (minus) into out
+        auto apply_F = [&](const double* C, int homog, int minus, double* out) -> cl_status {
+            k_walk<false><<<dim3(nb, 3), kSB, 0, s>>>(a, C, T, homog, nullptr, N, nullptr);
+            k_walk_fin<false><<<nb, kSB, 0, s>>>(a, C, T, homog, minus, out, nullptr);
             CK(cudaGetLastError());
             return CL_OK;
         };
         auto norm = [&](const double* v, double* out) -> cl_status {
-            k_norm2<<<kSBlk, kSB, 0, s>>>(N, v, part);
-            k_mdot_fin<<<1, 32, 0, s>>>(part, kSBlk, 1, hv);
+            k_norm_part<<<(n + kSB - 1) / kSB, kSB, 0, s>>>(v, n, nrm);
+            k_norm_fin<<<1, kSB, 0, s>>>(nrm, parts, dnorm);
             CK(cudaGetLastError());
-            double hs = 0.0;
-            CK(cudaMemcpyAsync(&hs, hv, sizeof(double), cudaMemcpyDeviceToHost, s));
+            CK(cudaMemcpyAsync(out, dnorm, sizeof(double), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
-            *out = sqrt(hs);
             return CL_OK;
         };
-        // z = L_D^{-1} v to cg_tol (diagonal-preconditioned CG, FP64)
-        // 16 CG iterations on fixed buffers (solution cx), replayed as one CUDA graph
-        double* cx = nullptr;
-        CK(mem.get(&cx, N));
-        constexpr int kCgBatch = 16;
-        cudaGraphExec_t cg_graph = nullptr;
-        struct GraphGuard {
-            cudaGraphExec_t* g;
-            ~GraphGuard() { if (*g) cudaGraphExecDestroy(*g); }
-        } guard{&cg_graph};
-        auto enqueue_cg = [&](cudaStream_t st) {
-            for (int k = 0; k < kCgBatch; ++k) {
-                k_cg_q64<<<kSBlk, kSB, 0, st>>>(a, cp, cq, cpart, cs);
-                k_cg_fin64<<<1, kSB, 0, st>>>(cpart, kSBlk, 1, cs);
-                k_cg_upd64<<<kSBlk, kSB, 0, st>>>(N, dinv, cp, cq, cx, cr, cpart, cs);
-                k_cg_fin64<<<1, kSB, 0, st>>>(cpart, kSBlk, 2, cs);
-                k_cg_p64<<<kSBlk, kSB, 0, st>>>(N, dinv, cr, cp, cs);
-            }
-        };
-        {
-            cudaStream_t cap = nullptr;
-            cudaGraph_t g = nullptr;
-            bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess;
-            if (ok) ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-            if (ok) {
-                enqueue_cg(cap);
-                ok = cudaStreamEndCapture(cap, &g) == cudaSuccess && g;
-            }
-            if (ok) ok = cudaGraphInstantiate(&cg_graph, g, 0) == cudaSuccess;
-            if (g) cudaGraphDestroy(g);
-            if (cap) cudaStreamDestroy(cap);
-            if (!ok) {
-                cg_graph = nullptr;
-                cudaGetLastError();  // the same kernels then run as plain launches
-            }
-        }
-        // z = L_D^{-1} v to cg_tol (diagonal-preconditioned CG, FP64)
-        auto precondition = [&](const double* v, double* z) -> cl_status {
-            k_cg_start64<<<kSBlk, kSB, 0, s>>>(N, v, dinv, cx, cr, cp, cpart);
-            k_cg_fin64<<<1, kSB, 0, s>>>(cpart, kSBlk, 0, cs);
-            CK(cudaGetLastError());
-            Cg64 hc;
-            CK(cudaMemcpyAsync(&hc, cs, sizeof(hc), cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            while (!hc.bad && hc.rr > cg_tol * cg_tol * hc.rr0 && hc.iters < 100000) {
-                if (cg_graph) CK(cudaGraphLaunch(cg_graph, s));
-                else enqueue_cg(s);
-                CK(cudaGetLastError());
-                CK(cudaMemcpyAsync(&hc, cs, sizeof(hc), cudaMemcpyDeviceToHost, s));
-                CK(cudaStreamSynchronize(s));
-            }
-            if (hc.bad == 1) { set_msg_txt("inner conjugate gradients broke down"); return CL_ERR_DIVERGED; }
-            CK(cudaMemcpyAsync(z, cx, sizeof(double) * (size_t)N, cudaMemcpyDeviceToDevice, s));
-            inf.inner_iterations += hc.iters;
-            return CL_OK;
-        };
-        k_schur_setup<<<kSBlk, kSB, 0, s>>>(a, om64, G, dinv);
         // start from the current state's concentration
-        k_field_to_f64<<<kSBlk, kSB, 0, s>>>(N, h->pop[h->cur], h->mask, h->src, x);
+        k_field64<<<nb, kSB, 0, s>>>(a, N, h->pop[h->cur], x);
         CK(cudaGetLastError());
         // the scale of the residual: |b| = |F(0)|, the right-hand side of (I - M) C = b; a warm
         // start that is already close needs no iteration
         double r0 = 0.0;
-        CK(cudaMemsetAsync(w, 0, sizeof(double) * (size_t)N, s));
-        CKS(apply_F(w, 0, V, nullptr));
+        CK(cudaMemsetAsync(w, 0, sizeof(double) * (size_t)n, s));
+        CKS(apply_F(w, 0, 0, V));
         CKS(norm(V, &r0));
         if (!(r0 > 0.0)) r0 = 1.0;
-        std::vector<double> H((size_t)(m + 1) * m), cs_(m), sn_(m), g(m + 1), hcol(m + 1);
+        std::vector<double> H((size_t)(m + 1) * m), cs_(m), sn_(m), g(m + 1), hcol(m + 1), hh(2 * (size_t)(m + 1) + 1);
         while (inf.iterations < max_iter) {
-            // r = F(x) - x  into V[0]
-            CKS(apply_F(x, 0, w, nullptr));
-            k_sub64<<<kSBlk, kSB, 0, s>>>(N, w, x, V);
-            CK(cudaGetLastError());
+            // r = F(x) - x  into V[0] (its negative; the sign enters below)
+            CKS(apply_F(x, 0, 1, w));
             double beta;
-            CKS(norm(V, &beta));
+            CKS(norm(w, &beta));
             inf.residual = beta / r0;
             if (!isfinite(beta)) { set_msg_txt("non-finite residual"); result = CL_ERR_DIVERGED; break; }
             if (beta <= tol * r0 || beta == 0.0) { result = CL_OK; break; }
-            k_axpy64<<<kSBlk, kSB, 0, s>>>(N, 1.0 / beta, V, V, 0);
+            k_scale64<<<nb, kSB, 0, s>>>(n, dnorm, w, V);
             std::fill(g.begin(), g.end(), 0.0);
-            g[0] = beta;
+            g[0] = -beta;
             int j = 0;
             for (; j < m && inf.iterations < max_iter; ++j) {
-                double* vj = V + (long long)j * N;
-                double* zj = Z + (long long)j * N;
-                CKS(precondition(vj, zj));
+                op.v = V + (long long)j * n;
+                op.z = Z + (long long)j * n;
+                CK(prec64(op, cg, s));
                 // w = (I - M) z = z - F_lin(z)
-                CKS(apply_F(zj, 1, w, nullptr));
-                k_sub64<<<kSBlk, kSB, 0, s>>>(N, zj, w, w);
-                // classical Gram-Schmidt, twice
-                for (int k = 0; k <= j; ++k) hcol[k] = 0.0;
+                CKS(apply_F(op.z, 1, 1, w));
+                // classical Gram-Schmidt, twice; |w| and the next vector
                 for (int pass = 0; pass < 2; ++pass) {
-                    k_mdot<<<kSBlk, kSB, 0, s>>>(V, N, j + 1, w, part);
-                    k_mdot_fin<<<(j + 1 + 127) / 128, 128, 0, s>>>(part, kSBlk, j + 1, hv);
-                    k_msub<<<kSBlk, kSB, 0, s>>>(V, N, j + 1, hv, w);
-                    CK(cudaGetLastError());
-                    std::vector<double> hh(j + 1);
-                    CK(cudaMemcpyAsync(hh.data(), hv, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, s));
-                    CK(cudaStreamSynchronize(s));
-                    for (int k = 0; k <= j; ++k) hcol[k] += hh[k];
+                    k_mdot<<<dim3(j + 1, chunks), kSB, 0, s>>>(V, n, w, part);
+                    k_msub<<<parts, kSB, 0, s>>>(V, n, j + 1, chunks, part, w, hv + (size_t)pass * (j + 1),
+                                                 pass ? nrm : nullptr);
                 }
-                double hn;
-                CKS(norm(w, &hn));
+                double* hn_dev = hv + 2 * (size_t)(j + 1);
+                k_norm_fin<<<1, kSB, 0, s>>>(nrm, parts, hn_dev);
+                k_scale64<<<nb, kSB, 0, s>>>(n, hn_dev, w, V + (long long)(j + 1) * n);
+                CK(cudaGetLastError());
+                PcgOut po;
+                CK(cudaMemcpyAsync(&po, cg.out, sizeof(po), cudaMemcpyDeviceToHost, s));
+                CK(cudaMemcpyAsync(hh.data(), hv, sizeof(double) * (2 * (size_t)(j + 1) + 1), cudaMemcpyDeviceToHost, s));
+                CK(cudaStreamSynchronize(s));
+                if (po.bad == 1) { set_msg_txt("inner conjugate gradients broke down"); return CL_ERR_DIVERGED; }
+                if (po.bad == 3) {
+                    set_msg_txt("a wait of the steady solve's blocks for one another ran out");
+                    return CL_ERR_TIMEOUT;
+                }
+                inf.inner_iterations += po.iters;
+                for (int k = 0; k <= j; ++k) hcol[k] = hh[k] + hh[j + 1 + k];
+                const double hn = hh[2 * (size_t)(j + 1)];
                 hcol[j + 1] = hn;
                 ++inf.iterations;
                 // Givens rotations of the new column
@@ -708,8 +629,6 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
                 g[j + 1] = -sn_[j] * g[j];
                 g[j] = cs_[j] * g[j];
                 for (int k = 0; k <= j; ++k) H[(size_t)k * m + j] = hcol[k];
-                if (hn > 0 && j + 1 <= m)
-                    k_axpy64<<<kSBlk, kSB, 0, s>>>(N, 1.0 / hn, w, V + (long long)(j + 1) * N, 0);
                 if (fabs(g[j + 1]) <= 0.5 * tol * r0 || hn == 0.0) { ++j; break; }
             }
             // x += Z y, y from the triangular system H y = g
@@ -719,26 +638,29 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
                 for (int l = k + 1; l < j; ++l) t -= H[(size_t)k * m + l] * y[l];
                 y[k] = t / H[(size_t)k * m + k];
             }
-            for (int k = 0; k < j; ++k) k_axpy64<<<kSBlk, kSB, 0, s>>>(N, y[k], Z + (long long)k * N, x, 1);
-            CK(cudaGetLastError());
+            if (j > 0) {
+                CK(cudaMemcpyAsync(dy, y.data(), sizeof(double) * j, cudaMemcpyHostToDevice, s));
+                k_comb64<<<nb, kSB, 0, s>>>(Z, n, j, dy, x);
+                CK(cudaGetLastError());
+                CK(cudaStreamSynchronize(s));  // y is the host's
+            }
             ++inf.cycles;
         }
         if (result == CL_ERR_NOT_CONVERGED) {
             // the residual of the last iterate
-            CKS(apply_F(x, 0, w, nullptr));
-            k_sub64<<<kSBlk, kSB, 0, s>>>(N, w, x, w);
+            CKS(apply_F(x, 0, 1, w));
             double rn;
             CKS(norm(w, &rn));
             inf.residual = r0 > 0 ? rn / r0 : 0.0;
             if (rn <= tol * r0) result = CL_OK;
         }
         // the state: post-collision populations of the steady field, and its fluxes in FP64
-        double* out3 = nullptr;
-        CK(mem.get(&out3, 3 * N));
-        CK(cudaMemsetAsync(out3, 0, sizeof(double) * 3 * (size_t)N, s));
-        CKS(apply_F(x, 0, w, h->pop[h->cur], out3));
-        k_sum3<<<kSBlk, kSB, 0, s>>>(N, out3, part);
-        k_sum3_fin<<<1, kSB, 0, s>>>(part, kSBlk, hv);
+        double* flux = nullptr;
+        CK(mem.get(&flux, 5LL * n));
+        CK(cudaMemsetAsync(flux, 0, sizeof(double) * 5 * (size_t)n, s));
+        k_walk<true><<<dim3(nb, 3), kSB, 0, s>>>(a, x, T, 0, h->pop[h->cur], N, flux);
+        k_walk_fin<true><<<nb, kSB, 0, s>>>(a, x, T, 0, 0, w, h->pop[h->cur]);
+        k_flux_sum<<<1, 1024, 0, s>>>(flux, n, hv);
         CK(cudaGetLastError());
         double fl[3];
         CK(cudaMemcpyAsync(fl, hv, sizeof(fl), cudaMemcpyDeviceToHost, s));
