@@ -147,7 +147,8 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
     constexpr int KR = K > 0 ? K : 1;
     constexpr int NW = NT / 32;
     constexpr bool kKeep = K > 0 && K * sizeof(typename Op::Row) <= 192;  // rows stay in registers too
-    __shared__ double sh[3][NW];
+    static_assert(NW % 2 == 0 && NW >= 4, "an even number of warps");
+    __shared__ double sh[3][sizeof(T) == 8 ? NT : NW];
     __shared__ double box[3][kPcgMaxCluster];
     __shared__ double tot[3];
     __shared__ T s_al, s_be;  // alpha, beta of the next iteration
@@ -192,20 +193,39 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
             g1 = fma(w, u, g1);
             g2 = fma(r, r, g2);
         });
+        if constexpr (sizeof(T) == 8) {
+            // three warps add up the threads' sums: a shuffle tree in every warp would issue an FP64 addition for
+            // idle lanes too, and those are what the SM has least of
+            sh[0][tid] = g0;
+            sh[1][tid] = g1;
+            sh[2][tid] = g2;
+        } else {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            g0 += __shfl_xor_sync(0xffffffffu, g0, o);
-            g1 += __shfl_xor_sync(0xffffffffu, g1, o);
-            g2 += __shfl_xor_sync(0xffffffffu, g2, o);
-        }
-        if (lane == 0) {
-            sh[0][warp] = (double)g0;
-            sh[1][warp] = (double)g1;
-            sh[2][warp] = (double)g2;
+            for (int o = 16; o > 0; o >>= 1) {
+                g0 += __shfl_xor_sync(0xffffffffu, g0, o);
+                g1 += __shfl_xor_sync(0xffffffffu, g1, o);
+                g2 += __shfl_xor_sync(0xffffffffu, g2, o);
+            }
+            if (lane == 0) {
+                sh[0][warp] = (double)g0;
+                sh[1][warp] = (double)g1;
+                sh[2][warp] = (double)g2;
+            }
         }
         __syncthreads();
         if (warp < 3) {
-            double v = lane < NW ? sh[warp][lane] : 0.0;
+            double v = 0.0;
+            if constexpr (sizeof(T) == 8) {
+                double v2 = 0.0;
+#pragma unroll
+                for (int k = 0; k < NW; k += 2) {
+                    v += sh[warp][k * 32 + lane];
+                    v2 += sh[warp][k * 32 + 32 + lane];
+                }
+                v += v2;
+            } else {
+                v = lane < NW ? sh[warp][lane] : 0.0;
+            }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             sync.put(a.meet, box, warp, v, lane);  // every lane holds the sum
@@ -229,19 +249,23 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
         R(k, i) = b;
         a.u[i] = d * b;
     });
-    PcgOut o;  // thread 0's
+    // the scalars are the last warp's: with few cells a block it has none, and forms the reciprocals of the next
+    // iteration's ratios while the others update
+    constexpr int kLead = NT - 32;
+    PcgOut o;
     o.iters = o.bad = 0;
     o.rr = o.rr0 = 0.0;
-    double gamma = 0.0;
-    T alpha = T(0);
+    T inv_gamma = T(0), inv_alpha = T(0);
     bool met = true;
     for (bool start = true;; start = false) {
         met = apply();
         if (!met) break;
-        if (tid == 0) {
+        T gn_t = T(0), alpha = T(0);
+        if (tid == kLead) {
             const double gn = tot[0], delta = tot[1], rr = tot[2];
             int go = 1;
             T be = T(0);
+            gn_t = (T)gn;
             o.rr = rr;
             if (start) o.rr0 = rr;
             else ++o.iters;
@@ -252,16 +276,15 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
                 // ratios in the vectors' own type
                 T den = (T)delta;
                 if (!start) {
-                    be = (T)gn / (T)gamma;
-                    den -= be * (T)gn / alpha;
+                    be = gn_t * inv_gamma;
+                    den -= be * gn_t * inv_alpha;
                 }
                 if (!(den > T(0))) {  // rounding has spoilt the recurrence: start it again from this residual
                     den = (T)delta;
                     be = T(0);
                 }
                 if (!(den > T(0)) || !(gn > 0.0)) { o.bad = 1; go = 0; }
-                else alpha = (T)gn / den;
-                gamma = gn;
+                else alpha = gn_t / den;
             }
             s_al = alpha;
             s_be = be;
@@ -270,6 +293,10 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
         __syncthreads();
         if (!s_go) break;
         const T al = s_al, be = s_be;
+        if (tid == kLead) {
+            inv_gamma = T(1) / gn_t;
+            inv_alpha = T(1) / alpha;
+        }
         each([&](int k, int i) {
             const T d = D(k, i), r = R(k, i);
             const T p = fma(be, P(k, i), d * r);
@@ -284,7 +311,7 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
     }
     if (!met) o.bad = 3;
     each([&](int k, int i) { op.done(i, X(k, i)); });
-    if (blockIdx.x == 0 && tid == 0) *a.out = o;
+    if (blockIdx.x == 0 && tid == kLead) *a.out = o;
 }
 
 // SMs of the current device

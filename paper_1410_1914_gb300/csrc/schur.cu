@@ -44,12 +44,12 @@ constexpr int kSB = 256;          // threads per block
 constexpr double kWa = 0.125;     // D3Q7 axis weight
 constexpr double kWr = 0.25;      // D3Q7 rest weight
 
-// A run of open faces along one axis: len cells from i on, or -len for a
-// closed loop (y, z) of len cells.  p = kL g*_-(first) + hL enters at the
+// A run of open faces along one axis: len cells, or -len for a closed loop
+// (y, z) of len cells, listed in order from entry pos of the axis on.  p = kL g*_-(first) + hL enters at the
 // first cell, m = kR g*_+(last) + hR at the last; al is the product of the
 // cells' decays 1 - omega, inv = 1 / (1 - kL al kR al) (a loop: 1 / (1 - al)).
 struct Run {
-    int i, len;
+    int pos, len;
     double al, inv, kL, kR, hL, hR;
 };
 
@@ -69,7 +69,9 @@ struct SchurArgs {
     double* G;      // [6][n] conductance of each link (0 where closed)
     double* dinv;   // [n] 1 / diagonal of the finite-volume operator
     Run* runs;      // [3][n]
-    int* n_runs;    // [3]
+    int* ord;       // [3][n] the cells of each axis run by run, and
+    double2* dso;   // [3][n] their 1 - omega and omega w
+    int* n_runs;    // [3] runs, then [3] cells listed
 };
 
 __device__ __forceinline__ double cat_factor(const SchurArgs& a, int c) {
@@ -125,37 +127,44 @@ __global__ void __launch_bounds__(kSB) k_schur_runs(SchurArgs a) {
     const int* __restrict__ bwd = a.nb + (long long)(2 * ax + 1) * a.n;
     for (int i = blockIdx.x * kSB + threadIdx.x; i < a.n; i += gridDim.x * kSB) {
         Run r;
-        r.i = i;
+        const bool start = bwd[i] < 0;
+        if (!start) {
+            if (ax == 0) continue;
+            const int c = a.list[i];
+            if ((ax == 1 ? (c / a.nx) % a.ny : c / (a.nx * a.ny)) != 0) continue;
+        }
+        int len = 1, last = i, t = fwd[i];
         r.al = 1.0 - a.om64[i];
-        if (bwd[i] < 0) {
-            int last = i;
-            r.len = 1;
-            for (int t = fwd[i]; t >= 0; t = fwd[t]) {
-                r.al *= 1.0 - a.om64[t];
-                last = t;
-                ++r.len;
-            }
+        for (; t >= 0 && t != i; t = fwd[t]) {
+            r.al *= 1.0 - a.om64[t];
+            last = t;
+            ++len;
+        }
+        if (start) {
+            r.len = len;
             end_rule(a, bwd[i], true, a.list[i], r.kL, r.hL);
             end_rule(a, fwd[last], false, a.list[last], r.kR, r.hR);
             r.inv = 1.0 / (1.0 - r.kL * r.al * r.kR * r.al);
         } else {
-            if (ax == 0) continue;
-            const int c = a.list[i];
-            const int coord = ax == 1 ? (c / a.nx) % a.ny : c / (a.nx * a.ny);
-            if (coord != 0) continue;
-            int len = 1, t = fwd[i];
-            for (; t >= 0 && t != i; t = fwd[t]) {
-                r.al *= 1.0 - a.om64[t];
-                ++len;
-            }
             if (t != i) continue;  // the line has a closed face
             r.len = -len;
             r.inv = 1.0 / (1.0 - r.al);
             r.kL = r.kR = r.hL = r.hR = 0.0;
         }
+        r.pos = atomicAdd(a.n_runs + 3 + ax, len);
+        const long long at = (long long)ax * a.n + r.pos;
+        for (int k = 0, u = i; k < len; ++k, u = fwd[u]) {
+            a.ord[at + k] = u;
+            a.dso[at + k] = make_double2(1.0 - a.om64[u], a.om64[u] * kWa);
+        }
         a.runs[(long long)ax * a.n + atomicAdd(a.n_runs + ax, 1)] = r;
     }
 }
+
+// A warp's time is its longest run's FP64 instructions, at 16 cycles each on
+// an SM: blocks of one warp spread the runs over the SMs (16^3: 23 us with 256
+// threads a block).
+constexpr int kWalkT = 32;
 
 // One thread per run: the incoming populations of the two directions of its
 // axis from C into T[axis] (their sum).  OUT: also the post-collision
@@ -163,34 +172,35 @@ __global__ void __launch_bounds__(kSB) k_schur_runs(SchurArgs a) {
 // consumed on its catalytic ends (flux[axis]), entering at x = 0 (flux[3]) and
 // leaving at x = L (flux[4]), lattice units per step, FP64.
 template <bool OUT>
-__global__ void __launch_bounds__(kSB) k_walk(SchurArgs a, const double* __restrict__ C, double* __restrict__ T,
+__global__ void __launch_bounds__(kWalkT) k_walk(SchurArgs a, const double* __restrict__ C, double* __restrict__ T,
                                               int homog, float* __restrict__ pop, long long N,
                                               double* __restrict__ flux) {
     const int ax = blockIdx.y, n = a.n;
-    const int* __restrict__ fwd = a.nb + (long long)(2 * ax) * n;
-    const int* __restrict__ bwd = a.nb + (long long)(2 * ax + 1) * n;
     double* __restrict__ Ta = T + (long long)ax * n;
     const int nr = a.n_runs[ax];
-    auto coef = [&](int i, double& dec, double& s) {
-        const double om = a.om64[i];
-        dec = 1.0 - om;
-        s = om * kWa * C[i] + (homog || !a.src ? 0.0 : kWa * a.src[a.list[i]]);
-    };
-    for (int q = blockIdx.x * kSB + threadIdx.x; q < nr; q += gridDim.x * kSB) {
+    const bool src = !homog && a.src;
+    for (int q = blockIdx.x * kWalkT + threadIdx.x; q < nr; q += gridDim.x * kWalkT) {
         const Run r = a.runs[(long long)ax * n + q];
         const bool loop = r.len < 0;
         const int len = loop ? -r.len : r.len;
+        const int* __restrict__ ord = a.ord + (long long)ax * n + r.pos;
+        const double2* __restrict__ dso = a.dso + (long long)ax * n + r.pos;
+        auto coef = [&](int t, double& dec, double& s) {
+            const double2 ds = dso[t];
+            const int i = ord[t];
+            dec = ds.x;
+            s = ds.y * C[i];
+            if (src) s += kWa * a.src[a.list[i]];
+        };
         // forward: g*_+(last) = al p + beB; backward: g*_-(first) = al m + beA
         double beA = 0.0, beB = 0.0, pre = 1.0;
-        int last = r.i;
-        for (int t = 0, i = r.i; t < len; ++t) {
+#pragma unroll 4
+        for (int t = 0; t < len; ++t) {
             double dec, s;
-            coef(i, dec, s);
-            beB = dec * beB + s;
-            beA += pre * s;
+            coef(t, dec, s);
+            beB = fma(dec, beB, s);
+            beA = fma(pre, s, beA);
             pre *= dec;
-            last = i;
-            i = ax == 0 ? i + 1 : fwd[i];
         }
         double p, m;
         if (loop) {
@@ -204,36 +214,39 @@ __global__ void __launch_bounds__(kSB) k_walk(SchurArgs a, const double* __restr
             if (OUT) {
                 // what leaves through the run's end faces: g*_-(first) and g*_+(last)
                 const double gA = r.al * m + beA, gB = r.al * p + beB;
-                const int tA = bwd[r.i], tB = fwd[last];
+                const int first = ord[0];
+                const int tA = a.nb[(long long)(2 * ax + 1) * n + first], tB = a.nb[(long long)(2 * ax) * n + ord[len - 1]];
                 double R = 0.0, jin = 0.0, jout = 0.0;
                 if (tA == DSA_FIXED) jin = 2.0 * kWa * a.c_in - 2.0 * gA;
                 else if (tA == DSA_SINK) R += (1.0 - r.kL) * gA;
                 if (tB == DSA_FIXED) jout = 2.0 * gB - 2.0 * kWa * a.c_out;
                 else if (tB == DSA_SINK) R += (1.0 - r.kR) * gB;
-                flux[(long long)ax * n + r.i] = R;
+                flux[(long long)ax * n + first] = R;
                 if (ax == 0) {
-                    flux[3LL * n + r.i] = jin;
-                    flux[4LL * n + r.i] = jout;
+                    flux[3LL * n + first] = jin;
+                    flux[4LL * n + first] = jout;
                 }
             }
         }
         double g = p;
-        for (int t = 0, i = r.i; t < len; ++t) {
+#pragma unroll 4
+        for (int t = 0; t < len; ++t) {
             double dec, s;
-            coef(i, dec, s);
+            coef(t, dec, s);
+            const int i = ord[t];
             Ta[i] = g;
-            g = dec * g + s;
+            g = fma(dec, g, s);
             if (OUT) pop[(1 + 2 * ax) * N + a.list[i]] = (float)g;
-            i = ax == 0 ? i + 1 : fwd[i];
         }
         g = m;
-        for (int t = 0, i = last; t < len; ++t) {
+#pragma unroll 4
+        for (int t = len - 1; t >= 0; --t) {
             double dec, s;
-            coef(i, dec, s);
+            coef(t, dec, s);
+            const int i = ord[t];
             Ta[i] += g;
-            g = dec * g + s;
+            g = fma(dec, g, s);
             if (OUT) pop[(2 + 2 * ax) * N + a.list[i]] = (float)g;
-            i = ax == 0 ? i - 1 : bwd[i];
         }
     }
 }
@@ -504,12 +517,19 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
         CK(mem.get(&a.G, 6LL * n));
         CK(mem.get(&a.dinv, n));
         CK(mem.get(&a.runs, 3LL * n));
-        CK(mem.get(&a.n_runs, 3));
-        CK(cudaMemsetAsync(a.n_runs, 0, 3 * sizeof(int), s));
+        CK(mem.get(&a.ord, 3LL * n));
+        CK(mem.get(&a.dso, 3LL * n));
+        CK(mem.get(&a.n_runs, 6));
+        CK(cudaMemsetAsync(a.n_runs, 0, 6 * sizeof(int), s));
         const int nb = std::min((n + kSB - 1) / kSB, 152 * 8);
         k_schur_setup<<<nb, kSB, 0, s>>>(a);
         k_schur_runs<<<dim3(nb, 3), kSB, 0, s>>>(a);
         CK(cudaGetLastError());
+        int n_runs[3];
+        CK(cudaMemcpyAsync(n_runs, a.n_runs, sizeof(n_runs), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        const int most_runs = std::max(1, std::max(n_runs[0], std::max(n_runs[1], n_runs[2])));
+        const dim3 walk_grid(std::min((most_runs + kWalkT - 1) / kWalkT, 152 * 64), 3);
         double *V = nullptr, *Z = nullptr, *x = nullptr, *w = nullptr, *T = nullptr, *part = nullptr, *nrm = nullptr;
         double *hv = nullptr, *dy = nullptr;
         const int chunks = (n + kDotCells - 1) / kDotCells, parts = (n + 31) / 32;
@@ -549,7 +569,7 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
         op.dinv_ = a.dinv;
         // F(C) (affine: homog = 0; linear part: homog = 1) or C - F(C) (minus) into out
         auto apply_F = [&](const double* C, int homog, int minus, double* out) -> cl_status {
-            k_walk<false><<<dim3(nb, 3), kSB, 0, s>>>(a, C, T, homog, nullptr, N, nullptr);
+            k_walk<false><<<walk_grid, kWalkT, 0, s>>>(a, C, T, homog, nullptr, N, nullptr);
             k_walk_fin<false><<<nb, kSB, 0, s>>>(a, C, T, homog, minus, out, nullptr);
             CK(cudaGetLastError());
             return CL_OK;
@@ -658,7 +678,7 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
         double* flux = nullptr;
         CK(mem.get(&flux, 5LL * n));
         CK(cudaMemsetAsync(flux, 0, sizeof(double) * 5 * (size_t)n, s));
-        k_walk<true><<<dim3(nb, 3), kSB, 0, s>>>(a, x, T, 0, h->pop[h->cur], N, flux);
+        k_walk<true><<<walk_grid, kWalkT, 0, s>>>(a, x, T, 0, h->pop[h->cur], N, flux);
         k_walk_fin<true><<<nb, kSB, 0, s>>>(a, x, T, 0, 0, w, h->pop[h->cur]);
         k_flux_sum<<<1, 1024, 0, s>>>(flux, n, hv);
         CK(cudaGetLastError());
