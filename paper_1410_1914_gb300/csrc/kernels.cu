@@ -5,7 +5,7 @@
 
 #include "device_util.cuh"
 #include "internal.cuh"
-#include "uf.cuh"
+#include "ccl.cuh"
 
 namespace cl {
 
@@ -29,42 +29,15 @@ cudaError_t launch_validate(const uint8_t* phase, long long N, int* d_err, cudaS
 
 // ------------------------------------------------ percolation (union-find)
 // Transport cells 6-connected (y, z periodic) to the inlet plane x = 0.
-// Union-find helpers: uf.cuh.
+// Labelling: ccl.cu.
 
-__global__ void k_uf_init(const uint8_t* __restrict__ phase, long long N, int tmask, int* L,
-                          uint8_t* touch) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        L[c] = is_transport(phase[c], tmask) ? (int)c : -1;
-        touch[c] = 0;
+// components that reach the inlet plane: one thread per row
+__global__ void k_uf_touch(int nx, long long rows, const int* __restrict__ L, uint8_t* touch) {
+    for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < rows;
+         r += (long long)gridDim.x * blockDim.x) {
+        const int root = L[r * nx];
+        if (root >= 0 && !touch[root]) touch[root] = 1;
     }
-}
-
-__global__ void k_uf_merge(const uint8_t* __restrict__ phase, int nx, int ny, int nz, int tmask, int* L,
-                           int* err) {
-    const long long N = (long long)nx * ny * nz;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        if (!is_transport(phase[c], tmask)) continue;
-        const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-        if (x > 0 && is_transport(phase[c - 1], tmask)) uf_union(L, (int)c, (int)(c - 1), err);
-        long long n = x + (long long)nx * (wrapi(y - 1, ny) + (long long)ny * z);
-        if (n != c && is_transport(phase[n], tmask)) uf_union(L, (int)c, (int)n, err);
-        n = x + (long long)nx * (y + (long long)ny * wrapi(z - 1, nz));
-        if (n != c && is_transport(phase[n], tmask)) uf_union(L, (int)c, (int)n, err);
-    }
-}
-
-__global__ void k_uf_flatten(long long N, int* L, int* err) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x)
-        if (L[c] >= 0) L[c] = uf_find(L, (int)c, err);
-}
-
-__global__ void k_uf_touch(int nx, long long N, const int* __restrict__ L, uint8_t* touch) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x)
-        if (c % nx == 0 && L[c] >= 0) touch[L[c]] = 1;
 }
 
 __global__ void k_uf_active(long long N, const int* __restrict__ L, const uint8_t* __restrict__ touch,
@@ -78,10 +51,11 @@ cudaError_t launch_percolation(const uint8_t* phase, int nx, int ny, int nz, int
                                uint8_t* touch, uint8_t* active, int* d_err, cudaStream_t s) {
     const long long N = (long long)nx * ny * nz;
     const int g = 152 * 8, b = 256;
-    k_uf_init<<<g, b, 0, s>>>(phase, N, tmask, labels, touch);
-    k_uf_merge<<<g, b, 0, s>>>(phase, nx, ny, nz, tmask, labels, d_err);
-    k_uf_flatten<<<g, b, 0, s>>>(N, labels, d_err);
-    k_uf_touch<<<g, b, 0, s>>>(nx, N, labels, touch);
+    cudaError_t e = launch_ccl(phase, nx, ny, nz, (unsigned)tmask, true, true, labels, d_err, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(touch, 0, (size_t)N, s);
+    if (e != cudaSuccess) return e;
+    const long long rows = (long long)ny * nz;
+    k_uf_touch<<<(int)(rows < (long long)g * b ? (rows + b - 1) / b : g), b, 0, s>>>(nx, rows, labels, touch);
     k_uf_active<<<g, b, 0, s>>>(N, labels, touch, active);
     return cudaGetLastError();
 }
