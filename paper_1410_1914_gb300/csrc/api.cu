@@ -363,11 +363,14 @@ cl_status need_structure(cl_lbm* h) {
 
 
 // stats + dt + omega, shared by set_structure and set_diffusivity
-cl_status derive_relaxation(cl_lbm* h, bool with_dp) {
+// with_dp: new pore lengths, as dp per cell or (counted) as the sums in d_plane
+cl_status derive_relaxation(cl_lbm* h, bool with_dp, bool counted) {
     double* stat_out = h->d_red + 8;  // 7 slots
-    CK(launch_stats(h->phase, h->mask, h->D, with_dp ? h->dp : nullptr, h->N, h->nx, transport_phases(h->p),
-                    h->partials, h->nblk_stats, stat_out, h->s));
+    CK(launch_stats(h->phase, h->mask, h->D, with_dp && !counted ? h->dp : nullptr, h->N, h->nx,
+                    transport_phases(h->p), h->partials, h->nblk_stats, stat_out, h->s));
     double st[7];
+    unsigned long long runs[4] = {0, 0, 0, 0};
+    if (counted) CK(cudaMemcpyAsync(runs, h->d_plane, sizeof(runs), cudaMemcpyDeviceToHost, h->s));
     CK(cudaMemcpyAsync(st, stat_out, sizeof(st), cudaMemcpyDeviceToHost, h->s));
     CK(cudaStreamSynchronize(h->s));
     h->info.n_cells = h->N;
@@ -375,7 +378,12 @@ cl_status derive_relaxation(cl_lbm* h, bool with_dp) {
     h->info.n_active = (long long)st[1];
     h->info.n_wall_links = (long long)st[2];
     h->info.n_react_links = (long long)st[3];
-    if (with_dp) h->info.mean_pore_diameter_m = st[5] > 0 ? st[4] / st[5] : 0.0;
+    if (counted)
+        h->info.mean_pore_diameter_m =
+            runs[3] ? ((double)runs[0] + sqrt(2.0) * (double)runs[1] + sqrt(3.0) * (double)runs[2]) * h->p.dx_m / 13.0 /
+                          (double)runs[3]
+                    : 0.0;
+    else if (with_dp) h->info.mean_pore_diameter_m = st[5] > 0 ? st[4] / st[5] : 0.0;
     if (h->info.n_active == 0) { set_msg_txt("no transport cell is connected to the inlet plane"); return CL_ERR_NO_PATH; }
     h->D_max = st[6];
     if (!(h->D_max > 0) || !isfinite(h->D_max)) { set_msg_txt("largest diffusivity is not positive"); return CL_ERR_ARG; }
@@ -728,16 +736,18 @@ cl_status cl_lbm_set_structure(cl_handle h, const uint8_t* phase, const uint8_t*
     CK(launch_percolation(h->phase, h->nx, h->ny, h->nz, transport_phases(h->p), h->labels, h->touch, h->active,
                           h->d_err, h->s));
     CKS(check_err_flag(h));
+    bool counted = false;
     // Eq. 7 unless the bulk value is given
     h->D_b = h->p.D_bulk > 0 ? h->p.D_bulk : 0.22e-4 * pow(h->p.T_K / 293.2, 1.5) / h->p.p_atm;
     CK(launch_diffusivity(h->phase, h->active, h->nx, h->ny, h->nz, h->p.dx_m, h->p.T_K, h->p.M_kgmol, h->D_b,
-                          h->p.D_ionomer, h->p.knudsen, nullptr, h->D, h->dp, nullptr, h->s));
+                          h->p.D_ionomer, h->p.knudsen, nullptr, h->D, h->dp, nullptr,
+                          (unsigned long long*)h->d_plane, &counted, h->s));
     CK(launch_masks(h->phase, h->active, h->have_react ? h->react : nullptr, h->p.react_rule, h->nx, h->ny,
                     h->nz, h->mask, h->s));
     if (h->q == 19)
         CK(launch_masks19(h->phase, h->active, h->have_react ? h->react : nullptr, h->p.react_rule, h->nx, h->ny,
                           h->nz, h->px19, h->mask19, h->react19, h->s));
-    CKS(derive_relaxation(h, true));
+    CKS(derive_relaxation(h, true, counted));
     CKS(do_init(h, nullptr));
     CK(cudaStreamSynchronize(h->s));
     h->have_structure = true;
@@ -750,10 +760,10 @@ cl_status cl_lbm_set_diffusivity(cl_handle h, const double* D, int ptr_is_device
     CK(cudaMemcpyAsync(h->dp, D, sizeof(double) * (size_t)h->N, kind_in(ptr_is_device), h->s));
     CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->s));
     CK(launch_diffusivity(h->phase, h->active, h->nx, h->ny, h->nz, h->p.dx_m, h->p.T_K, h->p.M_kgmol, h->D_b,
-                          h->p.D_ionomer, h->p.knudsen, h->dp, h->D, nullptr, nullptr, h->s));
+                          h->p.D_ionomer, h->p.knudsen, h->dp, h->D, nullptr, nullptr, nullptr, nullptr, h->s));
     CK(launch_check_positive(h->active, h->D, h->N, h->d_err, h->s));
     CKS(check_err_flag(h));
-    CKS(derive_relaxation(h, false));
+    CKS(derive_relaxation(h, false, false));
     CKS(do_init(h, nullptr));
     CK(cudaStreamSynchronize(h->s));
     return CL_OK;

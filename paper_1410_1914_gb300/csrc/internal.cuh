@@ -117,10 +117,12 @@ cudaError_t launch_validate(const uint8_t* phase, long long N, int* d_err, cudaS
 cudaError_t launch_percolation(const uint8_t* phase, int nx, int ny, int nz, int transport_phase_mask,
                                int* labels, uint8_t* touch, uint8_t* active, int* d_err,
                                cudaStream_t s);
+// tot (4) allows the bit-mask path; *counted says that it was taken: dp was then its scratch, and tot holds the run
+// sums of chords.cuh instead
 cudaError_t launch_diffusivity(const uint8_t* phase, const uint8_t* active, int nx, int ny, int nz,
                                double dx, double T, double M, double D_b, double D_ionomer,
                                int knudsen, const double* D_override, double* D, double* dp,
-                               int32_t* chord13, cudaStream_t s);
+                               int32_t* chord13, unsigned long long* tot, bool* counted, cudaStream_t s);
 cudaError_t launch_chords13(const uint8_t* phase, int nx, int ny, int nz, int32_t* chord13,
                             cudaStream_t s);
 cudaError_t launch_check_positive(const uint8_t* active, const double* D, long long N, int* d_err,

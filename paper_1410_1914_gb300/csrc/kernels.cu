@@ -6,6 +6,7 @@
 #include "device_util.cuh"
 #include "internal.cuh"
 #include "ccl.cuh"
+#include "chords.cuh"
 
 namespace cl {
 
@@ -398,21 +399,30 @@ static long long gcd_host(long long a, long long b) {
 cudaError_t launch_diffusivity(const uint8_t* phase, const uint8_t* active, int nx, int ny, int nz,
                                double dx, double T, double M, double D_b, double D_ionomer, int knudsen,
                                const double* D_override, double* D, double* dp, int32_t* chord13,
-                               cudaStream_t s) {
+                               unsigned long long* tot, bool* counted, cudaStream_t s) {
+    if (counted) *counted = false;
     if (!dp || D_override || chord13) {
         k_diffusivity<<<152 * 16, 128, 0, s>>>(phase, active, nx, ny, nz, dx, T, M, D_b, D_ionomer, knudsen,
                                                D_override, D, dp, chord13);
         return cudaGetLastError();
     }
     const long long N = (long long)nx * ny * nz;
-    cudaError_t e = cudaMemsetAsync(dp, 0, sizeof(double) * (size_t)N, s);
-    if (e != cudaSuccess) return e;
     // lines longer than the warp kernels' masks hold take one thread per line;
     // CL_LBM_LINE_THREADS=1 takes that path on any box (it is tested that way)
     static const bool force_threads = [] {
         const char* e = getenv("CL_LBM_LINE_THREADS");
         return e && atoi(e) != 0;
     }();
+    // Bit masks where they apply: 1.7 ms against 3.0 + 0.8 ms at 256^3.  Boxes of short rows (whose bit sets
+    // would not fit dp) and lines longer than the line kernels' masks stay with the lines.
+    const double vkn = sqrt(8.0 * 8.314462618 * T / (M_PI * M));
+    if (counted && tot && !force_threads &&
+        chord_bits_fit(nx, ny, nz, 32 * kChordChunks - 1, dx, vkn, D_b)) {
+        *counted = true;
+        return launch_chord_bits(phase, active, nx, ny, nz, dx, vkn, D_b, D_ionomer, knudsen, dp, D, tot, s);
+    }
+    cudaError_t e = cudaMemsetAsync(dp, 0, sizeof(double) * (size_t)N, s);
+    if (e != cudaSuccess) return e;
     const int dirs[13][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1},  {1, 1, 0},  {1, -1, 0},
                              {1, 0, 1},  {1, 0, -1}, {0, 1, 1},  {0, 1, -1}, {1, 1, 1},
                              {1, 1, -1}, {1, -1, 1}, {1, -1, -1}};
@@ -444,7 +454,6 @@ cudaError_t launch_diffusivity(const uint8_t* phase, const uint8_t* active, int 
             }
         }
     }
-    const double vkn = sqrt(8.0 * 8.314462618 * T / (M_PI * M));
     k_diffusivity_dp<<<152 * 16, 128, 0, s>>>(phase, active, N, vkn, 1.0 / D_b, D_b, D_ionomer, knudsen, D, dp);
     return cudaGetLastError();
 }
@@ -482,15 +491,24 @@ cudaError_t launch_check_positive(const uint8_t* active, const double* D, long l
 
 // ---------------------------------------------------- omega (Eq. 24, D3Q7)
 // tau = 1/2 + (tau_ref - 1/2) D / D_max  (dt fixed by tau_ref at D_max)
-__global__ void k_omega(const uint8_t* __restrict__ active, const double* __restrict__ D, long long N,
-                        double tau_ref, const double* __restrict__ Dmax, float* omega) {
-    const double dmax = *Dmax;
+// FP64 issues at 1/64 of the FP32 rate, and two FP64 divisions a cell were the
+// time of this kernel (0.48 ms at 256^3): the factor (tau_ref - 1/2) / D_max
+// is formed once per block, and 1/tau comes from the f32 reciprocal and one
+// Newton step in FP64 (48 bits, then rounded to f32; tau lies in (1/2, tau_ref]).
+__global__ void __launch_bounds__(256) k_omega(const uint8_t* __restrict__ active, const double* __restrict__ D,
+                                               long long N, double tau_ref, const double* __restrict__ Dmax,
+                                               float* omega) {
+    __shared__ double f;
+    if (threadIdx.x == 0) f = (tau_ref - 0.5) / *Dmax;
+    __syncthreads();
+    const double k = f;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
          c += (long long)gridDim.x * blockDim.x) {
         float om = 0.f;
         if (active[c]) {
-            const double tau = 0.5 + (tau_ref - 0.5) * D[c] / dmax;
-            om = (float)(1.0 / tau);
+            const double tau = fma(D[c], k, 0.5);
+            const double r = (double)__frcp_rn((float)tau);
+            om = (float)fma(r, fma(-tau, r, 1.0), r);
         }
         omega[c] = om;
     }
@@ -503,66 +521,88 @@ cudaError_t launch_omega(const uint8_t* active, const double* D, long long N, do
 }
 
 // --------------------------------------------------------------- link masks
-__global__ void k_masks(const uint8_t* __restrict__ phase, const uint8_t* __restrict__ active,
-                        const uint8_t* __restrict__ react_in, int rule, int nx, int ny, int nz,
-                        uint16_t* mask) {
-    const long long N = (long long)nx * ny * nz;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
+// One warp per row of 32 cells: the neighbours along x come from the row's
+// active bits, the others from the four neighbouring rows.
+__global__ void __launch_bounds__(256) k_masks(const uint8_t* __restrict__ phase, const uint8_t* __restrict__ active,
+                                               const uint8_t* __restrict__ react_in, int rule, int nx, int ny, int nz,
+                                               uint16_t* __restrict__ mask) {
+    const int lane = threadIdx.x & 31;
+    const int nw = (nx + 31) >> 5;
+    const long long words = (long long)nw * ny * nz;
+    const bool reacts = rule != CL_REACT_GIVEN || react_in;
+    for (long long w = blockIdx.x * 8LL + (threadIdx.x >> 5); w < words; w += gridDim.x * 8LL) {
+        const int row = (int)(w / nw), wx = (int)(w - (long long)row * nw);
+        const int y = row % ny, z = row / ny;
+        const int x = wx * 32 + lane;
+        const bool in = x < nx;
+        const long long c = x + (long long)nx * row;
+        const bool act = in && active[c];
+        const unsigned a = __ballot_sync(0xffffffffu, act);
+        if (a == 0) {
+            if (in) mask[c] = 0;
+            continue;
+        }
+        const int rows[4] = {y == ny - 1 ? row - (ny - 1) : row + 1, y == 0 ? row + (ny - 1) : row - 1,
+                             z == nz - 1 ? row - ny * (nz - 1) : row + ny, z == 0 ? row + ny * (nz - 1) : row - ny};
         uint16_t m = 0;
-        if (active[c]) {
+        if (act) {
             m = kActiveBit;
-            const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-            const int dx[6] = {1, -1, 0, 0, 0, 0}, dy[6] = {0, 0, 1, -1, 0, 0}, dz[6] = {0, 0, 0, 0, 1, -1};
+            const uint8_t pc = reacts ? phase[c] : 0;
+            const unsigned given = rule == CL_REACT_GIVEN ? (react_in ? react_in[c] : 0u)
+                                                          : (rule == CL_REACT_ALL_PORE_SOLID ? pc == 0 : pc == 2) ? 0x3fu : 0u;
+#pragma unroll
             for (int d = 0; d < 6; ++d) {
-                const int qx = x + dx[d];
+                const int qx = x + (d == 0) - (d == 1);
                 if (qx < 0 || qx >= nx) { m |= (uint16_t)(1u << (kClosedShift + d)); continue; }
-                const long long n = qx + (long long)nx * (wrapi(y + dy[d], ny) + (long long)ny * wrapi(z + dz[d], nz));
-                if (active[n]) continue;
+                const long long n = d < 2 ? c + (d == 0 ? 1 : -1) : x + (long long)nx * rows[d < 2 ? 0 : d - 2];
+                // the row's own bits, except past the ends of these 32 cells
+                const bool on = d == 0 && lane < 31 ? (a >> (lane + 1)) & 1u
+                                : (d == 1 && lane > 0 ? (a >> (lane - 1)) & 1u : active[n] != 0);
+                if (on) continue;
                 m |= (uint16_t)(1u << (kClosedShift + d));
-                bool react = false;
-                if (phase[n] == 1) {
-                    if (rule == CL_REACT_ALL_PORE_SOLID) react = phase[c] == 0;
-                    else if (rule == CL_REACT_IONOMER_SOLID) react = phase[c] == 2;
-                    else if (react_in) react = (react_in[c] >> d) & 1;
-                }
-                if (react) m |= (uint16_t)(1u << (kReactShift + d));
+                if (((given >> d) & 1u) && phase[n] == 1) m |= (uint16_t)(1u << (kReactShift + d));
             }
         }
-        mask[c] = m;
+        if (in) mask[c] = m;
     }
 }
 
 cudaError_t launch_masks(const uint8_t* phase, const uint8_t* active, const uint8_t* react_in, int rule,
                          int nx, int ny, int nz, uint16_t* mask, cudaStream_t s) {
-    k_masks<<<152 * 8, 256, 0, s>>>(phase, active, react_in, rule, nx, ny, nz, mask);
+    k_masks<<<152 * 16, 256, 0, s>>>(phase, active, react_in, rule, nx, ny, nz, mask);
     return cudaGetLastError();
 }
 
 // -------------------------------------------------------------------- stats
 constexpr int kStatN = 7;
-__global__ void k_stats(const uint8_t* __restrict__ phase, const uint16_t* __restrict__ mask,
+__global__ void __launch_bounds__(256) k_stats(const uint8_t* __restrict__ phase, const uint16_t* __restrict__ mask,
                         const double* __restrict__ D, const double* __restrict__ dp, long long N, int nx,
                         int tmask, double* partials) {
-    double v[kStatN] = {0, 0, 0, 0, 0, 0, 0};
-    double dmax = 0.0;
+    // whole numbers in integers, and the largest D as the bit pattern that orders positive doubles alike: FP64 is scarce
+    unsigned cnt[4] = {0, 0, 0, 0}, pores = 0;
+    long long top = 0;
+    double sum_dp = 0.0;
+    const unsigned unx = (unsigned)nx;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
          c += (long long)gridDim.x * blockDim.x) {
         const uint8_t ph = phase[c];
         const uint16_t m = mask[c];
-        v[0] += is_transport(ph, tmask) ? 1.0 : 0.0;
+        cnt[0] += is_transport(ph, tmask);
         if (m & kActiveBit) {
-            v[1] += 1.0;
-            const int x = (int)(c % nx);
+            cnt[1] += 1;
+            const unsigned x = (unsigned)c % unx;  // N < 2^31
             unsigned closed = m & 0x3fu;
-            if (x == 0) closed &= ~2u;       // -x face on the inlet plane
-            if (x == nx - 1) closed &= ~1u;  // +x face on the outlet plane
-            v[2] += __popc(closed);
-            v[3] += __popc((m >> kReactShift) & 0x3fu);
-            dmax = fmax(dmax, D[c]);
+            if (x == 0) closed &= ~2u;        // -x face on the inlet plane
+            if (x == unx - 1) closed &= ~1u;  // +x face on the outlet plane
+            cnt[2] += __popc(closed);
+            cnt[3] += __popc((m >> kReactShift) & 0x3fu);
+            const long long d = __double_as_longlong(D[c]);
+            top = d > top ? d : top;
         }
-        if (dp && is_pore(ph)) { v[4] += dp[c]; v[5] += 1.0; }
+        if (dp && is_pore(ph)) { sum_dp += dp[c]; pores += 1; }
     }
+    double dmax = __longlong_as_double(top);
+    double v[kStatN] = {(double)cnt[0], (double)cnt[1], (double)cnt[2], (double)cnt[3], sum_dp, (double)pores, 0.0};
     // sums for 0..5, max for 6 (max via the same tree with fmax)
     __shared__ double shm[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
