@@ -11,6 +11,7 @@
 #include "device_util.cuh"
 #include "handle.cuh"
 #include "dsa.cuh"
+#include "planes.cuh"
 
 using namespace cl;
 
@@ -434,6 +435,7 @@ cl_status do_init(cl_lbm* h, const float* C0dev) {
         CK(cudaStreamSynchronize(h->s));
         cmax = fmax(cmax, m);
     }
+    float2* ramp = C0dev ? nullptr : (float2*)h->d_plane;  // the linear field per plane, in the readout scratch
     if (h->march) {
         set_scales(h, cmax);
         drop_graphs(h);
@@ -443,7 +445,8 @@ cl_status do_init(cl_lbm* h, const float* C0dev) {
         CK(cudaMemsetAsync(o.clo, 0, (size_t)h->el * h->NP, h->s));
         for (int i = 0; i < 6; ++i) CK(cudaMemsetAsync(o.d[i], 0, (size_t)h->el * h->NP, h->s));
         MarchArgs a = make_margs(h, 0);
-        CK(launch_state_init(h->p.storage, a, h->mask_p, C0dev, h->s));
+        if (ramp) CK(launch_ramp(ramp, h->nx, a.c_in, a.c_out, h->s));
+        CK(launch_state_init(h->p.storage, a, h->mask_p, C0dev, ramp, h->s));
     } else if (h->q19s) {
         set_scales(h, cmax);
         drop_graphs(h);  // the scales are baked into captured kernel arguments
@@ -452,14 +455,16 @@ cl_status do_init(cl_lbm* h, const float* C0dev) {
         CK(cudaMemsetAsync(o.hl, 0, sizeof(float2) * (size_t)h->NP19, h->s));
         CK(cudaMemsetAsync(o.d, 0, (size_t)h->el * 18 * h->NP19, h->s));
         Q19Args a = make_args19(h);
-        CK(launch_init19s(h->p.storage, h->st19[0], a, C0dev, h->s));
+        if (ramp) CK(launch_ramp(ramp, h->nx, h->p.c_in, h->p.c_out, h->s));
+        CK(launch_init19s(h->p.storage, h->st19[0], a, C0dev, ramp, h->s));
     } else if (h->q == 19) {
         CK(cudaMemsetAsync(h->pop[1], 0, sizeof(float) * 19 * (size_t)h->NP19, h->s));
-        CK(launch_init19(h->pop[0], h->mask19, C0dev, h->nx, h->ny, h->nz, h->px19, h->p.c_in, h->p.c_out, h->Csnap,
-                         h->s));
+        if (ramp) CK(launch_ramp(ramp, h->nx, h->p.c_in, h->p.c_out, h->s));
+        CK(launch_init19(h->pop[0], h->mask19, C0dev, ramp, h->nx, h->ny, h->nz, h->px19, h->Csnap, h->s));
     } else {
         CK(cudaMemsetAsync(h->pop[1], 0, sizeof(float) * 7 * (size_t)h->N, h->s));
-        CK(launch_init_fp32(h->pop[0], h->mask, C0dev, h->nx, h->ny, h->nz, h->p.c_in, h->p.c_out, h->Csnap,
+        if (ramp) CK(launch_ramp(ramp, h->nx, h->p.c_in, h->p.c_out, h->s));
+        CK(launch_init_fp32(h->pop[0], h->mask, C0dev, ramp, h->nx, h->ny, h->nz, h->Csnap,
                             h->q == 7 ? h->src : nullptr, h->s));
     }
     h->step = 0;
@@ -649,7 +654,7 @@ cl_status cl_lbm_create(cl_handle* out, const cl_params* p) {
     if ((st = dalloc_n(h, &h->fbuf, N)) != CL_OK) return fail(st);
     if ((st = dalloc_n(h, &h->partials, npart)) != CL_OK) return fail(st);
     if ((st = dalloc_n(h, &h->d_red, 16)) != CL_OK) return fail(st);
-    if ((st = dalloc_n(h, &h->d_plane, 5LL * h->nx)) != CL_OK) return fail(st);
+    if ((st = dalloc_n(h, &h->d_plane, plane_doubles(h->nx, (long long)h->ny * h->nz))) != CL_OK) return fail(st);
     if (h->march) {
         for (int b = 0; b < 2; ++b) {
             if ((st = dalloc_n(h, &h->st[b].chi, h->NP)) != CL_OK) return fail(st);

@@ -94,7 +94,7 @@ struct cl_lbm {
     double* partials = nullptr;
     int nblk_step = 0, nblk_stats = 0;
     double* d_red = nullptr;    // [16]
-    double* d_plane = nullptr;  // [5 * nx]
+    double* d_plane = nullptr;  // [5 * nx] and the readouts' scratch behind it (planes.cuh)
     double* h_red = nullptr;    // pinned [16 + 5 * nx]
     bool have_react = false;
     bool have_structure = false;

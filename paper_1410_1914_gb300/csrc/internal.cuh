@@ -94,8 +94,8 @@ cudaError_t launch_masks19(const uint8_t* phase, const uint8_t* active, const ui
 cudaError_t launch_pad_omega19(const float* omega, int nx, int ny, int nz, int px, float* out, cudaStream_t s);
 cudaError_t launch_linkcount19(const uint32_t* mask, const uint32_t* react, long long NP, double* partials,
                                int nblocks, double* out, cudaStream_t s);
-cudaError_t launch_init19(float* pop, const uint32_t* mask, const float* C0, int nx, int ny, int nz, int px,
-                          double c_in, double c_out, float* Csnap, cudaStream_t s);
+cudaError_t launch_init19(float* pop, const uint32_t* mask, const float* C0, const float2* ramp, int nx, int ny, int nz,
+                          int px, float* Csnap, cudaStream_t s);
 int step19_blocks(const Q19Args& a);
 cudaError_t launch_step19(const float* src, float* dst, const Q19Args& a, bool reduce, cudaStream_t s);
 // the same step in FP64 on FP64 populations (no reduction)
@@ -106,7 +106,8 @@ cudaError_t launch_out19(const float* pop, const uint32_t* mask, int nx, int ny,
 int step19s_blocks(int px, int ny, int nz);
 cudaError_t launch_step19s(int storage, const Q19State& src, const Q19State& dst, const Q19Args& a, bool reduce,
                            cudaStream_t s);
-cudaError_t launch_init19s(int storage, const Q19State& st, const Q19Args& a, const float* C0, cudaStream_t s);
+cudaError_t launch_init19s(int storage, const Q19State& st, const Q19Args& a, const float* C0, const float2* ramp,
+                           cudaStream_t s);
 cudaError_t launch_readout19s(int storage, const Q19State& st, const Q19Args& a, double* out, cudaStream_t s);
 cudaError_t launch_out19s(int storage, const Q19State& st, const Q19Args& a, float* C, float* g, cudaStream_t s);
 cudaError_t launch_links_out(const uint32_t* mask19, const uint32_t* react19, const uint16_t* mask7, int nx, int ny,
@@ -138,8 +139,10 @@ cudaError_t launch_stats(const uint8_t* phase, const uint16_t* mask, const doubl
                          double* partials, int nblocks, double* out, cudaStream_t s);
 
 // ---- FP32 solver (kernels.cu) ----
-cudaError_t launch_init_fp32(float* pop, const uint16_t* mask, const float* C0, int nx, int ny,
-                             int nz, double c_in, double c_out, float* Csnap, const double* src, cudaStream_t s);
+// the linear field per plane (hi, lo), read by the initialisers when C0 is NULL
+cudaError_t launch_ramp(float2* ramp, int nx, double c_in, double c_out, cudaStream_t s);
+cudaError_t launch_init_fp32(float* pop, const uint16_t* mask, const float* C0, const float2* ramp, int nx, int ny,
+                             int nz, float* Csnap, const double* src, cudaStream_t s);
 cudaError_t launch_step_fp32(const float* src, float* dst, const StepArgs& a, bool reduce,
                              cudaStream_t s);
 // the same step in FP64 on FP64 populations (no reduction)
@@ -151,7 +154,7 @@ cudaError_t launch_finalize(const double* partials, int nblocks, int nslots, dou
                             cudaStream_t s);
 cudaError_t launch_field_fp32(const float* pop, const uint16_t* mask, long long N, float* C,
                               const double* src, cudaStream_t s);
-// per-plane readout: out[5*nx]: sumC, count, R, J_in part, J_out part
+// per-plane readout: out[5*nx]: sumC, count, R, J_in part, J_out part (and scratch behind it, planes.cuh)
 cudaError_t launch_readout_fp32(const float* pop, const StepArgs& a, double* out, cudaStream_t s);
 cudaError_t launch_cell_reaction_fp32(const float* pop, const StepArgs& a, double* out, cudaStream_t s);
 

@@ -7,6 +7,7 @@
 #include "internal.cuh"
 #include "ccl.cuh"
 #include "chords.cuh"
+#include "planes.cuh"
 
 namespace cl {
 
@@ -679,20 +680,30 @@ cudaError_t launch_finalize(const double* partials, int nblocks, int nslots, dou
 // Initial post-collision state: equilibrium w_i C0, plus the w_i S of a
 // per-cell source where one is set (the stored state is the post-collision
 // populations of the current step, source included).
+// The linear field between the half-way faces, per plane, as an unevaluated sum of two floats.  Its FP64 division
+// per plane instead of per cell: FP64 issues at 1/64 of the FP32 rate.
+__global__ void __launch_bounds__(256) k_ramp(float2* __restrict__ ramp, int nx, double c_in, double c_out) {
+    const int x = blockIdx.x * 256 + threadIdx.x;
+    if (x >= nx) return;
+    const double C = c_in + (c_out - c_in) * (x + 0.5) / nx;
+    const float hi = (float)C;
+    ramp[x] = make_float2(hi, (float)(C - (double)hi));
+}
+
+cudaError_t launch_ramp(float2* ramp, int nx, double c_in, double c_out, cudaStream_t s) {
+    k_ramp<<<(nx + 255) / 256, 256, 0, s>>>(ramp, nx, c_in, c_out);
+    return cudaGetLastError();
+}
+
 __global__ void k_init_fp32(float* __restrict__ pop, const uint16_t* __restrict__ mask,
-                            const float* __restrict__ C0, int nx, long long N, double c_in, double c_out,
+                            const float* __restrict__ C0, const float2* __restrict__ ramp, int nx, long long N,
                             float* __restrict__ Csnap, const double* __restrict__ src) {
+    const unsigned unx = (unsigned)nx;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
          c += (long long)gridDim.x * blockDim.x) {
         float C = 0.f;
         const bool act = (mask[c] & kActiveBit) != 0;
-        if (act) {
-            if (C0) C = C0[c];
-            else {
-                const int x = (int)(c % nx);
-                C = (float)(c_in + (c_out - c_in) * (x + 0.5) / nx);
-            }
-        }
+        if (act) C = C0 ? C0[c] : ramp[(unsigned)c % unx].x;  // N < 2^31
         const float S = (act && src) ? (float)src[c] : 0.f;
         pop[c] = act ? kW0 * (C + S) : 0.f;
 #pragma unroll
@@ -701,10 +712,10 @@ __global__ void k_init_fp32(float* __restrict__ pop, const uint16_t* __restrict_
     }
 }
 
-cudaError_t launch_init_fp32(float* pop, const uint16_t* mask, const float* C0, int nx, int ny, int nz,
-                             double c_in, double c_out, float* Csnap, const double* src, cudaStream_t s) {
+cudaError_t launch_init_fp32(float* pop, const uint16_t* mask, const float* C0, const float2* ramp, int nx, int ny,
+                             int nz, float* Csnap, const double* src, cudaStream_t s) {
     const long long N = (long long)nx * ny * nz;
-    k_init_fp32<<<152 * 8, 256, 0, s>>>(pop, mask, C0, nx, N, c_in, c_out, Csnap, src);
+    k_init_fp32<<<152 * 8, 256, 0, s>>>(pop, mask, C0, ramp, nx, N, Csnap, src);
     return cudaGetLastError();
 }
 
@@ -875,41 +886,59 @@ cudaError_t launch_field_fp32(const float* pop, const uint16_t* mask, long long 
     return cudaGetLastError();
 }
 
-// Per-plane readouts from the stored post-collision populations: one block
-// per x-plane, fixed-order sums.  out[5*x + k]: sum C, active count, R,
-// J_in part, J_out part.
-__global__ void k_readout_fp32(const float* __restrict__ pop, StepArgs a, double* out) {
-    const int x = blockIdx.x;
-    const long long N = a.N;
-    const long long nyz = (long long)a.ny * a.nz;
-    double v[5] = {0, 0, 0, 0, 0};
-    const double sink = a.rsink_d;
-    for (long long j = threadIdx.x; j < nyz; j += blockDim.x) {
-        const long long c = x + (long long)a.nx * j;
-        const uint16_t m = a.mask[c];
-        if (!(m & kActiveBit)) continue;
-        double C = 0.0;
+// Per-plane readouts from the stored post-collision populations (planes.cuh).
+struct PopPlaneOp {
+    static constexpr int kRows = 2;
+    const float* __restrict__ pop;
+    StepArgs a;
+    struct Item {
+        long long c;
+        uint16_t m;
         float h[7];
+    };
+    __device__ __forceinline__ double sink() const { return a.rsink_d; }
+    __device__ __forceinline__ Item load(int x, int row) const {
+        Item t;
+        t.c = x + (long long)a.nx * row;
+        t.m = a.mask[t.c];
 #pragma unroll
-        for (int i = 0; i < 7; ++i) { h[i] = pop[(long long)i * N + c]; }
-        C = (double)(((h[0] + h[1]) + (h[2] + h[3])) + ((h[4] + h[5]) + h[6]));
-        if (a.src) C -= a.src[c];  // the concentration before the last collision's source
-        v[0] += C;
-        v[1] += 1.0;
-        const unsigned rb = (m >> kReactShift) & 0x3fu;
-        double r = 0.0;
-        for (int d = 0; d < 6; ++d)
-            if (rb & (1u << d)) r += h[d + 1];
-        v[2] += (rb && a.kscale ? cell_sink(a.k_lu, a.kscale[c]) : sink) * r;
-        if (x == 0 && a.bc_in == CL_BC_DIRICHLET) v[3] += 2.0 * ((double)a.w_cin - (double)h[2]);
-        if (x == a.nx - 1 && a.bc_out == CL_BC_DIRICHLET) v[4] += 2.0 * ((double)h[1] - (double)a.w_cout);
+        for (int i = 0; i < 7; ++i) t.h[i] = pop[(long long)i * a.N + t.c];
+        return t;
     }
-    block_sum_store<5>(v, out + 5LL * x);
-}
+    __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
+        if (!(t.m & kActiveBit)) return;
+        const float* h = t.h;
+        const float C = ((h[0] + h[1]) + (h[2] + h[3])) + ((h[4] + h[5]) + h[6]);
+        if (a.src) acc.v[0] += (double)C - a.src[t.c];  // the concentration before the last collision's source
+        else acc.add_c(C, 0.f);
+        acc.n += 1;
+        const unsigned rb = (t.m >> kReactShift) & 0x3fu;
+        if (!rb) return;
+        if (a.kscale) {
+            double r = 0.0;
+            for (int d = 0; d < 6; ++d)
+                if (rb & (1u << d)) r += t.h[d + 1];
+            acc.v[2] += cell_sink(a.k_lu, a.kscale[t.c]) * r;
+        } else {
+#pragma unroll
+            for (int d = 0; d < 6; ++d)
+                if (rb & (1u << d)) acc.add_r(t.h[d + 1], 0.f);
+        }
+    }
+    __device__ __forceinline__ double inflow(int row) const {
+        const long long c = (long long)a.nx * row;
+        if (!(a.mask[c] & kActiveBit) || a.bc_in != CL_BC_DIRICHLET) return 0.0;
+        return 2.0 * ((double)a.w_cin - (double)pop[2 * a.N + c]);
+    }
+    __device__ __forceinline__ double outflow(int row) const {
+        const long long c = a.nx - 1 + (long long)a.nx * row;
+        if (!(a.mask[c] & kActiveBit) || a.bc_out != CL_BC_DIRICHLET) return 0.0;
+        return 2.0 * ((double)pop[a.N + c] - (double)a.w_cout);
+    }
+};
 
 cudaError_t launch_readout_fp32(const float* pop, const StepArgs& a, double* out, cudaStream_t s) {
-    k_readout_fp32<<<a.nx, 256, 0, s>>>(pop, a, out);
-    return cudaGetLastError();
+    return launch_planes(PopPlaneOp{pop, a}, a.nx, (long long)a.ny * a.nz, out, s);
 }
 
 // Per-cell amount consumed per step on the catalytic links, from the stored

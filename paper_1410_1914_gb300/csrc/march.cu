@@ -33,6 +33,7 @@
 #include "device_util.cuh"
 #include "internal.cuh"
 #include "march.cuh"
+#include "planes.cuh"
 
 namespace cl {
 
@@ -119,6 +120,14 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
     const float bb = s - a;
     e = (a - (s - bb)) + (b - bb);
+}
+
+// p += hi + lo, p.y keeping what the additions to p.x lose
+__device__ __forceinline__ void pair_add(float2& p, float hi, float lo) {
+    const float t = __fadd_rn(p.x, hi);
+    const float z = __fsub_rn(t, p.x);
+    p.y = __fadd_rn(p.y, __fadd_rn(__fadd_rn(__fsub_rn(p.x, __fsub_rn(t, z)), __fsub_rn(hi, z)), lo));
+    p.x = t;
 }
 
 // (hi, lo) + d, renormalised
@@ -223,7 +232,7 @@ template <class S, bool REDUCE>
 __device__ __forceinline__ void cell_update(const MarchArgs& a, uint32_t m, float om, float hx, float lxs,
                                             const float (&dds)[6], const float (&nh)[6], const float (&nls)[6],
                                             const float (&nds)[6], int x, float& hnew, float& lnew_s,
-                                            float (&dns)[6], double (&rv)[RED_N], float (&rs)[4], float csnap,
+                                            float (&dns)[6], float2 (&rp)[3], float (&rs)[4], float csnap,
                                             float& csnap_out) {
     constexpr bool HALF = sizeof(typename S::T) == 2;
     const float inv_lo = HALF ? a.inv_lo : 1.0f, s_lo = HALF ? a.s_lo : 1.0f;
@@ -259,25 +268,30 @@ __device__ __forceinline__ void cell_update(const MarchArgs& a, uint32_t m, floa
 #pragma unroll
     for (int i = 0; i < 6; ++i) dns[i] = fmaf(om1, av[i], -t);  // (1 - omega)(a_i - w dC)
     if (REDUCE) {
-        // Fluxes and reaction in FP64 (boundary and catalytic cells only:
-        // the stopping rule resolves their changes down to 1e-9); the
-        // per-cell diagnostics in per-thread FP32 partials that the block
-        // sums in FP64 (GB300's FP64 rate is a small fraction of FP32)
-        const double id = inv_d;
-        if (x == 0 && a.bc_in == CL_BC_DIRICHLET)
-            rv[RED_JIN] += 2.0 * (double)w * ((double)a.c_in - ((double)hnew + (double)lnew)) -
-                           2.0 * (double)dns[1] * id;
-        if (x == a.nx - 1 && a.bc_out == CL_BC_DIRICHLET)
-            rv[RED_JOUT] += 2.0 * (double)w * (((double)hnew + (double)lnew) - (double)a.c_out) +
-                            2.0 * (double)dns[0] * id;
+        // Fluxes and reaction (boundary and catalytic cells only: the stopping rule resolves their changes
+        // down to 1e-9) in pairs of floats with the rounding errors kept, summed in FP64 by the block; the
+        // per-cell diagnostics in per-thread FP32 partials.  In FP64 these conditions were predicated off in
+        // most lanes but issued in every one, at 1/64 of the FP32 rate: the reducing step took 0.40 ms at
+        // 256^3 and 2.7 ms on the 400^3 NPMC layer, against 0.12 and 0.44 ms of a plain one.
+        float s, e;
+        if (x == 0 && a.bc_in == CL_BC_DIRICHLET) {
+            two_sum(a.c_in, -hnew, s, e);
+            pair_add(rp[0], 2.0f * w * s, 2.0f * w * (e - lnew));
+            pair_add(rp[0], -2.0f * dns[1] * inv_d, 0.f);
+        }
+        if (x == a.nx - 1 && a.bc_out == CL_BC_DIRICHLET) {
+            two_sum(hnew, -a.c_out, s, e);
+            pair_add(rp[1], 2.0f * w * s, 2.0f * w * (e + lnew));
+            pair_add(rp[1], 2.0f * dns[0] * inv_d, 0.f);
+        }
         const unsigned rb = (m >> kReactShift) & 0x3fu;
         if (rb) {
-            const double Cn = (double)hnew + (double)lnew;
-            double r = 0.0;
 #pragma unroll
             for (int d = 0; d < 6; ++d)
-                if (rb & (1u << d)) r += (double)w * Cn + (double)dns[d] * id;
-            rv[RED_R] += a.rsink_d * r;
+                if (rb & (1u << d)) {  // w C + delta, the weight a power of two
+                    pair_add(rp[2], w * hnew, w * lnew);
+                    pair_add(rp[2], dns[d] * inv_d, 0.f);
+                }
         }
         const float Cf = hnew + lnew;  // the f32 rounding of the double-float C
         rs[0] += Cf;
@@ -400,6 +414,9 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
     }
     // ---------------------------------------------------------- consumers
     float rs[4] = {0.f, 0.f, 0.f, 0.f};  // FP32 partials of sum C, sum |dC|, sum |C|, non-finite
+    float2 rp[3];                        // J_in, J_out, and R before the sink's factor
+#pragma unroll
+    for (int i = 0; i < 3; ++i) rp[i] = make_float2(0.f, 0.f);
     const int xl = tx & (LPR - 1);        // lane within its tile row
     const int row = ty * RW + tx / LPR;   // tile row of this lane
     const int xa = x0 + 2 * xl;  // this lane's cells: xa, xa + 1
@@ -506,16 +523,16 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
             if (REDUCE) {
                 // the reductions must see active cells only
                 if (act_a)
-                    cell_update<S, true>(a, ma, om.x, hx.x, lx.x, dda, nha, nla, nda, xa, hA, lA, dA, rv, rs, cs.x, cso.x);
+                    cell_update<S, true>(a, ma, om.x, hx.x, lx.x, dda, nha, nla, nda, xa, hA, lA, dA, rp, rs, cs.x, cso.x);
                 if (act_b)
-                    cell_update<S, true>(a, mb, om.y, hx.y, lx.y, ddb, nhb, nlb, ndb, xa + 1, hB, lB, dB, rv, rs, cs.y,
+                    cell_update<S, true>(a, mb, om.y, hx.y, lx.y, ddb, nhb, nlb, ndb, xa + 1, hB, lB, dB, rp, rs, cs.y,
                                          cso.y);
             } else {
                 // both cells of the pair without a branch; an inactive cell's
                 // result (finite: its neighbours and omega slots hold zeros or
                 // state values) is replaced by the zeros it keeps
-                cell_update<S, false>(a, ma, om.x, hx.x, lx.x, dda, nha, nla, nda, xa, hA, lA, dA, rv, rs, cs.x, cso.x);
-                cell_update<S, false>(a, mb, om.y, hx.y, lx.y, ddb, nhb, nlb, ndb, xa + 1, hB, lB, dB, rv, rs, cs.y,
+                cell_update<S, false>(a, ma, om.x, hx.x, lx.x, dda, nha, nla, nda, xa, hA, lA, dA, rp, rs, cs.x, cso.x);
+                cell_update<S, false>(a, mb, om.y, hx.y, lx.y, ddb, nhb, nlb, ndb, xa + 1, hB, lB, dB, rp, rs, cs.y,
                                       cso.y);
                 if (!act_a) {
                     hA = 0.f; lA = 0.f;
@@ -562,6 +579,9 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
     }
     if (ok) release(nplanes - 1);  // plane ze, read only as a z+1 neighbour
     if (REDUCE) {
+        rv[RED_JIN] += (double)rp[0].x + (double)rp[0].y;
+        rv[RED_JOUT] += (double)rp[1].x + (double)rp[1].y;
+        rv[RED_R] += a.rsink_d * ((double)rp[2].x + (double)rp[2].y);
         rv[RED_SUMC] += (double)rs[0];
         rv[RED_DC] += (double)rs[1];
         rv[RED_ABSC] += (double)rs[2];
@@ -909,30 +929,60 @@ int march_blocks_per_sm(int storage, int rw) {
 // Stored row yr in [0, ny+2) -> actual row (ghost rows wrap).
 __device__ __forceinline__ int actual_row(int yr, int ny) { return yr == 0 ? ny - 1 : (yr == ny + 1 ? 0 : yr - 1); }
 
+// Eight cells of a row per thread, whole 16-byte words throughout (the pitch is
+// a multiple of 16 cells): one store per array and thread instead of one per
+// cell, and the ramp's FP64 arithmetic once per plane (k_ramp) instead of once
+// per cell (0.50 ms at 256^3 that way, now 0.1 ms).
 template <class S>
-__global__ void k_state_init(MarchArgs a, const uint16_t* __restrict__ mask_p, const float* __restrict__ C0) {
+__global__ void __launch_bounds__(256) k_state_init(MarchArgs a, const uint16_t* __restrict__ mask_p,
+                                                    const float* __restrict__ C0, const float2* __restrict__ ramp) {
     using T = typename S::T;
-    const long long pstride = (long long)a.px * (a.ny + 2);
-    const long long total = pstride * a.nz;
-    for (long long gi = blockIdx.x * (long long)blockDim.x + threadIdx.x; gi < total;
-         gi += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(gi % a.px);
-        const int yr = (int)((gi / a.px) % (a.ny + 2));
-        const int z = (int)(gi / pstride);
-        const int y = actual_row(yr, a.ny);
-        const long long gm = x + (long long)a.px * (y + 1) + pstride * z;  // owner's slot
-        float hi = 0.f, lo = 0.f;
-        if (x < a.nx && (mask_p[gm] & kActiveBit)) {
-            double C;
-            if (C0) C = C0[x + (long long)a.nx * (y + (long long)a.ny * z)];
-            else C = (double)a.c_in + ((double)a.c_out - (double)a.c_in) * (x + 0.5) / a.nx;
-            hi = (float)C;
-            lo = (float)(C - (double)hi);
+    const unsigned px8 = (unsigned)a.px / 8, rpp = (unsigned)a.ny + 2;
+    const unsigned long long groups = (unsigned long long)px8 * rpp * a.nz;
+    for (unsigned long long q = blockIdx.x * 256ull + threadIdx.x; q < groups; q += gridDim.x * 256ull) {
+        const unsigned row = (unsigned)(q / px8), x0 = (unsigned)(q - (unsigned long long)row * px8) * 8;
+        const unsigned z = row / rpp;
+        const int y = actual_row((int)(row - z * rpp), a.ny);
+        const long long gm = x0 + (long long)a.px * (y + 1 + (long long)rpp * z);  // owner's slot
+        const long long gi = x0 + (long long)a.px * row;
+        alignas(16) uint16_t m[8];
+        *reinterpret_cast<uint4*>(m) = *reinterpret_cast<const uint4*>(mask_p + gm);
+        alignas(16) float hi[8], cs[8];
+        alignas(16) T lo[8], zero[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int x = (int)x0 + k;
+            float h = 0.f, l = 0.f;
+            if (x < a.nx && (m[k] & kActiveBit)) {
+                if (C0) {
+                    h = C0[x + (long long)a.nx * (y + (long long)a.ny * z)];
+                } else {
+                    const float2 r = ramp[x];
+                    h = r.x;
+                    l = r.y;
+                }
+            }
+            hi[k] = h;
+            lo[k] = S::st(l, a.s_lo);
+            zero[k] = S::st(0.f, a.s_d);
+            cs[k] = h + l;
         }
-        a.chi[gi] = hi;
-        reinterpret_cast<T*>(a.clo)[gi] = S::st(lo, a.s_lo);
-        for (int i = 0; i < 6; ++i) reinterpret_cast<T*>(a.d[i])[gi] = S::st(0.f, a.s_d);
-        if (a.Csnap) a.Csnap[gi] = hi + lo;
+        constexpr int W = 8 * sizeof(T) / 16;  // words of eight stored values
+        auto put = [&](void* p, const void* v, int words) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if (k < words) reinterpret_cast<uint4*>(p)[k] = reinterpret_cast<const uint4*>(v)[k];
+        };
+        put(a.chi + gi, hi, 2);
+        put(reinterpret_cast<T*>(a.clo) + gi, lo, W);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) put(reinterpret_cast<T*>(a.d[i]) + gi, zero, W);
+        if (a.Csnap && (reinterpret_cast<uintptr_t>(a.Csnap) & 15) == 0) {
+            put(a.Csnap + gi, cs, 2);
+        } else if (a.Csnap) {  // the one array here that no TMA descriptor has checked
+#pragma unroll
+            for (int k = 0; k < 8; ++k) a.Csnap[gi + k] = cs[k];
+        }
     }
 }
 
@@ -962,40 +1012,69 @@ __global__ void k_state_out(MarchArgs a, const uint16_t* __restrict__ mask_p, fl
     }
 }
 
-// per-plane readouts (one block per x-plane): sum C, count, R, J_in part, J_out part
+// per-plane readouts (planes.cuh)
 template <class S>
-__global__ void k_state_readout(MarchArgs a, const uint16_t* __restrict__ mask_p, double* out) {
+struct StatePlaneOp {
     using T = typename S::T;
-    const int x = blockIdx.x;
-    const long long nyz = (long long)a.ny * a.nz;
-    const long long pstride = (long long)a.px * (a.ny + 2);
-    const double w = kW1;
-    double v[5] = {0, 0, 0, 0, 0};
-    for (long long j = threadIdx.x; j < nyz; j += blockDim.x) {
-        const int y = (int)(j % a.ny), z = (int)(j / a.ny);
-        const long long gi = x + (long long)a.px * (y + 1) + pstride * z;
-        const uint16_t m = mask_p[gi];
-        if (!(m & kActiveBit)) continue;
-        const double C = (double)a.chi[gi] + (double)S::ld(reinterpret_cast<const T*>(a.clo)[gi], a.inv_lo);
-        double d[6];
-        for (int i = 0; i < 6; ++i) d[i] = S::ld(reinterpret_cast<const T*>(a.d[i])[gi], a.inv_d);
-        v[0] += C;
-        v[1] += 1.0;
-        const unsigned rb = (m >> kReactShift) & 0x3fu;
-        double r = 0.0;
-        for (int dd = 0; dd < 6; ++dd)
-            if (rb & (1u << dd)) r += w * C + d[dd];
-        v[2] += a.rsink_d * r;
-        if (x == 0 && a.bc_in == CL_BC_DIRICHLET) v[3] += 2.0 * w * ((double)a.c_in - C) - 2.0 * d[1];
-        if (x == a.nx - 1 && a.bc_out == CL_BC_DIRICHLET) v[4] += 2.0 * w * (C - (double)a.c_out) + 2.0 * d[0];
+    static constexpr int kRows = 4;
+    MarchArgs a;
+    const uint16_t* __restrict__ mask_p;
+    struct Item {
+        long long gi;
+        uint16_t m;
+        float hi, lo;
+    };
+    __device__ __forceinline__ long long at(int x, int row) const {
+        const int z = row / a.ny, y = row - z * a.ny;
+        return x + (long long)a.px * (y + 1 + (long long)(a.ny + 2) * z);
     }
-    block_sum_store<5>(v, out + 5LL * x);
-}
+    __device__ __forceinline__ float d(int i, long long gi) const {
+        return S::ld(reinterpret_cast<const T*>(a.d[i])[gi], a.inv_d);
+    }
+    __device__ __forceinline__ double sink() const { return a.rsink_d; }
+    __device__ __forceinline__ Item load(int x, int row) const {
+        Item t;
+        t.gi = at(x, row);
+        t.m = mask_p[t.gi];
+        t.hi = a.chi[t.gi];
+        t.lo = S::ld(reinterpret_cast<const T*>(a.clo)[t.gi], a.inv_lo);
+        return t;
+    }
+    __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
+        if (!(t.m & kActiveBit)) return;
+        acc.add_c(t.hi, t.lo);
+        acc.n += 1;
+        const unsigned rb = (t.m >> kReactShift) & 0x3fu;
+        if (rb) {
+            float dv[6];  // all six in flight together
+#pragma unroll
+            for (int i = 0; i < 6; ++i) dv[i] = d(i, t.gi);
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+                if (rb & (1u << i)) {  // w C + d: the weight is a power of two
+                    acc.add_r(kW1 * t.hi, kW1 * t.lo);
+                    acc.add_r(dv[i], 0.f);
+                }
+        }
+    }
+    __device__ __forceinline__ double inflow(int row) const {
+        const Item t = load(0, row);
+        if (!(t.m & kActiveBit) || a.bc_in != CL_BC_DIRICHLET) return 0.0;
+        return 2.0 * (double)kW1 * ((double)a.c_in - ((double)t.hi + (double)t.lo)) - 2.0 * (double)d(1, t.gi);
+    }
+    __device__ __forceinline__ double outflow(int row) const {
+        const Item t = load(a.nx - 1, row);
+        if (!(t.m & kActiveBit) || a.bc_out != CL_BC_DIRICHLET) return 0.0;
+        return 2.0 * (double)kW1 * (((double)t.hi + (double)t.lo) - (double)a.c_out) + 2.0 * (double)d(0, t.gi);
+    }
+};
 
 cudaError_t launch_state_init(int storage, const MarchArgs& a, const uint16_t* mask_p, const float* C0,
-                              cudaStream_t s) {
-    if (storage == CL_STORE_FP16DEV) k_state_init<StoreF16><<<152 * 8, 256, 0, s>>>(a, mask_p, C0);
-    else k_state_init<StoreF32><<<152 * 8, 256, 0, s>>>(a, mask_p, C0);
+                              const float2* ramp, cudaStream_t s) {
+    const long long groups = (long long)a.px / 8 * (a.ny + 2) * a.nz;
+    const int g = (int)((groups + 255) / 256 < 152 * 16 ? (groups + 255) / 256 : 152 * 16);
+    if (storage == CL_STORE_FP16DEV) k_state_init<StoreF16><<<g, 256, 0, s>>>(a, mask_p, C0, ramp);
+    else k_state_init<StoreF32><<<g, 256, 0, s>>>(a, mask_p, C0, ramp);
     return cudaGetLastError();
 }
 
@@ -1008,9 +1087,9 @@ cudaError_t launch_state_out(int storage, const MarchArgs& a, const uint16_t* ma
 
 cudaError_t launch_state_readout(int storage, const MarchArgs& a, const uint16_t* mask_p, double* out,
                                  cudaStream_t s) {
-    if (storage == CL_STORE_FP16DEV) k_state_readout<StoreF16><<<a.nx, 256, 0, s>>>(a, mask_p, out);
-    else k_state_readout<StoreF32><<<a.nx, 256, 0, s>>>(a, mask_p, out);
-    return cudaGetLastError();
+    const long long rows = (long long)a.ny * a.nz;
+    if (storage == CL_STORE_FP16DEV) return launch_planes(StatePlaneOp<StoreF16>{a, mask_p}, a.nx, rows, out, s);
+    return launch_planes(StatePlaneOp<StoreF32>{a, mask_p}, a.nx, rows, out, s);
 }
 
 // unpadded -> padded (ghosted) copy of the static per-cell arrays

@@ -92,10 +92,12 @@ double march_tile_cost(int nx, int ny, int storage, int rw);
 int march_auto_rows(int nx, int ny, int storage);
 cudaError_t launch_march(int storage, bool reduce, int rw, const MarchMaps& maps, const MarchArgs& a, dim3 grid,
                          cudaStream_t s);
+// ramp: the linear field per plane (launch_ramp), read when C0 is NULL
 cudaError_t launch_state_init(int storage, const MarchArgs& a, const uint16_t* mask_p, const float* C0,
-                              cudaStream_t s);
+                              const float2* ramp, cudaStream_t s);
 cudaError_t launch_state_out(int storage, const MarchArgs& a, const uint16_t* mask_p, float* C, float* g,
                              cudaStream_t s);
+// out: plane_doubles(nx, ny nz) doubles, the first 5 nx of them the result
 cudaError_t launch_state_readout(int storage, const MarchArgs& a, const uint16_t* mask_p, double* out,
                                  cudaStream_t s);
 cudaError_t launch_pad_static(const uint16_t* mask, const float* omega, int nx, int ny, int nz, int px,

@@ -25,6 +25,7 @@
 
 #include "device_util.cuh"
 #include "internal.cuh"
+#include "planes.cuh"
 
 namespace cl {
 
@@ -152,23 +153,23 @@ cudaError_t launch_linkcount19(const uint32_t* mask, const uint32_t* react, long
 // Equilibrium a_i C (Eq. 23) from C0 (unpadded, nullable: the linear ramp
 // between the half-way faces); Csnap (padded) gets C.
 __global__ void k_init19(float* __restrict__ pop, const uint32_t* __restrict__ mask, const float* __restrict__ C0,
-                         int nx, int ny, int nz, int px, double c_in, double c_out, float* __restrict__ Csnap) {
+                         const float2* __restrict__ ramp, int nx, int ny, int nz, int px, float* __restrict__ Csnap) {
     const long long NP = (long long)px * ny * nz;
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < NP;
          p += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(p % px);
         const bool act = (mask[p] & kQ19Active) != 0;
         float C = 0.f;
-        if (act) C = C0 ? C0[x + (long long)nx * (p / px)] : (float)(c_in + (c_out - c_in) * (x + 0.5) / nx);
+        if (act) C = C0 ? C0[x + (long long)nx * (p / px)] : ramp[x].x;
 #pragma unroll
         for (int i = 0; i < 19; ++i) pop[(long long)i * NP + p] = act ? q19_w(i) * C : 0.f;
         Csnap[p] = C;
     }
 }
 
-cudaError_t launch_init19(float* pop, const uint32_t* mask, const float* C0, int nx, int ny, int nz, int px,
-                          double c_in, double c_out, float* Csnap, cudaStream_t s) {
-    k_init19<<<152 * 8, 256, 0, s>>>(pop, mask, C0, nx, ny, nz, px, c_in, c_out, Csnap);
+cudaError_t launch_init19(float* pop, const uint32_t* mask, const float* C0, const float2* ramp, int nx, int ny, int nz,
+                          int px, float* Csnap, cudaStream_t s) {
+    k_init19<<<152 * 8, 256, 0, s>>>(pop, mask, C0, ramp, nx, ny, nz, px, Csnap);
     return cudaGetLastError();
 }
 
@@ -313,42 +314,60 @@ cudaError_t launch_step19_f64(const double* src, double* dst, const Q19Args& a, 
 }
 
 // --------------------------------------------------------------- readouts
-// Per x-plane from the stored post-collision populations, one block per
-// plane: out[5*x + k] = sum C, active count, R, J_in part, J_out part.
-__global__ void k_readout19(const float* __restrict__ pop, Q19Args a, double* out) {
-    const int x = blockIdx.x;
-    const long long nyz = (long long)a.ny * a.nz;
-    double v[5] = {0, 0, 0, 0, 0};
-    const double sink = a.rsink_d;
-    for (long long j = threadIdx.x; j < nyz; j += blockDim.x) {
-        const long long c = x + (long long)a.px * j;
-        const uint32_t m = a.mask[c];
-        if (!(m & kQ19Active)) continue;
-        const uint32_t rb = (m & kQ19HasReact) ? a.react[c] : 0u;
+// Per x-plane from the stored post-collision populations (planes.cuh).
+struct Pop19PlaneOp {
+    static constexpr int kRows = 1;
+    const float* __restrict__ pop;
+    Q19Args a;
+    struct Item {
+        long long c;
+        uint32_t m;
         float h[19];
-        double C = 0.0;
+    };
+    __device__ __forceinline__ double sink() const { return a.rsink_d; }
+    __device__ __forceinline__ Item load(int x, int row) const {
+        Item t;
+        t.c = x + (long long)a.px * row;
+        t.m = a.mask[t.c];
 #pragma unroll
-        for (int i = 0; i < 19; ++i) { h[i] = pop[(long long)i * a.NP + c]; C += (double)h[i]; }
-        v[0] += C;
-        v[1] += 1.0;
-        double r = 0.0;
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            const bool wall = (m >> (i - 1)) & 1u;
-            if (rb & (1u << (i - 1))) r += h[i];
-            if (q19_cx(i) < 0 && x == 0 && !wall && a.bc_in == CL_BC_DIRICHLET)
-                v[3] += 2.0 * ((double)q19_w(i) * a.c_in_d - (double)h[i]);
-            if (q19_cx(i) > 0 && x == a.nx - 1 && !wall && a.bc_out == CL_BC_DIRICHLET)
-                v[4] += 2.0 * ((double)h[i] - (double)q19_w(i) * a.c_out_d);
-        }
-        v[2] += sink * r;
+        for (int i = 0; i < 19; ++i) t.h[i] = pop[(long long)i * a.NP + t.c];
+        return t;
     }
-    block_sum_store<5>(v, out + 5LL * x);
-}
+    __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
+        if (!(t.m & kQ19Active)) return;
+#pragma unroll
+        for (int i = 0; i < 19; ++i) acc.add_c(t.h[i], 0.f);
+        acc.n += 1;
+        if (!(t.m & kQ19HasReact)) return;
+        const uint32_t rb = a.react[t.c];
+#pragma unroll
+        for (int i = 1; i < 19; ++i)
+            if (rb & (1u << (i - 1))) acc.add_r(t.h[i], 0.f);
+    }
+    __device__ __forceinline__ double inflow(int row) const {
+        const long long c = (long long)a.px * row;
+        const uint32_t m = a.mask[c];
+        double s = 0.0;
+        if (!(m & kQ19Active) || a.bc_in != CL_BC_DIRICHLET) return s;
+        for (int i = 1; i < 19; ++i)
+            if (q19_cx(i) < 0 && !((m >> (i - 1)) & 1u))
+                s += 2.0 * ((double)q19_w(i) * a.c_in_d - (double)pop[(long long)i * a.NP + c]);
+        return s;
+    }
+    __device__ __forceinline__ double outflow(int row) const {
+        const long long c = a.nx - 1 + (long long)a.px * row;
+        const uint32_t m = a.mask[c];
+        double s = 0.0;
+        if (!(m & kQ19Active) || a.bc_out != CL_BC_DIRICHLET) return s;
+        for (int i = 1; i < 19; ++i)
+            if (q19_cx(i) > 0 && !((m >> (i - 1)) & 1u))
+                s += 2.0 * ((double)pop[(long long)i * a.NP + c] - (double)q19_w(i) * a.c_out_d);
+        return s;
+    }
+};
 
 cudaError_t launch_readout19(const float* pop, const Q19Args& a, double* out, cudaStream_t s) {
-    k_readout19<<<a.nx, 256, 0, s>>>(pop, a, out);
-    return cudaGetLastError();
+    return launch_planes(Pop19PlaneOp{pop, a}, a.nx, (long long)a.ny * a.nz, out, s);
 }
 
 // C (unpadded, 0 on inactive cells) and/or the populations as [19][nz][ny][nx]

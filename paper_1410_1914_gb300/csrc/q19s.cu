@@ -25,6 +25,7 @@
 
 #include "device_util.cuh"
 #include "internal.cuh"
+#include "planes.cuh"
 
 namespace cl {
 
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(kS19X * kS19Y) k_step19s(Q19State src, Q19Stat
 // ----------------------------------------------------------- init / readout
 // C0 (unpadded, nullable: the linear ramp) into (hi, lo), deviations 0.
 template <class S>
-__global__ void k_init19s(Q19State st, Q19Args a, const float* __restrict__ C0) {
+__global__ void k_init19s(Q19State st, Q19Args a, const float* __restrict__ C0, const float2* __restrict__ ramp) {
     using T = typename S::T;
     const long long NP = a.NP;
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < NP;
@@ -205,10 +206,12 @@ __global__ void k_init19s(Q19State st, Q19Args a, const float* __restrict__ C0) 
         const int x = (int)(p % a.px);
         float hi = 0.f, lo = 0.f;
         if (a.mask[p] & kQ19Active) {
-            const double C = C0 ? (double)C0[x + (long long)a.nx * (p / a.px)]
-                                : a.c_in_d + (a.c_out_d - a.c_in_d) * (x + 0.5) / a.nx;
-            hi = (float)C;
-            lo = (float)(C - (double)hi);
+            if (C0) {
+                hi = C0[x + (long long)a.nx * (p / a.px)];
+            } else {
+                hi = ramp[x].x;
+                lo = ramp[x].y;
+            }
         }
         st.hl[p] = make_float2(hi, lo);
         for (int i = 0; i < 18; ++i) reinterpret_cast<T*>(st.d)[i * NP + p] = S::st(0.f);
@@ -232,38 +235,59 @@ __device__ __forceinline__ double state_cell(const Q19State& st, const Q19Args& 
     return C;
 }
 
-// per x-plane: out[5*x + k] = sum C, active count, R, J_in part, J_out part
+// per x-plane (planes.cuh): the deviations are read only where a catalytic or boundary link needs them
 template <class S>
-__global__ void k_readout19s(Q19State st, Q19Args a, double* out) {
-    const int x = blockIdx.x;
-    const long long nyz = (long long)a.ny * a.nz;
-    double v[5] = {0, 0, 0, 0, 0};
-    const double sink = a.rsink_d;
-    for (long long j = threadIdx.x; j < nyz; j += blockDim.x) {
-        const long long p = x + (long long)a.px * j;
-        const uint32_t m = a.mask[p];
-        if (!(m & kQ19Active)) continue;
-        const uint32_t rb = (m & kQ19HasReact) ? a.react[p] : 0u;
-        float g[19];
-        const double C = state_cell<S>(st, a, p, g);
-        v[0] += C;
-        v[1] += 1.0;
-        double r = 0.0;
-        for (int i = 1; i < 19; ++i) {
-            const bool wall = (m >> (i - 1)) & 1u;
-            const double gs = (double)s19_w(i) * C +
-                              (double)S::ld(reinterpret_cast<const typename S::T*>(st.d)[(i - 1) * a.NP + p]) *
-                                  (sizeof(typename S::T) == 2 ? (double)a.inv_d : 1.0);
-            if (rb & (1u << (i - 1))) r += gs;
-            if (s19_cx(i) < 0 && x == 0 && !wall && a.bc_in == CL_BC_DIRICHLET)
-                v[3] += 2.0 * ((double)s19_w(i) * a.c_in_d - gs);
-            if (s19_cx(i) > 0 && x == a.nx - 1 && !wall && a.bc_out == CL_BC_DIRICHLET)
-                v[4] += 2.0 * (gs - (double)s19_w(i) * a.c_out_d);
-        }
-        v[2] += sink * r;
+struct State19PlaneOp {
+    using T = typename S::T;
+    static constexpr int kRows = 4;
+    Q19State st;
+    Q19Args a;
+    struct Item {
+        long long p;
+        uint32_t m;
+        float2 hl;
+    };
+    __device__ __forceinline__ double sink() const { return a.rsink_d; }
+    __device__ __forceinline__ float d(int i, long long p) const {
+        return S::ld(reinterpret_cast<const T*>(st.d)[(i - 1) * a.NP + p]) * (sizeof(T) == 2 ? a.inv_d : 1.f);
     }
-    block_sum_store<5>(v, out + 5LL * x);
-}
+    __device__ __forceinline__ Item load(int x, int row) const {
+        Item t;
+        t.p = x + (long long)a.px * row;
+        t.m = a.mask[t.p];
+        t.hl = st.hl[t.p];
+        return t;
+    }
+    __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
+        if (!(t.m & kQ19Active)) return;
+        acc.add_c(t.hl.x, t.hl.y);
+        acc.n += 1;
+        if (!(t.m & kQ19HasReact)) return;
+        for (unsigned left = a.react[t.p]; left; left &= left - 1) {  // g*_i = a_i C + d_i of the catalytic links
+            const int i = __ffs(left);
+            const float w = s19_w(i), h = w * t.hl.x;
+            acc.add_r(h, fmaf(w, t.hl.x, -h) + w * t.hl.y);
+            acc.add_r(d(i, t.p), 0.f);
+        }
+    }
+    // 2 (a_i C_bc - g*_i) over the open links through the plane (sgn -1: x = 0, which take in; +1: x = L)
+    __device__ __forceinline__ double through(int x, int row, int sgn, double c_bc) const {
+        const Item t = load(x, row);
+        double s = 0.0;
+        if (!(t.m & kQ19Active)) return s;
+        const double C = (double)t.hl.x + (double)t.hl.y;
+        for (int i = 1; i < 19; ++i)
+            if (s19_cx(i) == sgn && !((t.m >> (i - 1)) & 1u))
+                s += 2.0 * ((double)s19_w(i) * c_bc - ((double)s19_w(i) * C + (double)d(i, t.p)));
+        return s;
+    }
+    __device__ __forceinline__ double inflow(int row) const {
+        return a.bc_in == CL_BC_DIRICHLET ? through(0, row, -1, a.c_in_d) : 0.0;
+    }
+    __device__ __forceinline__ double outflow(int row) const {
+        return a.bc_out == CL_BC_DIRICHLET ? -through(a.nx - 1, row, 1, a.c_out_d) : 0.0;
+    }
+};
 
 // unpadded C and/or g* as [19][nz][ny][nx]
 template <class S>
@@ -306,16 +330,17 @@ int step19s_blocks(int px, int ny, int nz) {
     return ((px + kS19X - 1) / kS19X) * ((ny + kS19Y - 1) / kS19Y) * nz;
 }
 
-cudaError_t launch_init19s(int storage, const Q19State& st, const Q19Args& a, const float* C0, cudaStream_t s) {
-    if (storage == CL_STORE_FP16DEV) k_init19s<SF16><<<152 * 8, 256, 0, s>>>(st, a, C0);
-    else k_init19s<SF32><<<152 * 8, 256, 0, s>>>(st, a, C0);
+cudaError_t launch_init19s(int storage, const Q19State& st, const Q19Args& a, const float* C0, const float2* ramp,
+                           cudaStream_t s) {
+    if (storage == CL_STORE_FP16DEV) k_init19s<SF16><<<152 * 8, 256, 0, s>>>(st, a, C0, ramp);
+    else k_init19s<SF32><<<152 * 8, 256, 0, s>>>(st, a, C0, ramp);
     return cudaGetLastError();
 }
 
 cudaError_t launch_readout19s(int storage, const Q19State& st, const Q19Args& a, double* out, cudaStream_t s) {
-    if (storage == CL_STORE_FP16DEV) k_readout19s<SF16><<<a.nx, 256, 0, s>>>(st, a, out);
-    else k_readout19s<SF32><<<a.nx, 256, 0, s>>>(st, a, out);
-    return cudaGetLastError();
+    const long long rows = (long long)a.ny * a.nz;
+    if (storage == CL_STORE_FP16DEV) return launch_planes(State19PlaneOp<SF16>{st, a}, a.nx, rows, out, s);
+    return launch_planes(State19PlaneOp<SF32>{st, a}, a.nx, rows, out, s);
 }
 
 cudaError_t launch_out19s(int storage, const Q19State& st, const Q19Args& a, float* C, float* g, cudaStream_t s) {
