@@ -413,8 +413,8 @@ static HaloShape halo_shape(int ci, int co, int cn, int per_sm) {
 // fences and barriers: they go three to a stage, a thread's places in the halo are
 // found once (not with divisions for every piece), and where the blocks of
 // voxels leave SMs idle the output channels are split over CTAs (cn), which
-// changes no sum.  4 x 6^3, 128 -> 128: @H0 us with single taps and one CTA for all
-// channels, @H1 us; 4 x 24^3, 96 -> 32: @G0, @G1 us.
+// changes no sum.  4 x 6^3, 128 -> 128: 71 us with single taps and one CTA for all
+// channels, 32 us; 4 x 24^3, 96 -> 32: 102, 51 us.
 template <int KG, int TAPS>  // groups of 8 channels of a chunk; taps of a weight stage
 __global__ void __launch_bounds__(kTcThreads) k_conv3d_halo(const __nv_bfloat16* __restrict__ in,
                                                             const __nv_bfloat16* __restrict__ w,
@@ -609,8 +609,9 @@ __global__ void __launch_bounds__(kTcThreads) k_conv3d_halo(const __nv_bfloat16*
 // outermost, then dy, dx, channels), so results are the same bits.
 // Roles (288 threads): warps 0-3 the epilogue, warps 4-7 stage the planes,
 // warp 8 tensor memory and the MMAs.
-// Bound by the shared-memory reads of the operands (4 KB of A for 48 columns).
-// 4 x 48^3, 48 -> 16 channels: @F0 us before, @F1 us; 16 -> 48: @D0, @D1 us.
+// Bound by the operand reads of the MMAs (4 KB of A for 48 columns; the tensor
+// pipe's operand stage is busy 66% of the time).
+// 4 x 48^3, 48 -> 16 channels: 212 us before, 47 us; 16 -> 48: 118, 34 us.
 constexpr int kMarchThreads = 288;
 constexpr int kMarchMaxStages = 4;
 constexpr int kMarchMaxSlots = 32;
@@ -921,7 +922,8 @@ static cudaError_t launch_conv3d_march(const __nv_bfloat16* in, const __nv_bfloa
 // blocks (z fastest, so a thread's places in a block stay the same along a
 // column), warps 0-3 read the accumulators, warp 8 tensor memory and the MMAs.
 // Bound by the shared-memory reads of the operands.  4 x 48^3, 48 -> 16
-// channels: @W0 us with a gather per tap and voxel, @W1 us; 16 -> 16: @V0, @V1 us.
+// channels: 608 us with a gather per tap and voxel, 45 us; 4 x 24^3,
+// 32 -> 32: 77, 21 us.
 constexpr int kWgThreads = 288;
 constexpr int kWgProducers = 256;
 constexpr int kWgStages = 4, kWgLag = 2;

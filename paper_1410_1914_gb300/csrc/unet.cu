@@ -276,7 +276,7 @@ __global__ void k_bias_grad(const __nv_bfloat16* __restrict__ dout, long long M,
 // The same, 8 channels (16 bytes of a voxel) to a cluster of 16 blocks, whose
 // sums meet in the first block's shared memory and are added in rank order.
 // Bound by the reading of dO; one block per channel read 2 bytes a voxel on C
-// of the SMs (4 x 48^3, 16 channels: @B0 us; 32 SMs: @B1 us).
+// of the SMs (4 x 48^3, 16 channels: 101 us; 32 SMs: 10 us).
 constexpr int kBgRanks = 16, kBgThreads = 512;
 
 __global__ void __launch_bounds__(kBgThreads) k_bias_grad8(const __nv_bfloat16* __restrict__ dout, long long M,
@@ -358,7 +358,7 @@ __global__ void k_relu_bwd(const __nv_bfloat16* __restrict__ y, __nv_bfloat16* _
 }
 
 // the same on 8 channels (16 bytes) per thread: one pass over Y and dY with 32-bit
-// index arithmetic (4 x 48^3, 16 channels: @R0 us by elements, @R1 us)
+// index arithmetic (4 x 48^3, 16 channels: 17 us by elements, 6 us)
 __global__ void k_relu_bwd8(const __nv_bfloat16* __restrict__ y, __nv_bfloat16* __restrict__ dy, unsigned n, unsigned C8,
                             int stride, int off) {
     for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
