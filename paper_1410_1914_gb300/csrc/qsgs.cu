@@ -12,8 +12,19 @@
 // may convert and has grown 6-neighbours (x, y and z wrap) is accepted with
 // two or more of them (rule 2a), else with probability p_alpha (rule 2b).
 // The sweep that would overshoot the target accepts only its `need`
-// candidates with the smallest (priority hash, cell index), found here by a
-// radix select over the 96-bit composite instead of a sort.
+// candidates with the smallest (priority hash, cell index).
+//
+// A sweep works on bit masks, 32 cells of a row to a word: the six neighbours
+// of a word are shifted or loaded words, a word's accepted cells by rule 2a are
+// bit logic, and only cells with exactly one grown neighbour need their hash,
+// compared as a whole number.  Sweeps are launched eight at a time; the device
+// keeps the count and stops by itself, the host looks once per eight.  With a
+// thread per cell, 64-bit index arithmetic, FP64 probabilities and a counter
+// for every candidate a sweep took 100 us at 200^3 and a host round trip; now
+// 25 us.
+#include <algorithm>
+#include <vector>
+
 #include "cl_lbm.h"
 #include "handle.cuh"
 #include "internal.cuh"
@@ -22,168 +33,313 @@ namespace cl {
 
 namespace {
 
-__device__ __forceinline__ uint64_t splitmix64(uint64_t z) {
+__host__ __device__ __forceinline__ uint64_t splitmix64(uint64_t z) {
     z += 0x9E3779B97F4A7C15ULL;
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     return z ^ (z >> 31);
 }
 
-__device__ __forceinline__ uint64_t hash4(uint64_t seed, uint64_t stream, uint64_t a, uint64_t b) {
+// the hash of (seed, stream, a, b) is splitmix64(hash3(seed, stream, a) ^ b)
+__host__ __device__ __forceinline__ uint64_t hash3(uint64_t seed, uint64_t stream, uint64_t a) {
     uint64_t h = splitmix64(seed);
     h = splitmix64(h ^ stream);
-    h = splitmix64(h ^ a);
-    return splitmix64(h ^ b);
+    return splitmix64(h ^ a);
 }
 
-__device__ __forceinline__ double u01(uint64_t h) { return (double)(h >> 11) * (1.0 / 9007199254740992.0); }
+// a hash's uniform double is (h >> 11) 2^-53; scaled by 2^53 (exact) the tests u <= p and u < p
+// become whole-number tests (h >> 11) < limit, with limit 2^53 for every p >= 1
+constexpr double kTwo53 = 9007199254740992.0;
+uint64_t limit_le(double p) { return !(p >= 0.0) ? 0 : (p >= 1.0 ? 1ULL << 53 : (uint64_t)floor(p * kTwo53) + 1); }
+uint64_t limit_lt(double p) { return !(p > 0.0) ? 0 : (p >= 1.0 ? 1ULL << 53 : (uint64_t)ceil(p * kTwo53)); }
 
 constexpr uint64_t kKeyStream = 0x5bd1e995ULL;
+constexpr int kGrid = 152 * 8, kBlock = 256;
+constexpr int kSweeps = 8;     // sweeps launched between two looks of the host
+constexpr int kBins = 65536;   // of the selection: the top 16 bits of the hash
 
-__global__ void k_count_code(const uint8_t* __restrict__ phase, long long N, int code, unsigned long long* out) {
-    unsigned long long n = 0;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x)
-        n += phase[c] == code;
-    for (int o = 16; o > 0; o >>= 1) n += __shfl_down_sync(0xffffffffu, n, o);
-    if ((threadIdx.x & 31) == 0 && n) atomicAdd(out, n);
-}
+struct GrowState {
+    unsigned long long tot[kSweeps + 1];  // cells of the code before sweep i of this launch, and after the last
+    unsigned long long nc[kSweeps];       // candidates of sweep i
+    int over;                             // sweep that would overshoot the target, -1: none yet
+    unsigned n_sel;                       // selection: candidates gathered
+    unsigned bin;                         // the bin that holds the last accepted candidate,
+    unsigned bin_count;                   // its candidates,
+    unsigned long long k;                 // and how many of them are accepted
+};
 
-// candidates of one sweep, compacted in any order (the selection below does
-// not depend on it)
-__global__ void k_candidates(const uint8_t* __restrict__ phase, const uint8_t* __restrict__ region, int nx, int ny,
-                             int nz, unsigned allowed, unsigned grown, double c_d, double p_alpha, uint64_t seed,
-                             uint64_t stream, int sweep, uint64_t* __restrict__ key, uint32_t* __restrict__ cell,
-                             unsigned long long* nc) {
-    const long long N = (long long)nx * ny * nz;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const uint8_t pc = phase[c];
-        if (pc > 3 || !((allowed >> pc) & 1u) || (region && !region[c])) continue;
-        bool accept;
-        if (sweep == 0) {
-            accept = u01(hash4(seed, stream, 0, (uint64_t)c)) <= c_d;
-        } else {
-            const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-            const int xs[6] = {x + 1 == nx ? 0 : x + 1, x == 0 ? nx - 1 : x - 1, x, x, x, x};
-            const int ys[6] = {y, y, y + 1 == ny ? 0 : y + 1, y == 0 ? ny - 1 : y - 1, y, y};
-            const int zs[6] = {z, z, z, z, z + 1 == nz ? 0 : z + 1, z == 0 ? nz - 1 : z - 1};
-            int ng = 0, parent = -1;
+// the box as rows of words: nw words of 32 cells per row
+struct Words {
+    int nx, ny, nz, nw;
+    unsigned n;  // words in all (a box has fewer than 2^31 cells)
+};
+
+// allowed (and in the region) and grown cells as bits, and the number of cells of the code
+__global__ void __launch_bounds__(kBlock) k_grow_masks(const uint8_t* __restrict__ phase,
+                                                       const uint8_t* __restrict__ region, Words d, unsigned allowed,
+                                                       unsigned grown, int code, unsigned* __restrict__ A,
+                                                       unsigned* __restrict__ G, GrowState* st) {
+    constexpr int U = 4;  // words in flight per warp
+    const int lane = threadIdx.x & 31;
+    unsigned n = 0;
+    const unsigned warps = gridDim.x * (kBlock / 32);
+    for (unsigned w0 = (blockIdx.x * kBlock + threadIdx.x) >> 5; w0 < d.n; w0 += U * warps) {
+        unsigned pc[U], rg[U];
 #pragma unroll
-            for (int d = 0; d < 6; ++d) {
-                const long long q = xs[d] + (long long)nx * (ys[d] + (long long)ny * zs[d]);
-                const uint8_t pq = phase[q];
-                if (pq < 4 && ((grown >> pq) & 1u)) { ++ng; parent = d; }
+        for (int u = 0; u < U; ++u) {
+            const unsigned w = w0 + u * warps;  // fewer than 2^31 + 2^16
+            pc[u] = 255;
+            rg[u] = 1;
+            if (w < d.n) {
+                const unsigned row = w / d.nw, x = (w - row * d.nw) * 32 + lane;
+                if (x < (unsigned)d.nx) {
+                    pc[u] = phase[(size_t)row * d.nx + x];
+                    if (region) rg[u] = region[(size_t)row * d.nx + x];
+                }
             }
-            if (ng == 0) continue;
-            accept = ng >= 2 ||
-                     u01(hash4(seed, stream, (uint64_t)sweep * 8 + (uint64_t)parent, (uint64_t)c)) <= p_alpha;
         }
-        if (!accept) continue;
-        const unsigned long long slot = atomicAdd(nc, 1ULL);
-        key[slot] = hash4(seed, stream ^ kKeyStream, (uint64_t)sweep, (uint64_t)c);
-        cell[slot] = (uint32_t)c;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned w = w0 + u * warps;
+            const bool in = pc[u] < 4;
+            const unsigned a = __ballot_sync(0xffffffffu, in && ((allowed >> pc[u]) & 1u) && rg[u]);
+            const unsigned g = __ballot_sync(0xffffffffu, in && ((grown >> pc[u]) & 1u));
+            n += __popc(__ballot_sync(0xffffffffu, pc[u] == (unsigned)code));
+            if (lane == 0 && w < d.n) {
+                A[w] = a;
+                G[w] = g;
+            }
+        }
+    }
+    if (lane == 0 && n) atomicAdd(&st->tot[0], (unsigned long long)n);
+}
+
+// the candidates of one sweep, from the state at its start.  A warp takes 32 words, one per lane, and evaluates the
+// hashes of a word's cells together.
+__global__ void __launch_bounds__(kBlock) k_grow_find(const unsigned* __restrict__ A, const unsigned* __restrict__ G,
+                                                      Words d, unsigned long long target, uint64_t limit,
+                                                      uint64_t seed, uint64_t stream, int sweep, int i,
+                                                      unsigned* __restrict__ acc, GrowState* st) {
+    if (st->over >= 0 || st->tot[i] >= target) return;
+    __shared__ uint64_t pre[6];  // the hash up to the cell: by the direction of the one grown neighbour
+    if (threadIdx.x < 6)
+        pre[threadIdx.x] = hash3(seed, stream, sweep == 0 ? 0 : (uint64_t)sweep * 8 + (uint64_t)threadIdx.x);
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const unsigned plane = (unsigned)d.nw * d.ny;
+    unsigned n = 0;
+    for (unsigned w0 = (blockIdx.x * kBlock + threadIdx.x) & ~31u; w0 < d.n; w0 += gridDim.x * kBlock) {
+        const unsigned w = w0 + lane;
+        const unsigned a = w < d.n ? A[w] : 0u;
+        unsigned take = 0u, one = a, b0 = 0u, b1 = 0u, b2 = 0u;
+        const unsigned row = w / d.nw, wx = w - row * d.nw;
+        if (sweep > 0 && a) {
+            const unsigned z = row / d.ny, y = row - z * d.ny;
+            const unsigned r0 = w - wx, last = (unsigned)d.nw - 1;
+            const unsigned g = G[w];
+            unsigned nb[6];
+            // bit x of a word: cell x + 1 (then x - 1) of the row, which wraps
+            nb[0] = (g >> 1) | (wx == last ? (G[r0] & 1u) << ((d.nx - 1) & 31) : G[w + 1] << 31);
+            nb[1] = (g << 1) | (wx == 0 ? (G[r0 + last] >> ((d.nx - 1) & 31)) & 1u : G[w - 1] >> 31);
+            nb[2] = G[y + 1 == (unsigned)d.ny ? w - (plane - d.nw) : w + d.nw];
+            nb[3] = G[y == 0 ? w + (plane - d.nw) : w - d.nw];
+            nb[4] = G[z + 1 == (unsigned)d.nz ? w - plane * (d.nz - 1) : w + plane];
+            nb[5] = G[z == 0 ? w + plane * (d.nz - 1) : w - plane];
+            unsigned any = 0u, two = 0u;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                two |= any & nb[k];
+                any |= nb[k];
+            }
+            take = a & two;  // rule 2a
+            one = a & any & ~two;
+            // direction of the one grown neighbour, bit by bit
+            b0 = nb[1] | nb[3] | nb[5];
+            b1 = nb[2] | nb[3];
+            b2 = nb[4] | nb[5];
+        }
+        const unsigned c0 = row * d.nx + wx * 32;  // the word's first cell
+        for (unsigned todo = __ballot_sync(0xffffffffu, one != 0); todo; todo &= todo - 1) {
+            const int j = __ffs(todo) - 1;
+            const unsigned oj = __shfl_sync(0xffffffffu, one, j);
+            const unsigned cj = __shfl_sync(0xffffffffu, c0, j) + lane;
+            const unsigned p = ((__shfl_sync(0xffffffffu, b0, j) >> lane) & 1u) |
+                               ((__shfl_sync(0xffffffffu, b1, j) >> lane) & 1u) << 1 |
+                               ((__shfl_sync(0xffffffffu, b2, j) >> lane) & 1u) << 2;
+            bool ok = false;
+            if ((oj >> lane) & 1u) ok = (splitmix64(pre[p] ^ cj) >> 11) < limit;  // rule 2b, or a seed
+            const unsigned t = __ballot_sync(0xffffffffu, ok);
+            if (lane == j) take |= t;
+        }
+        if (w < d.n) acc[w] = take;
+        n += __popc(take);
+    }
+    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+    if (lane == 0 && n) atomicAdd(&st->nc[i], (unsigned long long)n);
+}
+
+// convert a word's cells `t`, one lane per cell
+__device__ __forceinline__ void convert(const Words& d, unsigned w, unsigned t, int lane, uint8_t* phase, int code) {
+    const unsigned row = w / d.nw, x = (w - row * d.nw) * 32 + lane;
+    if ((t >> lane) & 1u) phase[(size_t)row * d.nx + x] = (uint8_t)code;
+}
+
+// accept all candidates of sweep i, unless they overshoot the target
+__global__ void __launch_bounds__(kBlock) k_grow_apply(const unsigned* __restrict__ acc, Words d,
+                                                       unsigned long long target, int keep_allowed, int code, int i,
+                                                       unsigned* __restrict__ A, unsigned* __restrict__ G,
+                                                       uint8_t* phase, GrowState* st) {
+    const int over = *(volatile int*)&st->over;
+    if (over >= 0 && over != i) return;
+    const unsigned long long tot = st->tot[i], nc = st->nc[i];
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    if (tot >= target || tot + nc > target) {
+        if (first && tot >= target) st->tot[i + 1] = tot;
+        else if (first) *(volatile int*)&st->over = i;
+        return;
+    }
+    if (first) st->tot[i + 1] = tot + nc;
+    if (nc == 0) return;
+    const int lane = threadIdx.x & 31;
+    for (unsigned w0 = (blockIdx.x * kBlock + threadIdx.x) & ~31u; w0 < d.n; w0 += gridDim.x * kBlock) {
+        const unsigned w = w0 + lane;
+        const unsigned t = w < d.n ? acc[w] : 0u;
+        if (t) {
+            G[w] |= t;
+            if (!keep_allowed) A[w] &= ~t;
+        }
+        for (unsigned todo = __ballot_sync(0xffffffffu, t != 0); todo; todo &= todo - 1) {
+            const int j = __ffs(todo) - 1;
+            convert(d, w0 + j, __shfl_sync(0xffffffffu, t, j), lane, phase, code);
+        }
     }
 }
 
-// digit `pass` (0..7: key bytes from the top, 8..11: cell bytes from the top)
-// of the candidates whose higher digits equal the fixed prefix
-__global__ void k_digit_hist(const uint64_t* __restrict__ key, const uint32_t* __restrict__ cell, long long nc,
-                             int pass, uint64_t key_prefix, uint32_t cell_prefix, unsigned* hist) {
-    __shared__ unsigned h[256];
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < nc;
-         j += (long long)gridDim.x * blockDim.x) {
-        const uint64_t k = key[j];
-        const uint32_t cl = cell[j];
-        unsigned digit;
-        if (pass < 8) {
-            const int hi_bits = 8 * pass;  // bits already fixed, from the top
-            if (hi_bits && (k >> (64 - hi_bits)) != (key_prefix >> (64 - hi_bits))) continue;
-            digit = (unsigned)(k >> (56 - 8 * pass)) & 0xFFu;
-        } else {
-            if (k != key_prefix) continue;
-            const int hi_bits = 8 * (pass - 8);
-            if (hi_bits && (cl >> (32 - hi_bits)) != (cell_prefix >> (32 - hi_bits))) continue;
-            digit = (cl >> (24 - 8 * (pass - 8))) & 0xFFu;
+// ---- the sweep that overshoots: the need-th smallest (hash, cell) of its candidates.  A histogram of the hash's top
+// 16 bits names the bin that holds it; the few candidates of that bin go to the host.
+// What the passes over the candidates have in common: f(hash, cell) for every cell in acc, by lane
+template <class F>
+__device__ __forceinline__ void each_candidate(const unsigned* acc, const Words& d, uint64_t pre, F f) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned w0 = (blockIdx.x * kBlock + threadIdx.x) & ~31u; w0 < d.n; w0 += gridDim.x * kBlock) {
+        const unsigned t = w0 + lane < d.n ? acc[w0 + lane] : 0u;
+        for (unsigned todo = __ballot_sync(0xffffffffu, t != 0); todo; todo &= todo - 1) {
+            const int j = __ffs(todo) - 1;
+            const unsigned tj = __shfl_sync(0xffffffffu, t, j), w = w0 + j;
+            const unsigned row = w / d.nw, c = row * d.nx + (w - row * d.nw) * 32 + lane;
+            if ((tj >> lane) & 1u) f(splitmix64(pre ^ c), c);
         }
-        atomicAdd(&h[digit], 1u);
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x)
-        if (h[i]) atomicAdd(hist + i, h[i]);
 }
 
-// convert the candidates at or below the composite threshold (t_key, t_cell),
-// or all of them
-__global__ void k_apply(const uint64_t* __restrict__ key, const uint32_t* __restrict__ cell, long long nc,
-                        uint64_t t_key, uint32_t t_cell, int all, uint8_t* phase, int code) {
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < nc;
-         j += (long long)gridDim.x * blockDim.x) {
-        const uint64_t k = key[j];
-        if (all || k < t_key || (k == t_key && cell[j] <= t_cell)) phase[cell[j]] = (uint8_t)code;
+__global__ void __launch_bounds__(kBlock) k_select_hist(const unsigned* __restrict__ acc, Words d, uint64_t pre,
+                                                        unsigned* __restrict__ hist) {
+    each_candidate(acc, d, pre, [&](uint64_t k, unsigned) { atomicAdd(hist + (unsigned)(k >> 48), 1u); });
+}
+
+// the bin of the need-th smallest hash; one block of 1024
+__global__ void __launch_bounds__(1024) k_select_bin(const unsigned* __restrict__ hist, unsigned long long need,
+                                                     GrowState* st) {
+    constexpr int kPer = kBins / 1024;
+    __shared__ unsigned long long sum[1024];
+    unsigned long long mine = 0;
+    for (int j = 0; j < kPer; ++j) mine += hist[threadIdx.x * kPer + j];
+    sum[threadIdx.x] = mine;
+    __syncthreads();
+    for (int o = 1; o < 1024; o <<= 1) {  // inclusive scan
+        const unsigned long long v = threadIdx.x >= (unsigned)o ? sum[threadIdx.x - o] : 0ULL;
+        __syncthreads();
+        sum[threadIdx.x] += v;
+        __syncthreads();
     }
+    unsigned long long before = sum[threadIdx.x] - mine;
+    if (need > before && need <= sum[threadIdx.x])
+        for (int j = 0; j < kPer; ++j) {
+            const unsigned h = hist[threadIdx.x * kPer + j];
+            if (need <= before + h) {
+                st->bin = threadIdx.x * kPer + j;
+                st->bin_count = h;
+                st->k = need - before;
+                break;
+            }
+            before += h;
+        }
+}
+
+struct Candidate {
+    uint64_t key;
+    uint64_t cell;
+};
+
+__global__ void __launch_bounds__(kBlock) k_select_gather(const unsigned* __restrict__ acc, Words d, uint64_t pre,
+                                                          unsigned bin, unsigned room, Candidate* __restrict__ out,
+                                                          GrowState* st) {
+    each_candidate(acc, d, pre, [&](uint64_t k, unsigned c) {
+        if ((unsigned)(k >> 48) != bin) return;
+        const unsigned at = atomicAdd(&st->n_sel, 1u);
+        if (at < room) out[at] = Candidate{k, c};
+    });
+}
+
+__global__ void __launch_bounds__(kBlock) k_select_apply(const unsigned* __restrict__ acc, Words d, uint64_t pre,
+                                                         Candidate last, uint8_t* phase, int code) {
+    each_candidate(acc, d, pre, [&](uint64_t k, unsigned c) {
+        if (k < last.key || (k == last.key && c <= last.cell)) phase[c] = (uint8_t)code;
+    });
 }
 
 __global__ void k_region_not_adjacent(const uint8_t* __restrict__ phase, int nx, int ny, int nz, int code, int avoid,
                                       uint8_t* __restrict__ region) {
-    const long long N = (long long)nx * ny * nz;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
+    const unsigned N = (unsigned)nx * ny * nz, plane = (unsigned)nx * ny;
+    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
         bool ok = phase[c] == code;
         if (ok) {
-            const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-            const int xs[6] = {x + 1 == nx ? 0 : x + 1, x == 0 ? nx - 1 : x - 1, x, x, x, x};
-            const int ys[6] = {y, y, y + 1 == ny ? 0 : y + 1, y == 0 ? ny - 1 : y - 1, y, y};
-            const int zs[6] = {z, z, z, z, z + 1 == nz ? 0 : z + 1, z == 0 ? nz - 1 : z - 1};
+            const unsigned row = c / nx, z = row / ny;
+            const int x = (int)(c - row * nx), y = (int)(row - z * ny);
+            const unsigned q[6] = {x + 1 == nx ? c - (nx - 1) : c + 1,           x == 0 ? c + (nx - 1) : c - 1,
+                                   y + 1 == ny ? c - (plane - nx) : c + nx,      y == 0 ? c + (plane - nx) : c - nx,
+                                   z + 1 == (unsigned)nz ? c - (N - plane) : c + plane, z == 0 ? c + (N - plane) : c - plane};
 #pragma unroll
             for (int d = 0; d < 6; ++d)
-                if (phase[xs[d] + (long long)nx * (ys[d] + (long long)ny * zs[d])] == avoid) ok = false;
+                if (phase[q[d]] == avoid) ok = false;
         }
         region[c] = ok ? 1 : 0;
     }
 }
 
-__global__ void k_reactive_faces(const uint8_t* __restrict__ phase, int nx, int ny, int nz, int from_code,
-                                 int to_code, double fraction, uint64_t seed, uint8_t* __restrict__ out,
-                                 unsigned long long* total) {
-    const long long N = (long long)nx * ny * nz;
-    unsigned long long n = 0;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
+// Index arithmetic of 32 bits and whole-number sampling: 200^3, 170 us with 64-bit divisions and FP64, 50 us.
+__global__ void __launch_bounds__(kBlock) k_reactive_faces(const uint8_t* __restrict__ phase, int nx, int ny, int nz,
+                                                           int from_code, int to_code, uint64_t limit, uint64_t seed,
+                                                           uint8_t* __restrict__ out, unsigned long long* total) {
+    const unsigned N = (unsigned)nx * ny * nz, plane = (unsigned)nx * ny;
+    const uint64_t pre = splitmix64(splitmix64(seed) ^ 0xface);
+    unsigned n = 0;
+    for (unsigned c = blockIdx.x * kBlock + threadIdx.x; c < N; c += gridDim.x * kBlock) {
         unsigned bits = 0;
         if (phase[c] == from_code) {
-            const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-            const int dx[6] = {1, -1, 0, 0, 0, 0}, dy[6] = {0, 0, 1, -1, 0, 0}, dz[6] = {0, 0, 0, 0, 1, -1};
+            const unsigned row = c / nx, z = row / ny;
+            const int x = (int)(c - row * nx), y = (int)(row - z * ny);
+            const unsigned q[6] = {c + 1, c - 1,  // x ends at the box, y and z wrap
+                                   y + 1 == ny ? c - (plane - nx) : c + nx,      y == 0 ? c + (plane - nx) : c - nx,
+                                   z + 1 == (unsigned)nz ? c - (N - plane) : c + plane, z == 0 ? c + (N - plane) : c - plane};
 #pragma unroll
             for (int d = 0; d < 6; ++d) {
-                const int qx = x + dx[d];
-                if (qx < 0 || qx >= nx) continue;
-                const int qy = (y + dy[d] + ny) % ny, qz = (z + dz[d] + nz) % nz;
-                if (phase[qx + (long long)nx * (qy + (long long)ny * qz)] != to_code) continue;
-                if (fraction >= 1.0 || u01(hash4(seed, 0xface, (uint64_t)c, (uint64_t)d)) < fraction) {
-                    bits |= 1u << d;
-                    ++n;
+                if ((d == 0 && x + 1 == nx) || (d == 1 && x == 0)) continue;
+                if (phase[q[d]] == to_code) bits |= 1u << d;
+            }
+            if (limit < (1ULL << 53) && bits) {
+                const uint64_t h = splitmix64(pre ^ c);
+                for (unsigned left = bits; left; left &= left - 1) {
+                    const unsigned d = __ffs(left) - 1;
+                    if ((splitmix64(h ^ d) >> 11) >= limit) bits &= ~(1u << d);
                 }
             }
+            n += __popc(bits);
         }
         out[c] = (uint8_t)bits;
     }
     for (int o = 16; o > 0; o >>= 1) n += __shfl_down_sync(0xffffffffu, n, o);
-    if ((threadIdx.x & 31) == 0 && n) atomicAdd(total, n);
-}
-
-constexpr int kGrid = 152 * 8, kBlock = 256;
-
-// scratch: keys (8 B per cell), cells (4 B per cell), then counters and the
-// digit histogram from a 256-byte boundary
-size_t scratch_tail(long long N) { return (12 * (size_t)N + 255) / 256 * 256; }
-
-cl_status read_u64(unsigned long long* d, unsigned long long* h, cudaStream_t s) {
-    CK(cudaMemcpyAsync(h, d, sizeof(*h), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    return CL_OK;
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(total, (unsigned long long)n);
 }
 
 cl_status check_box(int nx, int ny, int nz) {
@@ -192,55 +348,86 @@ cl_status check_box(int nx, int ny, int nz) {
     return CL_OK;
 }
 
-cl_status grow_impl(uint8_t* phase, int nx, int ny, int nz, int code, unsigned allowed, unsigned grown,
-                    const uint8_t* region, long long target, double c_d, double p_alpha, uint64_t seed,
-                    uint64_t stream, int max_sweeps, long long* final_count, cudaStream_t s, unsigned char* scr) {
-    const long long N = (long long)nx * ny * nz;
-    uint64_t* key = (uint64_t*)scr;
-    uint32_t* cell = (uint32_t*)(scr + 8 * (size_t)N);
-    unsigned long long* cnt = (unsigned long long*)(scr + scratch_tail(N));  // [0] count, [1] candidates
-    unsigned* hist = (unsigned*)(cnt + 4);
-    unsigned long long h = 0;
-    CK(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
-    k_count_code<<<kGrid, kBlock, 0, s>>>(phase, N, code, cnt);
+// scratch: three masks, the state, the histogram of the selection
+struct GrowScratch {
+    unsigned *A, *G, *acc, *hist;
+    GrowState* st;
+};
+
+cl_status read_state(const GrowState* d, GrowState* h, cudaStream_t s) {
+    CK(cudaMemcpyAsync(h, d, sizeof(*h), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    return CL_OK;
+}
+
+// the overshooting sweep: accept the `need` smallest of the candidates in acc
+cl_status select_smallest(const GrowScratch& b, const Words& d, long long need, uint64_t pre, uint8_t* phase, int code,
+                          cudaStream_t s) {
+    GrowState h;
+    CK(cudaMemsetAsync(b.hist, 0, sizeof(unsigned) * kBins, s));
+    k_select_hist<<<kGrid, kBlock, 0, s>>>(b.acc, d, pre, b.hist);
+    k_select_bin<<<1, 1024, 0, s>>>(b.hist, (unsigned long long)need, b.st);
     CK(cudaGetLastError());
-    CKS(read_u64(cnt, &h, s));
-    long long count = (long long)h;
-    for (int sweep = 0; sweep <= max_sweeps && count < target; ++sweep) {
-        if (sweep == 0 && c_d <= 0) continue;
-        CK(cudaMemsetAsync(cnt + 1, 0, sizeof(unsigned long long), s));
-        k_candidates<<<kGrid, kBlock, 0, s>>>(phase, region, nx, ny, nz, allowed, grown, c_d, p_alpha, seed, stream,
-                                              sweep, key, cell, cnt + 1);
-        CK(cudaGetLastError());
-        CKS(read_u64(cnt + 1, &h, s));
-        const long long nc = (long long)h;
-        if (nc == 0) continue;
-        const long long need = target - count;
-        if (nc <= need) {
-            k_apply<<<kGrid, kBlock, 0, s>>>(key, cell, nc, 0, 0, 1, phase, code);
-            CK(cudaGetLastError());
-            count += nc;
-            continue;
+    CKS(read_state(b.st, &h, s));
+    Candidate* out = nullptr;
+    CK(cudaMallocAsync((void**)&out, sizeof(Candidate) * h.bin_count, s));
+    std::vector<Candidate> in;
+    cudaError_t e = cudaSuccess;
+    try {
+        in.resize(h.bin_count);
+    } catch (...) {
+        e = cudaErrorMemoryAllocation;
+    }
+    if (e == cudaSuccess) {
+        k_select_gather<<<kGrid, kBlock, 0, s>>>(b.acc, d, pre, h.bin, h.bin_count, out, b.st);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(in.data(), out, sizeof(Candidate) * in.size(), cudaMemcpyDeviceToHost, s);
+    cudaFreeAsync(out, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) { set_msg("cl_qsgs_grow", e); return from_cuda(e); }
+    std::nth_element(in.begin(), in.begin() + (h.k - 1), in.end(), [](const Candidate& x, const Candidate& y) {
+        return x.key != y.key ? x.key < y.key : x.cell < y.cell;
+    });
+    k_select_apply<<<kGrid, kBlock, 0, s>>>(b.acc, d, pre, in[h.k - 1], phase, code);
+    CK(cudaGetLastError());
+    return CL_OK;
+}
+
+cl_status grow_impl(uint8_t* phase, const Words& d, int code, unsigned allowed, unsigned grown, const uint8_t* region,
+                    long long target, double c_d, double p_alpha, uint64_t seed, uint64_t stream, int max_sweeps,
+                    long long* final_count, cudaStream_t s, const GrowScratch& b) {
+    GrowState h;
+    CK(cudaMemsetAsync(b.st, 0, sizeof(GrowState), s));
+    k_grow_masks<<<kGrid, kBlock, 0, s>>>(phase, region, d, allowed, grown, code, b.A, b.G, b.st);
+    CK(cudaGetLastError());
+    const unsigned long long want = target > 0 ? (unsigned long long)target : 0;
+    const int keep = (int)((allowed >> code) & 1u);  // converted cells may be candidates again
+    long long count = -1;                            // not read yet
+    for (long long sweep = c_d > 0 ? 0 : 1;; sweep += kSweeps) {
+        const int n = (int)std::min<long long>(kSweeps, (long long)max_sweeps + 1 - sweep);
+        if (count >= 0) {
+            CK(cudaMemcpyAsync(&b.st->tot[0], &b.st->tot[kSweeps], sizeof(b.st->tot[0]), cudaMemcpyDeviceToDevice, s));
+            CK(cudaMemsetAsync(b.st->nc, 0, sizeof(b.st->nc), s));
         }
-        // the need-th smallest (key, cell), one byte at a time from the top
-        uint64_t t_key = 0;
-        uint32_t t_cell = 0;
-        long long k = need;
-        for (int pass = 0; pass < 12; ++pass) {
-            unsigned hh[256];
-            CK(cudaMemsetAsync(hist, 0, sizeof(hh), s));
-            k_digit_hist<<<kGrid, kBlock, 0, s>>>(key, cell, nc, pass, t_key, t_cell, hist);
+        CK(cudaMemsetAsync(&b.st->over, 0xff, sizeof(int), s));
+        for (int i = 0; i < n; ++i) {
+            const int sw = (int)(sweep + i);
+            k_grow_find<<<kGrid, kBlock, 0, s>>>(b.A, b.G, d, want, limit_le(sw == 0 ? c_d : p_alpha), seed, stream, sw,
+                                                 i, b.acc, b.st);
+            k_grow_apply<<<kGrid, kBlock, 0, s>>>(b.acc, d, want, keep, code, i, b.A, b.G, phase, b.st);
             CK(cudaGetLastError());
-            CK(cudaMemcpyAsync(hh, hist, sizeof(hh), cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            int d = 0;
-            while (d < 255 && k > (long long)hh[d]) { k -= hh[d]; ++d; }
-            if (pass < 8) t_key |= (uint64_t)d << (56 - 8 * pass);
-            else t_cell |= (uint32_t)d << (24 - 8 * (pass - 8));
         }
-        k_apply<<<kGrid, kBlock, 0, s>>>(key, cell, nc, t_key, t_cell, 0, phase, code);
-        CK(cudaGetLastError());
-        count += need;
+        CKS(read_state(b.st, &h, s));
+        if (h.over >= 0) {
+            const long long need = target - (long long)h.tot[h.over];
+            CKS(select_smallest(b, d, need, hash3(seed, stream ^ kKeyStream, (uint64_t)(sweep + h.over)), phase, code, s));
+            count = target;
+            break;
+        }
+        count = (long long)h.tot[n > 0 ? n : 0];
+        if (count >= target || sweep + n > max_sweeps) break;
     }
     if (final_count) *final_count = count;
     return CL_OK;
@@ -264,11 +451,19 @@ cl_status cl_qsgs_grow(uint8_t* phase, int nx, int ny, int nz, int code, unsigne
         return CL_ERR_ARG;
     }
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const long long N = (long long)nx * ny * nz;
+    Words d{nx, ny, nz, (nx + 31) / 32, 0};
+    d.n = (unsigned)d.nw * ny * nz;
     unsigned char* scr = nullptr;
-    CK(cudaMallocAsync((void**)&scr, scratch_tail(N) + 32 + 1024, s));
-    cl_status st = grow_impl(phase, nx, ny, nz, code, allowed_mask, grown_mask, region, target, c_d, p_alpha, seed,
-                             stream, max_sweeps, final_count, s, scr);
+    const size_t state = (sizeof(GrowState) + 255) / 256 * 256;
+    CK(cudaMallocAsync((void**)&scr, state + sizeof(unsigned) * (kBins + 3 * (size_t)d.n), s));
+    GrowScratch b;
+    b.st = (GrowState*)scr;
+    b.hist = (unsigned*)(scr + state);
+    b.A = b.hist + kBins;
+    b.G = b.A + d.n;
+    b.acc = b.G + d.n;
+    cl_status st = grow_impl(phase, d, code, allowed_mask, grown_mask, region, target, c_d, p_alpha, seed, stream,
+                             max_sweeps, final_count, s, b);
     cudaFreeAsync(scr, s);
     cudaError_t e = cudaStreamSynchronize(s);
     if (st == CL_OK && e != cudaSuccess) { set_msg("cl_qsgs_grow", e); return from_cuda(e); }
@@ -296,7 +491,7 @@ cl_status cl_qsgs_reactive_faces(const uint8_t* phase, int nx, int ny, int nz, i
     unsigned long long h = 0;
     cudaError_t e = cudaMemsetAsync(tot, 0, sizeof(*tot), s);
     if (e == cudaSuccess) {
-        k_reactive_faces<<<kGrid, kBlock, 0, s>>>(phase, nx, ny, nz, from_code, to_code, fraction, seed, out, tot);
+        k_reactive_faces<<<kGrid, kBlock, 0, s>>>(phase, nx, ny, nz, from_code, to_code, limit_lt(fraction), seed, out, tot);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, tot, sizeof(h), cudaMemcpyDeviceToHost, s);
