@@ -83,7 +83,8 @@ struct Q19Args {
 };
 
 // One time level of the D3Q19 (C, delta) state in the padded layout:
-// (hi, lo) of C side by side as float2, 18 deviation planes (f32 | f16 * s_d).
+// (hi, lo) of C side by side as float2; 18 deviations (f32 | f16 * s_d) by groups of
+// 32 cells of a row, [group][18][32].
 struct Q19State {
     float2* hl;
     void* d;

@@ -16,10 +16,7 @@
 //     dC = sum_i e_i + delta_0(x),  C' = C + dC (double-float),
 //     delta'_i = (1 - omega) (e_i - a_i dC)
 // which is the BGK step rewritten exactly; delta_0 is implied, so the mass
-// of a cell is exact by construction.  Link classes, layout and store
-// sectors as in q19.cu; each link loads (hi, lo) and delta of the cell its
-// population comes from (its own cell for wall and boundary links)
-// unconditionally, so a cell's loads are all in flight together.
+// of a cell is exact by construction.  Link classes as in q19.cu.
 #include <cuda_fp16.h>
 #include <math.h>
 
@@ -44,6 +41,12 @@ __host__ __device__ constexpr int s19_cz(int i) {
     return t[i];
 }
 __host__ __device__ constexpr int s19_opp(int i) { return i == 0 ? 0 : ((i & 1) ? i + 1 : i - 1); }
+// the link with direction (cx, cy, cz)
+__host__ __device__ constexpr int s19_link(int cx, int cy, int cz) {
+    for (int i = 0; i < 19; ++i)
+        if (s19_cx(i) == cx && s19_cy(i) == cy && s19_cz(i) == cz) return i;
+    return 0;
+}
 __host__ __device__ constexpr float s19_w(int i) {
     return i == 0 ? 1.f / 3.f : (i <= 6 ? 1.f / 18.f : 1.f / 36.f);
 }
@@ -58,6 +61,47 @@ struct SF16 {
     static __device__ __forceinline__ float ld(T v) { return __half2float(v); }
     static __device__ __forceinline__ T st(float v) { return __float2half_rn(v); }
 };
+
+// Deviations are stored in groups of 32 cells of a row, [group][18][32], so that
+// the 18 of a cell lie at fixed distances from one address.  Index of the first
+// one (i = 1) of padded cell c; the others follow 32 apart.
+template <class I>
+__device__ __forceinline__ I dev_at(I c) {
+    return (c >> 5) * (I)(18 * 32) + (c & (I)31);
+}
+
+// two floats in a register pair: one instruction for both, rounded as the single ones are
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 f2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 f2_get(F2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 
 // s + e = a + b exactly (Knuth's two-sum)
 __device__ __forceinline__ void two_sum19(float a, float b, float& s, float& e) {
@@ -78,120 +122,272 @@ __device__ __forceinline__ void df_add19(float hi, float lo, float d, float& ho,
 }  // namespace
 
 // ------------------------------------------------------------------- step
-// A block is a 32 x 4 tile of cells (x, y) of one plane: a warp is one row,
-// and the y-neighbour rows a cell reads are mostly the block's own rows,
-// already in L1.  Deviations stay in storage units inside the update
-// (scaled by s_d, 1 for FP32), so nothing is rescaled on its way in or out.
-constexpr int kS19X = 32, kS19Y = 4;
+// A lane updates two neighbouring cells: own and y/z-shifted values come in
+// pairs (one load for two cells), x-shifted ones as the pair's inner value and
+// one more load, so a cell costs half the loads and index arithmetic of a
+// lane per cell; the 18 deviations of a cell lie at fixed distances from one
+// address, and sums and updates of the two cells are one instruction.  A block holds 256 cells of one plane, rows of 64 (of 32 where
+// the padded row is not a multiple of 64: no idle lanes), so that y-neighbour
+// rows are mostly its own, already in L1.  Every load is issued whatever the
+// link's class -- in bounds, see below -- and the classes select afterwards;
+// the end planes and catalytic links, which few cells have, are then set in
+// branches.  Deviations stay in storage units inside the update (scaled by s_d,
+// 1 for FP32), so nothing is rescaled on its way in or out.
+// Bound by issue and by the latency of the loads: 128^3 Pt layer, FP16 state,
+// 78 us a step with a cell per lane and plane-by-plane deviations, 49 us;
+// FP32 state 72, 56 us.
+// The reducing step keeps its sums in floats -- pairs of them (hi, lo) for the
+// fluxes and the reaction -- down to the warp and in FP64 from there: one FP64
+// lane per cell took 515 us at 128^3, 75 us now.
+constexpr int kS19T = 128;
+constexpr int kS19Cells = 2 * kS19T;
 
-template <class S, bool REDUCE, class I>
-__global__ void __launch_bounds__(kS19X * kS19Y) k_step19s(Q19State src, Q19State dst, Q19Args a) {
+template <class S>
+__device__ __forceinline__ float2 ld_pair(const typename S::T* p);
+template <>
+__device__ __forceinline__ float2 ld_pair<SF32>(const float* p) {
+    return *reinterpret_cast<const float2*>(p);
+}
+template <>
+__device__ __forceinline__ float2 ld_pair<SF16>(const __half* p) {
+    return __half22float2(*reinterpret_cast<const __half2*>(p));
+}
+__device__ __forceinline__ void st_pair(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
+__device__ __forceinline__ void st_pair(__half* p, float a, float b) {
+    *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b);
+}
+
+// p += hi + lo, p.y keeping what the additions to p.x lose
+__device__ __forceinline__ void pair_add19(float2& p, float hi, float lo) {
+    float s, e;
+    two_sum19(p.x, hi, s, e);
+    p.x = s;
+    p.y = __fadd_rn(p.y, __fadd_rn(e, lo));
+}
+
+// w (hi + lo) as a pair
+__device__ __forceinline__ float2 scaled19(float w, float hi, float lo) {
+    const float h = __fmul_rn(w, hi);
+    return make_float2(h, __fadd_rn(fmaf(w, hi, -h), __fmul_rn(w, lo)));
+}
+
+template <class S, bool REDUCE, int LX, class I>  // LX lanes to a row
+__global__ void __launch_bounds__(kS19T) k_step19s(Q19State src, Q19State dst, Q19Args a) {
     using T = typename S::T;
     constexpr bool HALF = sizeof(T) == 2;
-    const int x = blockIdx.x * kS19X + threadIdx.x;
-    const int y = blockIdx.y * kS19Y + threadIdx.y, z = blockIdx.z;
+    const int x = (blockIdx.x * LX + threadIdx.x % LX) * 2;
+    const int y = blockIdx.y * (kS19T / LX) + threadIdx.x / LX, z = blockIdx.z;
     const int nx = a.nx, ny = a.ny, nz = a.nz, px = a.px;
     const I NP = (I)a.NP;
-    const I c = (I)x + (I)px * ((I)y + (I)ny * (I)z);
+    const I c = (I)x + (I)px * ((I)y + (I)ny * (I)z);  // even: px is a multiple of 32
     const bool in_row = x < px && y < ny;
-    const uint32_t m = in_row ? a.mask[c] : 0u;
-    const bool act = (m & kQ19Active) != 0;
+    const uint2 mm = in_row ? *reinterpret_cast<const uint2*>(a.mask + c) : make_uint2(0u, 0u);
+    const uint32_t m[2] = {mm.x, mm.y};
+    // Whole 32-byte sectors are written -- 8 cells of FP32 or of C, 16 of FP16 (rows start on 32-cell boundaries) --
+    // so every lane of a sector with an active cell goes through the update; inactive cells come out as zeros.
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned vote = __ballot_sync(0xffffffffu, ((m[0] | m[1]) & kQ19Active) != 0);
+    const bool st_hl = ((vote >> (lane & ~3u)) & 0xFu) != 0;
+    const bool st_d = in_row && (HALF ? ((vote >> (lane & ~7u)) & 0xFFu) != 0 : st_hl);
     const float s_d = HALF ? a.s_d : 1.f, inv_d = HALF ? a.inv_d : 1.f;
     const float2* __restrict__ shl = src.hl;
     const T* __restrict__ sd = reinterpret_cast<const T*>(src.d);
-    float hnew = 0.f, lnew = 0.f;
-    float dn[18];
+    float2 rp[3];                        // J_in, J_out, and R before the sink's factor
+    float rs[4] = {0.f, 0.f, 0.f, 0.f};  // sum C, sum |dC|, sum |C|, non-finite
 #pragma unroll
-    for (int i = 0; i < 18; ++i) dn[i] = 0.f;
-    double rv[RED_N];
-    if (REDUCE)
-#pragma unroll
-        for (int k = 0; k < RED_N; ++k) rv[k] = 0.0;
-    if (act) {
-        const uint32_t rb = (m & kQ19HasReact) ? a.react[c] : 0u;
+    for (int i = 0; i < 3; ++i) rp[i] = make_float2(0.f, 0.f);
+    if (st_d) {
+        float hn[2], ln[2];
         const I plane = (I)px * (I)ny;
         const I oym = y == 0 ? (I)(ny - 1) * (I)px : (I)0 - (I)px;
         const I oyp = y == ny - 1 ? (I)0 - (I)(ny - 1) * (I)px : (I)px;
         const I ozm = z == 0 ? (I)(nz - 1) * plane : (I)0 - plane;
         const I ozp = z == nz - 1 ? (I)0 - (I)(nz - 1) * plane : plane;
-        const float2 own_hl = shl[c];
-        const float hx = own_hl.x, lx = own_hl.y;
-        const float Cx = hx + lx;
-        const float rs = a.rsink;  // 1 - r
-        // own deviations: their sum is -delta_0
-        float sdd = 0.f;
+        // the cells left and right of the pair; at the row's ends the pair's own (the value is not used there)
+        const int xl = x > 0 ? -1 : 0, xr = x + 2 < px ? 2 : 1;
+        // the same steps in deviations, whatever the row (rows start on groups)
+        const int dl = x > 0 && x % 32 == 0 ? -(18 * 32 - 31) : xl, dr2 = x % 32 == 30 && xr == 2 ? 18 * 32 - 30 : xr;
+        const float4 own4 = *reinterpret_cast<const float4*>(shl + c);
+        const float hx[2] = {own4.x, own4.z}, lx[2] = {own4.y, own4.w};
+        const F2 own_a = f2(own4.x, own4.y), own_b = f2(own4.z, own4.w);
+        const float rs_ = a.rsink;  // 1 - r
+        const I cd = dev_at(c);
+        const T* dc = sd + cd;
+        float own[18][2];
+        F2 sdd2 = f2(0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < 18; ++i) sdd += S::ld(sd[(I)i * NP + c]);
-        // per link: (hi, lo, delta) of the cell the population comes from, then e_i
-        float ev[18];
+        for (int i = 0; i < 18; ++i) {
+            const float2 v = ld_pair<S>(dc + i * 32);
+            own[i][0] = v.x;
+            own[i][1] = v.y;
+            sdd2 = f2_add(sdd2, f2(v.x, v.y));  // the sum of the own deviations is -delta_0
+        }
+        const float2 sdd = f2_get(sdd2);
+        // e_i of open and inert links, row by row of sources: (dy, dz) of the row, its links that come from the
+        // cell at the same x, from x - 1 and from x + 1 (0: none)
+        float ev[18][2];
 #pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            const int j = s19_opp(i);
-            const int cx = s19_cx(i), cy = s19_cy(i), cz = s19_cz(i);
-            const bool wall = (m >> (j - 1)) & 1u;
-            const bool own = wall || (cx > 0 && x == 0) || (cx < 0 && x == nx - 1);
-            const I s = c - (I)cx + (cy > 0 ? oym : (cy < 0 ? oyp : (I)0)) + (cz > 0 ? ozm : (cz < 0 ? ozp : (I)0));
-            const I e = own ? c : s;
-            const float2 nhl = shl[e];
-            const float nd = S::ld(sd[(I)((own ? j : i) - 1) * NP + e]);
-            const float ws = s19_w(i) * s_d;
-            // open link; for an own link (hi, lo) are the cell's own and nd = delta_opp: the inert wall value
-            float ei = ws * ((nhl.x - hx) + (nhl.y - lx)) + nd;
-            if (own) {
-                if (wall) {
-                    if ((rb >> (j - 1)) & 1u) ei = fmaf(-rs, nd + ws * Cx, nd);
-                } else if (cx > 0) {
-                    if (a.bc_in == CL_BC_DIRICHLET) ei = 2.0f * ws * ((a.c_in - hx) - lx) - nd;
+        for (int q = 0; q < 9; ++q) {
+            constexpr int row_dy[9] = {0, -1, 1, 0, 0, -1, 1, -1, 1}, row_dz[9] = {0, 0, 0, -1, 1, -1, 1, 1, -1};
+            const int dy = row_dy[q], dz = row_dz[q];
+            const I r = c + (dy < 0 ? oym : (dy > 0 ? oyp : (I)0)) + (dz < 0 ? ozm : (dz > 0 ? ozp : (I)0));
+            const T* dr = q == 0 ? dc : sd + dev_at(r);
+            const float2* hr = shl + r;
+            const float4 n4 = q == 0 ? own4 : *reinterpret_cast<const float4*>(hr);
+            const F2 na = f2(n4.x, n4.y), nb = f2(n4.z, n4.w);
+#pragma unroll
+            for (int cx = -1; cx <= 1; ++cx) {
+                if ((dy != 0 && dz != 0 && cx != 0) || (q == 0 && cx == 0)) continue;
+                const int i = s19_link(cx, -dy, -dz), j = s19_opp(i);
+                F2 sa = na, sb = nb;  // C of the cells that the pair's populations come from, and their deviations
+                float2 nd;
+                if (cx == 0) {
+                    nd = ld_pair<S>(dr + (i - 1) * 32);
                 } else {
-                    if (a.bc_out == CL_BC_DIRICHLET) ei = 2.0f * ws * ((a.c_out - hx) - lx) - nd;
+                    const float2 o = hr[cx > 0 ? xl : xr];
+                    const float od = S::ld(dr[(cx > 0 ? dl : dr2) + (i - 1) * 32]);
+                    const float2 v = q == 0 ? make_float2(own[i - 1][0], own[i - 1][1]) : ld_pair<S>(dr + (i - 1) * 32);
+                    if (cx > 0) {
+                        sa = f2(o.x, o.y);
+                        sb = na;
+                        nd = make_float2(od, v.x);
+                    } else {
+                        sa = nb;
+                        sb = f2(o.x, o.y);
+                        nd = make_float2(v.y, od);
+                    }
+                }
+                const float2 da = f2_get(f2_sub(sa, own_a)), db = f2_get(f2_sub(sb, own_b));
+                const float ws = s19_w(i) * s_d;
+                const float2 open = f2_get(f2_fma(f2(ws, ws), f2(da.x + da.y, db.x + db.y), f2(nd.x, nd.y)));
+                ev[i - 1][0] = (m[0] >> (j - 1)) & 1u ? own[j - 1][0] : open.x;
+                ev[i - 1][1] = (m[1] >> (j - 1)) & 1u ? own[j - 1][1] : open.y;
+            }
+        }
+        const float2 om = *reinterpret_cast<const float2*>(a.omega + c);
+        uint32_t rbits[2];
+        float2 snap = make_float2(0.f, 0.f);
+        if (REDUCE) snap = *reinterpret_cast<const float2*>(a.Csnap + c);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const bool inlet = x + k == 0, outlet = x + k == nx - 1;
+            uint32_t rb = 0u;
+            if (inlet || outlet || (m[k] & kQ19HasReact)) {
+                if (m[k] & kQ19HasReact) rb = a.react[c + k];
+#pragma unroll
+                for (int i = 1; i < 19; ++i) {
+                    const int j = s19_opp(i);
+                    const float ws = s19_w(i) * s_d, nd = own[j - 1][k];
+                    const bool wall = (m[k] >> (j - 1)) & 1u;
+                    if (wall) {
+                        if ((rb >> (j - 1)) & 1u) ev[i - 1][k] = fmaf(-rs_, nd + ws * (hx[k] + lx[k]), nd);
+                    } else if (s19_cx(i) > 0 && inlet) {
+                        ev[i - 1][k] = a.bc_in == CL_BC_DIRICHLET ? 2.0f * ws * ((a.c_in - hx[k]) - lx[k]) - nd : nd;
+                    } else if (s19_cx(i) < 0 && outlet) {
+                        ev[i - 1][k] = a.bc_out == CL_BC_DIRICHLET ? 2.0f * ws * ((a.c_out - hx[k]) - lx[k]) - nd : nd;
+                    }
                 }
             }
-            ev[i - 1] = ei;
+            rbits[k] = rb;
         }
-        float se = 0.f;
+        F2 se = f2(0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < 18; ++i) se += ev[i];
-        const float dCs = se - sdd;  // sum e_i + delta_0, storage units
-        df_add19(hx, lx, dCs * inv_d, hnew, lnew);
-        const float om1 = 1.0f - a.omega[c];
+        for (int i = 0; i < 18; ++i) se = f2_add(se, f2(ev[i][0], ev[i][1]));
+        const F2 dC2 = f2_sub(se, sdd2);  // sum e_i + delta_0, storage units
+        const float2 dCs = f2_get(dC2);
+        df_add19(hx[0], lx[0], dCs.x * inv_d, hn[0], ln[0]);
+        df_add19(hx[1], lx[1], dCs.y * inv_d, hn[1], ln[1]);
+        // an inactive cell's result (finite: it read zeros and state values) becomes zero
+        const bool on[2] = {(m[0] & kQ19Active) != 0, (m[1] & kQ19Active) != 0};
+        const F2 om1 = f2(on[0] ? 1.0f - om.x : 0.f, on[1] ? 1.0f - om.y : 0.f);
 #pragma unroll
-        for (int i = 1; i < 19; ++i) dn[i - 1] = om1 * (ev[i - 1] - s19_w(i) * dCs);
+        for (int k = 0; k < 2; ++k)
+            if (!on[k]) hn[k] = ln[k] = 0.f;
+        T* dd = reinterpret_cast<T*>(dst.d) + cd;
+        float2 dn[18];
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            const float w = s19_w(i);
+            dn[i - 1] = f2_get(f2_mul(om1, f2_fma(f2(-w, -w), dC2, f2(ev[i - 1][0], ev[i - 1][1]))));
+            st_pair(dd + (i - 1) * 32, dn[i - 1].x, dn[i - 1].y);
+        }
+        if (st_hl) *reinterpret_cast<float4*>(dst.hl + c) = make_float4(hn[0], ln[0], hn[1], ln[1]);
         if (REDUCE) {
-            const double id = inv_d;
-            const double Cn = (double)hnew + (double)lnew;
-            double jin = 0.0, jout = 0.0, r = 0.0;
 #pragma unroll
-            for (int i = 1; i < 19; ++i) {
-                const bool wall = (m >> (i - 1)) & 1u;
-                const double gs = (double)s19_w(i) * Cn + (double)dn[i - 1] * id;  // g*_i
-                if (s19_cx(i) < 0 && x == 0 && !wall && a.bc_in == CL_BC_DIRICHLET)
-                    jin += 2.0 * ((double)s19_w(i) * a.c_in_d - gs);
-                if (s19_cx(i) > 0 && x == nx - 1 && !wall && a.bc_out == CL_BC_DIRICHLET)
-                    jout += 2.0 * (gs - (double)s19_w(i) * a.c_out_d);
-                if (rb & (1u << (i - 1))) r += gs;
+            for (int k = 0; k < 2; ++k) {
+                if (!on[k]) continue;
+                const bool inlet = x + k == 0, outlet = x + k == nx - 1;
+                const uint32_t rb = rbits[k];
+                if (inlet || outlet || rb) {
+#pragma unroll
+                    for (int i = 1; i < 19; ++i) {
+                        const bool wall = (m[k] >> (i - 1)) & 1u;
+                        const float w = s19_w(i), d = (k == 0 ? dn[i - 1].x : dn[i - 1].y) * inv_d;  // g*_i = w C + d
+                        if (s19_cx(i) < 0 && inlet && !wall && a.bc_in == CL_BC_DIRICHLET) {
+                            float s, e;
+                            two_sum19(a.c_in, -hn[k], s, e);
+                            e += (float)(a.c_in_d - (double)a.c_in);
+                            const float2 f = scaled19(2.0f * w, s, e - ln[k]);
+                            pair_add19(rp[0], f.x, f.y);
+                            pair_add19(rp[0], -2.0f * d, 0.f);
+                        }
+                        if (s19_cx(i) > 0 && outlet && !wall && a.bc_out == CL_BC_DIRICHLET) {
+                            float s, e;
+                            two_sum19(hn[k], -a.c_out, s, e);
+                            e -= (float)(a.c_out_d - (double)a.c_out);
+                            const float2 f = scaled19(2.0f * w, s, e + ln[k]);
+                            pair_add19(rp[1], f.x, f.y);
+                            pair_add19(rp[1], 2.0f * d, 0.f);
+                        }
+                        if (rb & (1u << (i - 1))) {
+                            const float2 f = scaled19(w, hn[k], ln[k]);
+                            pair_add19(rp[2], f.x, f.y);
+                            pair_add19(rp[2], d, 0.f);
+                        }
+                    }
+                }
+                const float Cf = hn[k] + ln[k];
+                rs[0] += Cf;
+                rs[1] += fabsf(Cf - (k == 0 ? snap.x : snap.y));
+                rs[2] += fabsf(Cf);
+                if (!isfinite(hn[k])) rs[3] += 1.0f;
             }
-            rv[RED_JIN] = jin;
-            rv[RED_JOUT] = jout;
-            rv[RED_R] = a.rsink_d * r;
-            const float Cf = hnew + lnew;
-            rv[RED_SUMC] = Cf;
-            rv[RED_DC] = fabs((double)Cf - (double)a.Csnap[c]);
-            rv[RED_ABSC] = fabs((double)Cf);
-            rv[RED_NONFINITE] = isfinite(hnew) ? 0.0 : 1.0;
-            a.Csnap[c] = Cf;
         }
-    }
-    const unsigned lane = threadIdx.x;  // blockDim.x = 32: the lane
-    const unsigned vote = __ballot_sync(0xffffffffu, act);
-    if (in_row && ((vote >> (lane & ~7u)) & 0xFFu)) {
-        T* ddv = reinterpret_cast<T*>(dst.d);
-        dst.hl[c] = make_float2(hnew, lnew);
-#pragma unroll
-        for (int i = 0; i < 18; ++i) ddv[(I)i * NP + c] = S::st(dn[i]);
+        if (REDUCE) {
+            if (m[0] & kQ19Active) snap.x = hn[0] + ln[0];
+            if (m[1] & kQ19Active) snap.y = hn[1] + ln[1];
+            *reinterpret_cast<float2*>(a.Csnap + c) = snap;
+        }
     }
     if (REDUCE) {
-        const long long blk = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-        block_sum_store<RED_N>(rv, a.partials + blk * RED_N);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                pair_add19(rp[k], __shfl_xor_sync(0xffffffffu, rp[k].x, o), __shfl_xor_sync(0xffffffffu, rp[k].y, o));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) rs[k] += __shfl_xor_sync(0xffffffffu, rs[k], o);
+        }
+        __shared__ float2 part[kS19T / 32][RED_N];
+        if (lane == 0) {
+            float2* q = part[threadIdx.x >> 5];
+            q[RED_JIN] = rp[0];
+            q[RED_JOUT] = rp[1];
+            q[RED_R] = rp[2];
+            q[RED_SUMC] = make_float2(rs[0], 0.f);
+            q[RED_DC] = make_float2(rs[1], 0.f);
+            q[RED_ABSC] = make_float2(rs[2], 0.f);
+            q[RED_NONFINITE] = make_float2(rs[3], 0.f);
+        }
+        __syncthreads();
+        if (threadIdx.x < RED_N) {
+            double v = 0.0;
+            for (int w = 0; w < kS19T / 32; ++w)
+                v += (double)part[w][threadIdx.x].x + (double)part[w][threadIdx.x].y;
+            if (threadIdx.x == RED_R) v *= a.rsink_d;
+            const long long blk = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
+            a.partials[blk * RED_N + threadIdx.x] = v;
+        }
     }
 }
 
@@ -214,25 +410,9 @@ __global__ void k_init19s(Q19State st, Q19Args a, const float* __restrict__ C0, 
             }
         }
         st.hl[p] = make_float2(hi, lo);
-        for (int i = 0; i < 18; ++i) reinterpret_cast<T*>(st.d)[i * NP + p] = S::st(0.f);
+        for (int i = 0; i < 18; ++i) reinterpret_cast<T*>(st.d)[dev_at((unsigned long long)p) + i * 32] = S::st(0.f);
         a.Csnap[p] = hi + lo;
     }
-}
-
-// C = hi + lo and g*_i = a_i C + delta_i of one padded cell
-template <class S>
-__device__ __forceinline__ double state_cell(const Q19State& st, const Q19Args& a, long long p, float (&g)[19]) {
-    using T = typename S::T;
-    constexpr bool HALF = sizeof(T) == 2;
-    const double C = (double)st.hl[p].x + (double)st.hl[p].y;
-    float s = 0.f;
-    for (int i = 1; i < 19; ++i) {
-        const float d = S::ld(reinterpret_cast<const T*>(st.d)[(i - 1) * a.NP + p]) * (HALF ? a.inv_d : 1.f);
-        g[i] = (float)((double)s19_w(i) * C + (double)d);
-        s += d;
-    }
-    g[0] = (float)((double)s19_w(0) * C - (double)s);
-    return C;
 }
 
 // per x-plane (planes.cuh): the deviations are read only where a catalytic or boundary link needs them
@@ -249,7 +429,8 @@ struct State19PlaneOp {
     };
     __device__ __forceinline__ double sink() const { return a.rsink_d; }
     __device__ __forceinline__ float d(int i, long long p) const {
-        return S::ld(reinterpret_cast<const T*>(st.d)[(i - 1) * a.NP + p]) * (sizeof(T) == 2 ? a.inv_d : 1.f);
+        return S::ld(reinterpret_cast<const T*>(st.d)[dev_at((unsigned long long)p) + (i - 1) * 32]) *
+               (sizeof(T) == 2 ? a.inv_d : 1.f);
     }
     __device__ __forceinline__ Item load(int x, int row) const {
         Item t;
@@ -289,45 +470,68 @@ struct State19PlaneOp {
     }
 };
 
-// unpadded C and/or g* as [19][nz][ny][nx]
+// Unpadded C and/or g* as [19][nz][ny][nx]; g*_i = a_i C + delta_i of the pair (hi, lo), rounded once in effect (FP64
+// per cell and population took 120 us at 128^3 FP16, 48 us now, bound by the bytes written)
 template <class S>
-__global__ void k_out19s(Q19State st, Q19Args a, float* __restrict__ C, float* __restrict__ gout) {
+__global__ void __launch_bounds__(256) k_out19s(Q19State st, Q19Args a, float* __restrict__ C, float* __restrict__ gout) {
+    using T = typename S::T;
+    constexpr bool HALF = sizeof(T) == 2;
     const long long N = (long long)a.nx * a.ny * a.nz;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const long long p = (c % a.nx) + (long long)a.px * (c / a.nx);
+    for (long long c = blockIdx.x * 256LL + threadIdx.x; c < N; c += gridDim.x * 256LL) {
+        const long long row = N < (1LL << 32) ? (long long)((uint32_t)c / (uint32_t)a.nx) : c / a.nx;
+        const long long p = (c - row * a.nx) + (long long)a.px * row;
         const bool act = (a.mask[p] & kQ19Active) != 0;
-        float g[19];
-        double Cv = 0.0;
-        if (act) Cv = state_cell<S>(st, a, p, g);
-        else
-            for (int i = 0; i < 19; ++i) g[i] = 0.f;
-        if (C) C[c] = (float)Cv;
-        if (gout)
-            for (int i = 0; i < 19; ++i) gout[i * N + c] = g[i];
+        const float2 hl = act ? st.hl[p] : make_float2(0.f, 0.f);
+        if (C) C[c] = hl.x + hl.y;
+        if (!gout) continue;
+        const T* dp = reinterpret_cast<const T*>(st.d) + dev_at((unsigned long long)p);
+        float s = 0.f;
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            const float d = act ? S::ld(dp[(i - 1) * 32]) * (HALF ? a.inv_d : 1.f) : 0.f;
+            const float2 f = scaled19(s19_w(i), hl.x, hl.y);
+            float t, e;
+            two_sum19(f.x, d, t, e);
+            gout[i * N + c] = t + (e + f.y);
+            s += d;
+        }
+        const float2 f = scaled19(s19_w(0), hl.x, hl.y);
+        float t, e;
+        two_sum19(f.x, -s, t, e);
+        gout[c] = t + (e + f.y);
     }
 }
 
 // -------------------------------------------------------------- launchers
+// lanes of a row: 64-cell rows read the widest, 32-cell ones leave no lane idle (px is a multiple of 32)
+static int step19s_lanes(int px) { return px % 64 == 0 ? 32 : 16; }
+
+static dim3 step19s_grid(int px, int ny, int nz) {
+    const int lx = step19s_lanes(px), rows = kS19T / lx;
+    return dim3((unsigned)(px / (2 * lx)), (unsigned)((ny + rows - 1) / rows), (unsigned)nz);
+}
+
 cudaError_t launch_step19s(int storage, const Q19State& src, const Q19State& dst, const Q19Args& a, bool reduce,
                            cudaStream_t s) {
-    const dim3 g((a.px + kS19X - 1) / kS19X, (a.ny + kS19Y - 1) / kS19Y, a.nz);
-    const dim3 b(kS19X, kS19Y);
-    const bool narrow = !a.wide && 19LL * a.NP < (1LL << 32);
-#define CL_Q19S(SS, R, II) k_step19s<SS, R, II><<<g, b, 0, s>>>(src, dst, a)
+    const dim3 g = step19s_grid(a.px, a.ny, a.nz);
+    const bool narrow = !a.wide && 19LL * a.NP < (1LL << 32), wide_row = step19s_lanes(a.px) == 32;
+#define CL_Q19S(SS, R, LX, II) k_step19s<SS, R, LX, II><<<g, kS19T, 0, s>>>(src, dst, a)
+#define CL_Q19L(SS, R, II) do { if (wide_row) CL_Q19S(SS, R, 32, II); else CL_Q19S(SS, R, 16, II); } while (0)
     if (storage == CL_STORE_FP16DEV) {
-        if (narrow) { if (reduce) CL_Q19S(SF16, true, uint32_t); else CL_Q19S(SF16, false, uint32_t); }
-        else { if (reduce) CL_Q19S(SF16, true, unsigned long long); else CL_Q19S(SF16, false, unsigned long long); }
+        if (narrow) { if (reduce) CL_Q19L(SF16, true, uint32_t); else CL_Q19L(SF16, false, uint32_t); }
+        else { if (reduce) CL_Q19L(SF16, true, unsigned long long); else CL_Q19L(SF16, false, unsigned long long); }
     } else {
-        if (narrow) { if (reduce) CL_Q19S(SF32, true, uint32_t); else CL_Q19S(SF32, false, uint32_t); }
-        else { if (reduce) CL_Q19S(SF32, true, unsigned long long); else CL_Q19S(SF32, false, unsigned long long); }
+        if (narrow) { if (reduce) CL_Q19L(SF32, true, uint32_t); else CL_Q19L(SF32, false, uint32_t); }
+        else { if (reduce) CL_Q19L(SF32, true, unsigned long long); else CL_Q19L(SF32, false, unsigned long long); }
     }
+#undef CL_Q19L
 #undef CL_Q19S
     return cudaGetLastError();
 }
 
 int step19s_blocks(int px, int ny, int nz) {
-    return ((px + kS19X - 1) / kS19X) * ((ny + kS19Y - 1) / kS19Y) * nz;
+    const dim3 g = step19s_grid(px, ny, nz);
+    return (int)(g.x * g.y * g.z);
 }
 
 cudaError_t launch_init19s(int storage, const Q19State& st, const Q19Args& a, const float* C0, const float2* ramp,
