@@ -617,8 +617,10 @@ cl_status cl_lbm_create(cl_handle* out, const cl_params* p) {
         // memory, and no lane stores there (a sector with an active cell
         // lies inside the pitch)
         h->px = std::max((h->nx + 15) / 16 * 16, kBX);
-        // L2 prefetch pays off for the FP32 state (memory-latency bound), not for FP16 (issue bound)
-        h->prefetch = p->storage == CL_STORE_FP32 ? 2 : 0;
+        // No L2 prefetch ahead of the ring: two planes in flight keep the memory busy, and more of them cost
+        // more than they hide (FP32 state, two planes ahead and none: 161 x 187 x 203 82 and 69 us a step,
+        // 192^3 83 and 80, 128^3 22.3 and 22.1, 100^3 14.5 and 12.6)
+        h->prefetch = kPrefetchDefault;
         if (const char* e = getenv("CL_LBM_PREFETCH")) h->prefetch = atoi(e);  // tuning override
         h->NP = (long long)h->px * (h->ny + 2) * h->nz;
         h->tile_rw = march_auto_rows(h->nx, h->ny, h->p.storage);

@@ -130,15 +130,6 @@ __device__ __forceinline__ void pair_add(float2& p, float hi, float lo) {
     p.x = t;
 }
 
-// (hi, lo) + d, renormalised
-__device__ __forceinline__ void df_add(float hi, float lo, float d, float& ho, float& lo_out) {
-    float s, e;
-    two_sum(hi, d, s, e);
-    e += lo;
-    ho = s + e;
-    lo_out = e - (ho - s);
-}
-
 // ------------------------------------------------------- shared layout
 template <class S, int RW>
 struct SlotLayout {
@@ -222,83 +213,126 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// Per-cell update on the (C, delta) state, in storage units: deviations
-// scaled by s_d and low words by s_lo (both 1 for FP32 storage), so that no
-// value is rescaled on its way in or out.  nh/nls/nds: neighbour hi, low word
-// and the deviation travelling toward this cell, for i = 1..6 (+x, -x, +y,
-// -y, +z, -z).  Population i arrives through face opp(i), whose mask bit and
-// own opposite deviation index are both i ^ 1.
+// Update of two neighbouring cells (x, x + 1) on the (C, delta) state, in storage
+// units: deviations scaled by s_d and low words by s_lo (both 1 for FP32
+// storage), so that no value is rescaled on its way in or out.  nh/nls/nds:
+// neighbour hi, low word and the deviation travelling toward the cell, for
+// i = 1..6 (+x, -x, +y, -y, +z, -z).  Population i arrives through face opp(i),
+// whose mask bit and own opposite deviation index are both i ^ 1.
+// The step is bound by the instructions it issues (82% of the slots at 256^3
+// with the FP16 state, at 67% of the memory rate, when each cell had its own),
+// so both cells go through packed instructions; an inactive cell (zeros) counts
+// as closed on all sides, which leaves it the zeros it holds without a
+// selection per value; and the catalytic faces, which few cells have, are in a
+// branch.  256^3 FP16 state: 123 us a step before, 109 us;
+// 128^3 19.0, 16.9; FP32 state 256^3 176, 165.
 template <class S, bool REDUCE>
-__device__ __forceinline__ void cell_update(const MarchArgs& a, uint32_t m, float om, float hx, float lxs,
-                                            const float (&dds)[6], const float (&nh)[6], const float (&nls)[6],
-                                            const float (&nds)[6], int x, float& hnew, float& lnew_s,
-                                            float (&dns)[6], float2 (&rp)[3], float (&rs)[4], float csnap,
-                                            float& csnap_out) {
+__device__ __forceinline__ void pair_update(const MarchArgs& a, uint32_t ma, uint32_t mb, F2 om, F2 hx, F2 lxs,
+                                            const F2 (&dds)[6], const F2 (&nh)[6], const F2 (&nls)[6],
+                                            const F2 (&nds)[6], int x, F2& hnew, F2& lnew_s, F2 (&dns)[6],
+                                            float2 (&rp)[3], float (&rs)[4], float2& csnap) {
     constexpr bool HALF = sizeof(typename S::T) == 2;
-    const float inv_lo = HALF ? a.inv_lo : 1.0f, s_lo = HALF ? a.s_lo : 1.0f;
-    const float s_d = HALF ? a.s_d : 1.0f, inv_d = HALF ? a.inv_d : 1.0f;
-    const float w = kW1;
-    const float ws = w * s_d;
-    const float sink = a.rsink;  // 1 - r
-    const float lx = lxs * inv_lo;
-    const float Cx = hx + lx;
-    // catalytic face: r dopp - (1 - r) w C = dopp - (1 - r)(dopp + w C) (the half-way first-order sink)
-    const float wsC = ws * Cx;
-    float av[6];
+    const float s_lo = HALF ? a.s_lo : 1.0f, s_d = HALF ? a.s_d : 1.0f, inv_d = HALF ? a.inv_d : 1.0f;
+    const F2 inv_lo2 = f2(a.inv_lo, a.inv_lo);  // FP16 state
+    const float w = kW1, ws = w * s_d;
+    const F2 ws2 = f2(ws, ws);
+    const F2 lx = HALF ? f2_mul(lxs, inv_lo2) : lxs;
+    const bool act_a = (ma & kActiveBit) != 0, act_b = (mb & kActiveBit) != 0;
+    if (!act_a) ma = 0x3fu;
+    if (!act_b) mb = 0x3fu;
+    F2 av[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
         const int fb = i ^ 1;
-        const float dopp = dds[fb];
-        const float a_open = ws * ((nh[i] - hx) + (nls[i] - lxs) * inv_lo) + nds[i];
-        const float a_closed = (m & (1u << (kReactShift + fb))) ? fmaf(-sink, dopp + wsC, dopp) : dopp;
-        av[i] = (m & (1u << fb)) ? a_closed : a_open;
+        const F2 dh = f2_sub(nh[i], hx), dl = f2_sub(nls[i], lxs);
+        const float2 open = f2_get(f2_fma(ws2, HALF ? f2_fma(dl, inv_lo2, dh) : f2_add(dh, dl), nds[i]));
+        const float2 dopp = f2_get(dds[fb]);
+        av[i] = f2(ma & (1u << fb) ? dopp.x : open.x, mb & (1u << fb) ? dopp.y : open.y);
     }
-    // the x faces of the box (closed, never catalytic, so the loop gave the wall value dopp):
-    // anti-bounce-back at a fixed value, bounce-back at zero flux.  Only the first and last
-    // lanes of a row's end tiles take these branches; every other warp passes them uniformly.
-    if (x == 0 && a.bc_in == CL_BC_DIRICHLET) av[0] = 2.0f * ws * ((a.c_in - hx) - lx) - dds[1];
-    if (x == a.nx - 1 && a.bc_out == CL_BC_DIRICHLET) av[1] = 2.0f * ws * ((a.c_out - hx) - lx) - dds[0];
-    const float dCs = ((av[0] + av[1]) + (av[2] + av[3]) + (av[4] + av[5])) -
-                      ((dds[0] + dds[1]) + (dds[2] + dds[3]) + (dds[4] + dds[5]));
-    float lnew;
-    df_add(hx, lx, dCs * inv_d, hnew, lnew);
-    lnew_s = lnew * s_lo;
-    const float om1 = 1.0f - om;
-    const float t = om1 * w * dCs;
+    // catalytic face: r dopp - (1 - r) w C = dopp - (1 - r)(dopp + w C) (the half-way first-order sink)
+    if (((ma | mb) >> kReactShift) & 0x3fu) {
+        const F2 wsC = f2_mul(ws2, f2_add(hx, lx)), sink2 = f2(-a.rsink, -a.rsink);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) dns[i] = fmaf(om1, av[i], -t);  // (1 - omega)(a_i - w dC)
+        for (int i = 0; i < 6; ++i) {
+            const int fb = i ^ 1;
+            const uint32_t both = (1u << fb) | (1u << (kReactShift + fb));
+            const float2 r = f2_get(f2_fma(sink2, f2_add(dds[fb], wsC), dds[fb])), v = f2_get(av[i]);
+            av[i] = f2((ma & both) == both ? r.x : v.x, (mb & both) == both ? r.y : v.y);
+        }
+    }
+    // The x faces of the box (closed, never catalytic, so they have the wall value dopp): anti-bounce-back at a
+    // fixed value, bounce-back at zero flux.  Only the first and last lanes of a row's end tiles take these
+    // branches; every other warp passes them uniformly.
+    const bool in_a = x == 0 && act_a, out_a = x == a.nx - 1 && act_a, out_b = x + 1 == a.nx - 1 && act_b;
+    if (in_a && a.bc_in == CL_BC_DIRICHLET) {
+        const float2 h = f2_get(hx), l = f2_get(lx), d = f2_get(dds[1]), v = f2_get(av[0]);
+        av[0] = f2(2.0f * ws * ((a.c_in - h.x) - l.x) - d.x, v.y);
+    }
+    if ((out_a || out_b) && a.bc_out == CL_BC_DIRICHLET) {
+        const float2 h = f2_get(hx), l = f2_get(lx), d = f2_get(dds[0]), v = f2_get(av[1]);
+        av[1] = f2(out_a ? 2.0f * ws * ((a.c_out - h.x) - l.x) - d.x : v.x,
+                   out_b ? 2.0f * ws * ((a.c_out - h.y) - l.y) - d.y : v.y);
+    }
+    const F2 dCs = f2_sub(f2_add(f2_add(f2_add(av[0], av[1]), f2_add(av[2], av[3])), f2_add(av[4], av[5])),
+                          f2_add(f2_add(f2_add(dds[0], dds[1]), f2_add(dds[2], dds[3])), f2_add(dds[4], dds[5])));
+    // (hi, lo) + dC, renormalised
+    const F2 d = HALF ? f2_mul(dCs, f2(inv_d, inv_d)) : dCs;
+    const F2 t = f2_add(hx, d), bb = f2_sub(t, hx);
+    const F2 e = f2_add(f2_add(f2_sub(hx, f2_sub(t, bb)), f2_sub(d, bb)), lx);
+    hnew = f2_add(t, e);
+    const F2 lnew = f2_sub(e, f2_sub(hnew, t));
+    lnew_s = HALF ? f2_mul(lnew, f2(s_lo, s_lo)) : lnew;
+    const F2 om1 = f2_sub(f2(1.0f, 1.0f), om);
+    const F2 mt = f2_mul(f2_mul(om1, f2(-w, -w)), dCs);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) dns[i] = f2_fma(om1, av[i], mt);  // (1 - omega)(a_i - w dC)
     if (REDUCE) {
         // Fluxes and reaction (boundary and catalytic cells only: the stopping rule resolves their changes
         // down to 1e-9) in pairs of floats with the rounding errors kept, summed in FP64 by the block; the
         // per-cell diagnostics in per-thread FP32 partials.  In FP64 these conditions were predicated off in
         // most lanes but issued in every one, at 1/64 of the FP32 rate: the reducing step took 0.40 ms at
         // 256^3 and 2.7 ms on the 400^3 NPMC layer, against 0.12 and 0.44 ms of a plain one.
-        float s, e;
-        if (x == 0 && a.bc_in == CL_BC_DIRICHLET) {
-            two_sum(a.c_in, -hnew, s, e);
-            pair_add(rp[0], 2.0f * w * s, 2.0f * w * (e - lnew));
-            pair_add(rp[0], -2.0f * dns[1] * inv_d, 0.f);
-        }
-        if (x == a.nx - 1 && a.bc_out == CL_BC_DIRICHLET) {
-            two_sum(hnew, -a.c_out, s, e);
-            pair_add(rp[1], 2.0f * w * s, 2.0f * w * (e + lnew));
-            pair_add(rp[1], 2.0f * dns[0] * inv_d, 0.f);
-        }
-        const unsigned rb = (m >> kReactShift) & 0x3fu;
-        if (rb) {
+        const float2 hn = f2_get(hnew), ln = f2_get(lnew);
 #pragma unroll
-            for (int d = 0; d < 6; ++d)
-                if (rb & (1u << d)) {  // w C + delta, the weight a power of two
-                    pair_add(rp[2], w * hnew, w * lnew);
-                    pair_add(rp[2], dns[d] * inv_d, 0.f);
-                }
+        for (int k = 0; k < 2; ++k) {
+            if (!(k == 0 ? act_a : act_b)) {
+                if (k == 0) csnap.x = 0.f;
+                else csnap.y = 0.f;
+                continue;
+            }
+            const float hk = k == 0 ? hn.x : hn.y, lk = k == 0 ? ln.x : ln.y;
+            auto dev = [&](int i) {
+                const float2 v = f2_get(dns[i]);
+                return (k == 0 ? v.x : v.y) * inv_d;
+            };
+            float s, err;
+            if (k == 0 && in_a && a.bc_in == CL_BC_DIRICHLET) {
+                two_sum(a.c_in, -hk, s, err);
+                pair_add(rp[0], 2.0f * w * s, 2.0f * w * (err - lk));
+                pair_add(rp[0], -2.0f * dev(1), 0.f);
+            }
+            if ((k == 0 ? out_a : out_b) && a.bc_out == CL_BC_DIRICHLET) {
+                two_sum(hk, -a.c_out, s, err);
+                pair_add(rp[1], 2.0f * w * s, 2.0f * w * (err + lk));
+                pair_add(rp[1], 2.0f * dev(0), 0.f);
+            }
+            const unsigned rb = ((k == 0 ? ma : mb) >> kReactShift) & 0x3fu;
+            if (rb) {
+#pragma unroll
+                for (int q = 0; q < 6; ++q)
+                    if (rb & (1u << q)) {  // w C + delta, the weight a power of two
+                        pair_add(rp[2], w * hk, w * lk);
+                        pair_add(rp[2], dev(q), 0.f);
+                    }
+            }
+            const float Cf = hk + lk;  // the f32 rounding of the double-float C
+            rs[0] += Cf;
+            rs[1] += fabsf(Cf - (k == 0 ? csnap.x : csnap.y));
+            rs[2] += fabsf(Cf);
+            if (!isfinite(hk)) rs[3] += 1.0f;
+            if (k == 0) csnap.x = Cf;
+            else csnap.y = Cf;
         }
-        const float Cf = hnew + lnew;  // the f32 rounding of the double-float C
-        rs[0] += Cf;
-        rs[1] += fabsf(Cf - csnap);
-        rs[2] += fabsf(Cf);
-        if (!isfinite(hnew)) rs[3] += 1.0f;
-        csnap_out = Cf;
     }
 }
 
@@ -307,20 +341,18 @@ template <class S>
 struct Pair;
 template <>
 struct Pair<StoreF32> {
-    static __device__ __forceinline__ float2 ld(const unsigned char* p, float) {
-        return *reinterpret_cast<const float2*>(p);
-    }
-    static __device__ __forceinline__ void st(void* p, float a, float b, float) {
-        *reinterpret_cast<float2*>(p) = make_float2(a, b);
-    }
+    static __device__ __forceinline__ F2 ld(const unsigned char* p) { return *reinterpret_cast<const F2*>(p); }
+    static __device__ __forceinline__ void st(void* p, F2 v) { *reinterpret_cast<F2*>(p) = v; }
 };
 template <>
 struct Pair<StoreF16> {
-    static __device__ __forceinline__ float2 ld(const unsigned char* p, float) {
-        return __half22float2(*reinterpret_cast<const __half2*>(p));
+    static __device__ __forceinline__ F2 ld(const unsigned char* p) {
+        const float2 v = __half22float2(*reinterpret_cast<const __half2*>(p));
+        return f2(v.x, v.y);
     }
-    static __device__ __forceinline__ void st(void* p, float a, float b, float) {
-        *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b);
+    static __device__ __forceinline__ void st(void* p, F2 v) {
+        const float2 f = f2_get(v);
+        *reinterpret_cast<__half2*>(p) = __floats2half2_rn(f.x, f.y);
     }
 };
 
@@ -346,7 +378,7 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
     constexpr int LPR = BX / 2;  // lanes per tile row (two cells each)
     using P = Pair<S>;
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int nx = a.nx, ny = a.ny, nz = a.nz, px = a.px;
+    const int ny = a.ny, nz = a.nz, px = a.px;
     const int nplanes = (ze - zs) + 2;  // zs-1 .. ze
     const long long pstride = (long long)px * (ny + 2);
     bool ok = true;
@@ -424,13 +456,10 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
     const bool row_ok = y < ny;
     const int c_own = (row + 1) * BX + 2 * xl;  // element index, ghosted arrays
     const int c_pl = row * BX + 2 * xl;         // element index, plain arrays
-    // values stay in storage units; cell_update applies the scales
-    const float inv_lo = 1.0f, inv_d = 1.0f, s_lo = 1.0f, s_d = 1.0f;
+    // values stay in storage units; pair_update applies the scales
     constexpr int EL = L::EL;
     auto f1 = [&](const unsigned char* sl, int off) { return *reinterpret_cast<const float*>(sl + off); };
-    auto t1 = [&](const unsigned char* sl, int off, float inv) {
-        return S::ld(*reinterpret_cast<const T*>(sl + off), inv);
-    };
+    auto t1 = [&](const unsigned char* sl, int off) { return S::ld(*reinterpret_cast<const T*>(sl + off), 1.0f); };
     auto slot = [&](int k) { return slots + ((seq + k) % kStages) * L::bytes; };
     auto wait = [&](int k) {
         return mbar_wait_bounded(&full[(seq + k) % kStages], ((seq + k) / kStages) & 1, a.err, a.wait_limit);
@@ -452,9 +481,9 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
     ok = __all_sync(0xffffffffu, wait(0));  // plane zs-1
     // own cells one plane below
     const unsigned char* s0 = slot(0);
-    float2 ph = *reinterpret_cast<const float2*>(s0 + L::o_chi + 4 * c_own);
-    float2 pl = P::ld(s0 + L::o_clo + EL * c_own, inv_lo);
-    float2 pd5 = P::ld(s0 + L::o_d5 + EL * c_pl, inv_d);
+    F2 ph = *reinterpret_cast<const F2*>(s0 + L::o_chi + 4 * c_own);
+    F2 pl = P::ld(s0 + L::o_clo + EL * c_own);
+    F2 pd5 = P::ld(s0 + L::o_d5 + EL * c_pl);
     release(0);
     ok = __all_sync(0xffffffffu, ok && wait(1));  // plane zs
 
@@ -465,114 +494,74 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
         const unsigned char* sp = slot(k + 1);
         const uint32_t mm = row_ok ? *reinterpret_cast<const uint32_t*>(sc + L::o_mk + 2 * c_pl) : 0u;
         const uint32_t ma = mm & 0xffffu, mb = mm >> 16;
-        // Stores go by whole 32-byte sectors: a lane writes (zeros for an
-        // inactive pair, which those cells already hold) whenever any pair
+        // Stores go by whole 32-byte sectors: a lane updates and writes (zeros for
+        // an inactive pair, which those cells already hold) whenever any pair
         // in its sector is active, so that no sector is written in part --
         // a partial sector costs a DRAM read to fill it -- and sectors of
         // inactive cells only are not written at all.  Rows start on
         // 16-cell boundaries (px and every tile width are multiples of 16),
         // so 4 lanes of one tile row cover an f32 sector and 8 lanes an f16
         // sector.
-        const bool pact = ((ma | mb) & kActiveBit) != 0;
-        const unsigned vote = __ballot_sync(0xffffffffu, pact);
+        const unsigned vote = __ballot_sync(0xffffffffu, ((ma | mb) & kActiveBit) != 0);
         const bool st_f32 = ((vote >> (tx & ~3)) & 0xFu) != 0;
-        const bool st_el = EL == 4 ? st_f32 : ((vote >> (tx & ~7)) & 0xFFu) != 0;
-        float hA = 0.f, lA = 0.f, hB = 0.f, lB = 0.f, dA[6], dB[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) { dA[i] = 0.f; dB[i] = 0.f; }
-        float2 cso = make_float2(0.f, 0.f);
-        const long long gi = xa + (long long)px * (y + 1) + pstride * z;
-        if (pact) {
+        const bool st_el = EL == 4 ? st_f32 : ((vote >> (tx & ~7)) & 0xFFu) != 0;  // st_f32 implies it
+        if (st_el) {
+            const long long gi = xa + (long long)px * (y + 1) + pstride * z;
+            const F2* hc = reinterpret_cast<const F2*>(sc + L::o_chi + 4 * c_own);
             // own pair
-            const float2 hx = *reinterpret_cast<const float2*>(sc + L::o_chi + 4 * c_own);
-            const float2 lx = P::ld(sc + L::o_clo + EL * c_own, inv_lo);
-            float2 dp[6];
-            dp[0] = P::ld(sc + L::o_d1 + EL * c_pl, inv_d);
-            dp[1] = P::ld(sc + L::o_d2 + EL * c_pl, inv_d);
-            dp[2] = P::ld(sc + L::o_d3 + EL * c_own, inv_d);
-            dp[3] = P::ld(sc + L::o_d4 + EL * c_own, inv_d);
-            dp[4] = P::ld(sc + L::o_d5 + EL * c_pl, inv_d);
-            dp[5] = P::ld(sc + L::o_d6 + EL * c_pl, inv_d);
-            const float2 om = *reinterpret_cast<const float2*>(sc + L::o_om + 4 * c_pl);
-            // y and z neighbours of both cells
-            const float2 hym = *reinterpret_cast<const float2*>(sc + L::o_chi + 4 * (c_own - BX));
-            const float2 lym = P::ld(sc + L::o_clo + EL * (c_own - BX), inv_lo);
-            const float2 dym = P::ld(sc + L::o_d3 + EL * (c_own - BX), inv_d);
-            const float2 hyp = *reinterpret_cast<const float2*>(sc + L::o_chi + 4 * (c_own + BX));
-            const float2 lyp = P::ld(sc + L::o_clo + EL * (c_own + BX), inv_lo);
-            const float2 dyp = P::ld(sc + L::o_d4 + EL * (c_own + BX), inv_d);
-            const float2 hzp = *reinterpret_cast<const float2*>(sp + L::o_chi + 4 * c_own);
-            const float2 lzp = P::ld(sp + L::o_clo + EL * c_own, inv_lo);
-            const float2 dzp = P::ld(sp + L::o_d6 + EL * c_pl, inv_d);
-            // outer x neighbours
-            const float hxl = f1(sc, xl_f), lxl = t1(sc, xl_lo, inv_lo), dxl = t1(sc, xl_d1, inv_d);
-            const float hxr = f1(sc, xr_f), lxr = t1(sc, xr_lo, inv_lo), dxr = t1(sc, xr_d2, inv_d);
-
+            const F2 hx = *hc;
+            const F2 lx = P::ld(sc + L::o_clo + EL * c_own);
+            F2 dp[6];
+            dp[0] = P::ld(sc + L::o_d1 + EL * c_pl);
+            dp[1] = P::ld(sc + L::o_d2 + EL * c_pl);
+            dp[2] = P::ld(sc + L::o_d3 + EL * c_own);
+            dp[3] = P::ld(sc + L::o_d4 + EL * c_own);
+            dp[4] = P::ld(sc + L::o_d5 + EL * c_pl);
+            dp[5] = P::ld(sc + L::o_d6 + EL * c_pl);
+            const F2 om = *reinterpret_cast<const F2*>(sc + L::o_om + 4 * c_pl);
+            // x, y and z neighbours of both cells
+            const float2 hx1 = f2_get(hx), lx1 = f2_get(lx), d1 = f2_get(dp[0]), d2 = f2_get(dp[1]);
+            const F2 nh[6] = {f2(f1(sc, xl_f), hx1.x), f2(hx1.y, f1(sc, xr_f)),
+                              hc[-BX / 2],             hc[BX / 2],
+                              ph,                      *reinterpret_cast<const F2*>(sp + L::o_chi + 4 * c_own)};
+            const F2 nl[6] = {f2(t1(sc, xl_lo), lx1.x),
+                              f2(lx1.y, t1(sc, xr_lo)),
+                              P::ld(sc + L::o_clo + EL * (c_own - BX)),
+                              P::ld(sc + L::o_clo + EL * (c_own + BX)),
+                              pl,
+                              P::ld(sp + L::o_clo + EL * c_own)};
+            const F2 nd[6] = {f2(t1(sc, xl_d1), d1.x),
+                              f2(d2.y, t1(sc, xr_d2)),
+                              P::ld(sc + L::o_d3 + EL * (c_own - BX)),
+                              P::ld(sc + L::o_d4 + EL * (c_own + BX)),
+                              pd5,
+                              P::ld(sp + L::o_d6 + EL * c_pl)};
             float2 cs = make_float2(0.f, 0.f);
             if (REDUCE) cs = *reinterpret_cast<const float2*>(a.Csnap + gi);
-
-            const bool act_a = (ma & kActiveBit) != 0, act_b = (mb & kActiveBit) != 0;
-            const float dda[6] = {dp[0].x, dp[1].x, dp[2].x, dp[3].x, dp[4].x, dp[5].x};
-            const float nha[6] = {hxl, hx.y, hym.x, hyp.x, ph.x, hzp.x};
-            const float nla[6] = {lxl, lx.y, lym.x, lyp.x, pl.x, lzp.x};
-            const float nda[6] = {dxl, dp[1].y, dym.x, dyp.x, pd5.x, dzp.x};
-            const float ddb[6] = {dp[0].y, dp[1].y, dp[2].y, dp[3].y, dp[4].y, dp[5].y};
-            const float nhb[6] = {hx.x, hxr, hym.y, hyp.y, ph.y, hzp.y};
-            const float nlb[6] = {lx.x, lxr, lym.y, lyp.y, pl.y, lzp.y};
-            const float ndb[6] = {dp[0].x, dxr, dym.y, dyp.y, pd5.y, dzp.y};
-            if (REDUCE) {
-                // the reductions must see active cells only
-                if (act_a)
-                    cell_update<S, true>(a, ma, om.x, hx.x, lx.x, dda, nha, nla, nda, xa, hA, lA, dA, rp, rs, cs.x, cso.x);
-                if (act_b)
-                    cell_update<S, true>(a, mb, om.y, hx.y, lx.y, ddb, nhb, nlb, ndb, xa + 1, hB, lB, dB, rp, rs, cs.y,
-                                         cso.y);
-            } else {
-                // both cells of the pair without a branch; an inactive cell's
-                // result (finite: its neighbours and omega slots hold zeros or
-                // state values) is replaced by the zeros it keeps
-                cell_update<S, false>(a, ma, om.x, hx.x, lx.x, dda, nha, nla, nda, xa, hA, lA, dA, rp, rs, cs.x, cso.x);
-                cell_update<S, false>(a, mb, om.y, hx.y, lx.y, ddb, nhb, nlb, ndb, xa + 1, hB, lB, dB, rp, rs, cs.y,
-                                      cso.y);
-                if (!act_a) {
-                    hA = 0.f; lA = 0.f;
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) dA[i] = 0.f;
-                }
-                if (!act_b) {
-                    hB = 0.f; lB = 0.f;
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) dB[i] = 0.f;
-                }
-            }
+            F2 hn, ln, dn[6];
+            pair_update<S, REDUCE>(a, ma, mb, om, hx, lx, dp, nh, nl, nd, xa, hn, ln, dn, rp, rs, cs);
             // this plane becomes the z-1 neighbour of the next one
             ph = hx;
             pl = lx;
             pd5 = dp[4];
-        }
-        if (st_f32) {
-            *reinterpret_cast<float2*>(a.chi + gi) = make_float2(hA, hB);
-            if (REDUCE) *reinterpret_cast<float2*>(a.Csnap + gi) = cso;
-        }
-        if (st_el) {
-            P::st(reinterpret_cast<T*>(a.clo) + gi, lA, lB, s_lo);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) P::st(reinterpret_cast<T*>(a.d[i]) + gi, dA[i], dB[i], s_d);
-        }
-        if (y == ny - 1) {  // ghost row above row 0
-            const long long gg = xa + pstride * z;
-            if (st_f32) *reinterpret_cast<float2*>(a.chi + gg) = make_float2(hA, hB);
-            if (st_el) {
-                P::st(reinterpret_cast<T*>(a.clo) + gg, lA, lB, s_lo);
-                P::st(reinterpret_cast<T*>(a.d[2]) + gg, dA[2], dB[2], s_d);
+            if (st_f32) {
+                *reinterpret_cast<F2*>(a.chi + gi) = hn;
+                if (REDUCE) *reinterpret_cast<float2*>(a.Csnap + gi) = cs;
             }
-        }
-        if (y == 0) {  // ghost row below row ny-1
-            const long long gg = xa + (long long)px * (ny + 1) + pstride * z;
-            if (st_f32) *reinterpret_cast<float2*>(a.chi + gg) = make_float2(hA, hB);
-            if (st_el) {
-                P::st(reinterpret_cast<T*>(a.clo) + gg, lA, lB, s_lo);
-                P::st(reinterpret_cast<T*>(a.d[3]) + gg, dA[3], dB[3], s_d);
+            P::st(reinterpret_cast<T*>(a.clo) + gi, ln);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) P::st(reinterpret_cast<T*>(a.d[i]) + gi, dn[i]);
+            if (y == ny - 1) {  // ghost row above row 0
+                const long long gg = xa + pstride * z;
+                if (st_f32) *reinterpret_cast<F2*>(a.chi + gg) = hn;
+                P::st(reinterpret_cast<T*>(a.clo) + gg, ln);
+                P::st(reinterpret_cast<T*>(a.d[2]) + gg, dn[2]);
+            }
+            if (y == 0) {  // ghost row below row ny-1
+                const long long gg = xa + (long long)px * (ny + 1) + pstride * z;
+                if (st_f32) *reinterpret_cast<F2*>(a.chi + gg) = hn;
+                P::st(reinterpret_cast<T*>(a.clo) + gg, ln);
+                P::st(reinterpret_cast<T*>(a.d[3]) + gg, dn[3]);
             }
         }
         release(k);
