@@ -1132,7 +1132,9 @@ bool conv3d_wgrad_tc_supported(const ConvGeom& g) {
            g.in_off % 8 == 0 && g.out_stride % 8 == 0 && g.out_off % 8 == 0;
 }
 
-long long wgrad_tc_workspace_floats(const ConvGeom& g) { return (long long)wg_slices(g) * 27LL * g.co * g.ci; }
+long long wgrad_tc_workspace_floats(const ConvGeom& g) {
+    return conv3d_wgrad_tc_supported(g) ? (long long)wg_slices(g) * 27LL * g.co * g.ci : 0;
+}
 
 cudaError_t launch_conv3d_wgrad_tc(const __nv_bfloat16* in, const __nv_bfloat16* dout, float* partial,
                                    const ConvGeom& g, int* err, int* nslices, cudaStream_t s) {
@@ -1140,6 +1142,7 @@ cudaError_t launch_conv3d_wgrad_tc(const __nv_bfloat16* in, const __nv_bfloat16*
     cudaError_t e = cudaFuncSetAttribute(k_conv3d_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const long long nb = wg_blocks(g);
+    if (nb < 1) return cudaErrorInvalidConfiguration;
     const long long per = (nb + wg_slices(g) - 1) / wg_slices(g);
     const int ns = (int)((nb + per - 1) / per);  // no empty slice
     *nslices = ns;

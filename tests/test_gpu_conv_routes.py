@@ -111,3 +111,18 @@ def test_bias_gradient_and_relu_mask(cuda_lib, M, C, stride, off, skip):
     W._call("cl_nn_relu_bwd", W._p(y), W._p(dy), M, C, stride, off, None)
     torch.cuda.synchronize()
     assert torch.equal(dy, exp)
+
+
+def test_calls_outside_the_kernels_range(cuda_lib):
+    """Channel counts without a tensor-core weight gradient have a workspace
+    size, and an empty box is refused."""
+    import torch
+
+    from paper_1410_1914_gb300 import _lib as L
+    from paper_1410_1914_gb300 import warmstart as W
+    assert W._lib().cl_nn_wgrad_workspace(1, 2, 3, 4, 16, 8) > 0
+    assert W._lib().cl_nn_wgrad_workspace(1, 2, 3, 4, 16, 256) > 0
+    t = torch.zeros(27 * 16 * 16, device="cuda")
+    for call in ((0, 2, 3, 4, 16, 16), (1, 2, 3, 0, 16, 16), (1, 2, 3, 4, 16, 8)):
+        with pytest.raises(L.ClError):
+            W._call("cl_nn_conv3d_wgrad", W._p(t), W._p(t), W._p(t), W._p(t), *call, 16, 0, 16, 0, 1, None)
