@@ -644,7 +644,8 @@ cl_status cl_phase_connectivity(const uint8_t* phase, int nx, int ny, int nz, un
    else with probability p_alpha (rule 2b); the sweep that would overshoot
    converts only its candidates with the smallest (priority hash, cell
    index).  At most max_sweeps sweeps; *final_count (nullable) gets the
-   resulting count.  Scratch: 12 B per cell, allocated on the stream.
+   resulting count.  Scratch, allocated on the stream: 12 B per 32 cells of a
+   row (at most 12 B per cell) and 0.3 MB.
    Errors: CL_ERR_ARG (NULL, sizes, code not in 0..3 or not in grown_mask),
    CL_ERR_OOM, CL_ERR_CUDA. */
 cl_status cl_qsgs_grow(uint8_t* phase, int nx, int ny, int nz, int code, unsigned allowed_mask,
