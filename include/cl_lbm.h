@@ -514,7 +514,7 @@ const char* cl_last_error_message(void);
 typedef struct cl_batch* cl_batch_handle;
 
 /* Build the batch (work list, per-member TMA descriptors and arguments).
-   z_chunk: planes per work item (0: 32).  Errors: CL_ERR_ARG, CL_ERR_STATE
+   z_chunk: planes per work item (0: chosen from the members' sizes, 8..64).  Errors: CL_ERR_ARG, CL_ERR_STATE
    (member without structure or at another parity), CL_ERR_OOM, CL_ERR_CUDA. */
 cl_status cl_batch_create(cl_batch_handle* out, const cl_handle* members, int n, int z_chunk);
 

@@ -84,6 +84,31 @@ int batch_auto_rows(const cl_batch* b) {
     return best;
 }
 
+// z range length where the caller leaves it open.  In units of one plane of one block marching alone, a step of the
+// batch takes about W = 1.5 x planes per block (its share of all items' planes, four more per item for the halo and
+// the filling of the ring; three blocks on an SM slow each other) while there is work for every block, and about the
+// longest item's planes and 14 more (queue, dependency, start) when there is not; sqrt(W^2 + L^2) follows measured
+// times within 10% from 8 members of 24..80 cells an edge to 64 of 32..160.  Against 32 planes always, 200 steps: 8
+// members of 24..80 9.6 -> 4.2 ms, 40 of 24..64 12.2 -> 10.4, 24 of 32..160 51.6 -> 49.8 (FP32 state 68.6 -> 65.4).
+// Beyond 64 planes the few long items end unevenly (64 members, 160 planes: 813 against 712 units).
+int auto_z_chunk(const cl_batch* b) {
+    int best = 32;
+    double best_cost = 0.0;
+    bool first = true;
+    for (int zc : {8, 12, 16, 24, 32, 48, 64}) {
+        double planes = 0.0, longest = 0.0;
+        for (int i = 0; i < b->n; ++i) {
+            const int nz = b->m[i]->nz, g = (nz + zc - 1) / zc;
+            planes += (double)items_of(b->m[i], b->rw[i], zc) * ((double)nz / g + 4.0);
+            longest = std::max(longest, (double)((nz + g - 1) / g));
+        }
+        const double w = 1.5 * planes / b->grid, l = longest + 14.0, cost = sqrt(w * w + l * l);
+        if (first || cost < best_cost) { best = zc; best_cost = cost; }
+        first = false;
+    }
+    return best;
+}
+
 // Work list over the running structures: each column's planes split into
 // ceil(nz / z_chunk) ranges of nearly equal length (no short remainder range,
 // whose two halo planes and pipeline fill would cost as much as its work).
@@ -231,7 +256,6 @@ cl_status cl_batch_create(cl_batch_handle* out, const cl_handle* members, int n,
     b->K = h0->p.check_every;
     b->s = h0->s;
     b->parity = h0->cur;
-    b->z_chunk = z_chunk > 0 ? z_chunk : 32;
     b->prefetch = h0->prefetch;
     b->active.assign(n, 1);
     for (int i = 0; i < n; ++i) b->own_rw.push_back(members[i]->tile_rw);
@@ -249,6 +273,7 @@ cl_status cl_batch_create(cl_batch_handle* out, const cl_handle* members, int n,
     if (per_sm < 1 || per_sm_r < 1) { set_msg_txt("batched step kernel does not fit on an SM"); return fail(CL_ERR_CUDA); }
     b->grid = nsm * per_sm;
     b->grid_reduce = nsm * per_sm_r;
+    b->z_chunk = z_chunk > 0 ? z_chunk : auto_z_chunk(b);
     // the work list is largest at the smallest z chunk the autotuner tries, in the member's largest tiling
     for (int i = 0; i < n; ++i) {
         int most = 0;
