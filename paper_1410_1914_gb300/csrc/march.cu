@@ -255,9 +255,9 @@ __device__ __forceinline__ void pair_update(const MarchArgs& a, uint32_t ma, uin
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
             const int fb = i ^ 1;
-            const uint32_t both = (1u << fb) | (1u << (kReactShift + fb));
+            const uint32_t cat = 1u << (kReactShift + fb);  // set on closed faces only
             const float2 r = f2_get(f2_fma(sink2, f2_add(dds[fb], wsC), dds[fb])), v = f2_get(av[i]);
-            av[i] = f2((ma & both) == both ? r.x : v.x, (mb & both) == both ? r.y : v.y);
+            av[i] = f2(ma & cat ? r.x : v.x, mb & cat ? r.y : v.y);
         }
     }
     // The x faces of the box (closed, never catalytic, so they have the wall value dopp): anti-bounce-back at a
