@@ -219,15 +219,22 @@ cl_status cl_lbm_step(cl_handle h, long long nsteps);
    info may be NULL. */
 cl_status cl_lbm_solve(cl_handle h, cl_solve_info* info);
 
-/* Test hook of the step kernel's bounded waits (no counterpart in the
-   paper; D3Q7 (C, delta) storage, the only kernel with device-side waits).
-   wait_limit_clocks: SM clock cycles a consumer or producer warp waits on a
-   plane's mbarrier before it gives up (0: the default, about 1 s).
+/* Test hook of the bounded device-side waits (no counterpart in the paper).
+   D3Q7 (C, delta) storage, the step kernel: wait_limit_clocks: SM clock
+   cycles a consumer or producer warp waits on a plane's mbarrier before it
+   gives up (0: the default, about 1 s).
    never_arrive (needs a limit > 0): the producer issues no plane load, so
    the consumers' first wait runs out after the limit; the kernel then
    returns without touching the state, and cl_lbm_solve / _solve_budget
    report CL_ERR_TIMEOUT.  The error word is cleared once reported; set
    (0, 0) to restore normal stepping.  Drops the captured step graphs.
+   Population storage, cl_lbm_solve_krylov_dsa / _solve_steady_lines: the
+   limit is that of the meetings of a whole grid's blocks (0: about 2 s;
+   systems small enough for one cluster meet at its hardware barrier, which
+   has no limit and needs none: its blocks are resident together).
+   never_arrive 1: no meeting of a grid comes about; 2: one block alone
+   misses the last meeting of a Gram-Schmidt, which the others make.  Either
+   way the solve returns CL_ERR_TIMEOUT and leaves the state as it was.
    Errors: CL_ERR_ARG. */
 cl_status cl_lbm_set_wait_test(cl_handle h, long long wait_limit_clocks, int never_arrive);
 
@@ -343,7 +350,9 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
    post-collision populations of the result, so every readout applies.
    Needs D3Q7 and CL_STORE_FP32POP, else CL_ERR_STATE.  Returns
    CL_ERR_NOT_CONVERGED at max_iter, CL_ERR_DIVERGED on a non-finite
-   residual or a breakdown of the inner solve, CL_ERR_OOM / CL_ERR_CUDA. */
+   residual or a breakdown of the inner solve, CL_ERR_TIMEOUT when a wait of
+   its blocks for one another ran out (the state is then as it was),
+   CL_ERR_OOM / CL_ERR_CUDA. */
 typedef struct {
     int iterations;              /* GMRES iterations (applications of F) */
     int cycles;                  /* GMRES cycles */

@@ -71,7 +71,7 @@ MarchArgs make_margs(cl_lbm* h, int dst) {
     a.partials = h->partials;
     a.err = h->d_err;
     a.wait_limit = h->wait_limit;
-    a.never_arrive = h->never_arrive;
+    a.never_arrive = h->never_arrive != 0;
     return a;
 }
 
@@ -825,7 +825,7 @@ cl_status cl_lbm_set_wait_test(cl_handle h, long long wait_limit_clocks, int nev
         return CL_ERR_ARG;
     }
     h->wait_limit = wait_limit_clocks;
-    h->never_arrive = never_arrive ? 1 : 0;
+    h->never_arrive = never_arrive == 2 ? 2 : (never_arrive ? 1 : 0);
     drop_graphs(h);  // the wait settings are baked into captured kernel arguments
     return CL_OK;
 }
@@ -1144,8 +1144,7 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
         float *wv = Z + (size_t)Lc * kM, *e = wv + Lc, *c = e + Lc;
         float* cfull = nullptr;  // the residual in the population layout
         CKS(sc.get((void**)&cfull, sizeof(float) * (size_t)L));
-        PcgArgs<float> cg;
-        memset(&cg, 0, sizeof(cg));
+        PcgArgs<float> cg = {};
         cg.tol2 = kCgTol * kCgTol;
         cg.max_iters = kMaxCg;
         CKS(sc.get((void**)&cg.u, sizeof(float) * n));
@@ -1159,6 +1158,8 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
         cg.meet_blocks = dsa_mgs_blocks();
         CKS(sc.get(&cg.meet_mem, pcg_meet_bytes(cg.meet_blocks)));
         CKS(sc.get((void**)&cg.out, sizeof(PcgOut)));
+        CK(cudaMemsetAsync(cg.out, 0, sizeof(PcgOut), h->s));
+        cg.waits = PcgWaits(h->wait_limit, h->never_arrive);
         double *x64 = nullptr, *y64 = nullptr, *part = nullptr, *dcol = nullptr, *dnrm = nullptr, *dy = nullptr;
         KryScalars* ks = nullptr;
         CKS(sc.get((void**)&x64, sizeof(double) * (size_t)L));
@@ -1207,12 +1208,12 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
                     CK(launch_dsa_prec(d, V + (size_t)j * Lc, zj, cg, h->s));
                     CK(launch_dsa_apply(d, zj, wv, h->s));  // (I - A) Z_j
                     ++iters;
-                    CK(launch_dsa_mgs(V, Lc, j, wv, Lc, dcol, cg.meet_mem, h->s));
+                    CK(launch_dsa_mgs(V, Lc, j, wv, Lc, dcol, cg.meet_mem, cg.out, cg.waits, h->s));
                     PcgOut po;
                     CK(cudaMemcpyAsync(&po, cg.out, sizeof(po), cudaMemcpyDeviceToHost, h->s));
                     CKS(host_double(dcol, col, j + 2));
                     cg_total += po.iters;
-                    if (po.bad == 3 || col[j + 1] < 0.0) {
+                    if (po.gave_up) {
                         set_msg_txt("a wait of the steady solve's blocks for one another ran out");
                         return CL_ERR_TIMEOUT;
                     }

@@ -317,8 +317,10 @@ constexpr int kMgsT = 512;
 // One launch orthogonalises w against V[0..j]: w stays in registers (K4
 // float4 per thread; 0: in memory), each V_k is read once from memory and a
 // second time, for the subtraction, from the SM's own cache, and the blocks
-// meet once per vector (a wait that runs out leaves col[j + 1] = -1).  As a dot product, its finish and a subtraction per
-// vector the same took 38 + 3 + 10 us per vector at 96^3.
+// meet once per vector.  As a dot product, its finish and a subtraction per
+// vector the same took 38 + 3 + 10 us per vector at 96^3.  A block whose wait
+// runs out leaves its share of V[j + 1] unwritten; it says so in PcgOut::gave_up,
+// not in col: at the last meeting the others may not miss it.
 template <int K4>
 __global__ void __launch_bounds__(kMgsT, 2) k_dsa_mgs(const float* __restrict__ V, long long stride, int j, float* w,
                                                       long long L4, float* vnext, double* __restrict__ col,
@@ -351,7 +353,7 @@ __global__ void __launch_bounds__(kMgsT, 2) k_dsa_mgs(const float* __restrict__ 
     // sets of partials in turn: a block still reading one is not overwritten.
     PcgGrid sync;
     int set = 0;
-    auto total = [&](float s, float e) -> bool {
+    auto total = [&](float s, float e, bool last = false) -> bool {
         warp_dot2(s, e);
         if (lane == 0) sh[warp] = (double)s + (double)e;
         __syncthreads();
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(kMgsT, 2) k_dsa_mgs(const float* __restrict__ 
             for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
             sync.put(meet, nullptr, set, t, lane);
         }
-        if (!sync.meet(meet)) return false;
+        if (!sync.meet(meet, last)) return false;
         if (warp == 0) {
             const double t = sync.get(meet, nullptr, set, lane);
             if (lane == 0) { tot = t; s_f = (float)t; }
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(kMgsT, 2) k_dsa_mgs(const float* __restrict__ 
             if ((lane & 7) == 0)
                 for (long long i = t0; i < L4; i += step) asm volatile("prefetch.global.L2 [%0];" ::"l"(vx + i));
         }
-        if (!total(s, e)) { if (threadIdx.x == 0) col[j + 1] = -1.0; return; }
+        if (!total(s, e)) return;
         if (blockIdx.x == 0 && threadIdx.x == 0) col[k] = tot;
         h = s_f;
     }
@@ -413,7 +415,7 @@ __global__ void __launch_bounds__(kMgsT, 2) k_dsa_mgs(const float* __restrict__ 
             dot2(v.z, v.z, s, e);
             dot2(v.w, v.w, s, e);
         });
-        if (!total(s, e)) { if (threadIdx.x == 0) col[j + 1] = -1.0; return; }
+        if (!total(s, e, true)) return;
     }
     if (threadIdx.x == 0) {
         const double nrm = sqrt(tot);
@@ -540,7 +542,7 @@ int dsa_mgs_blocks() { return 2 * device_sms(); }
 
 template <int K4>
 static cudaError_t mgs_k(int blocks, const float* V, long long stride, int j, float* w, long long L4, float* vnext,
-                         double* col, void* meet_mem, cudaStream_t s) {
+                         double* col, void* meet_mem, PcgOut* out, const PcgWaits& waits, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(meet_mem, 0, pcg_meet_bytes(blocks), s);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -552,27 +554,27 @@ static cudaError_t mgs_k(int blocks, const float* V, long long stride, int j, fl
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_dsa_mgs<K4>, V, stride, j, w, L4, vnext, col, pcg_meet(meet_mem, blocks));
+    return cudaLaunchKernelEx(&cfg, k_dsa_mgs<K4>, V, stride, j, w, L4, vnext, col, pcg_meet(meet_mem, blocks, out, waits));
 }
 
 cudaError_t launch_dsa_mgs(float* V, long long stride, int j, float* w, long long L, double* col, void* meet_mem,
-                           cudaStream_t s) {
+                           PcgOut* out, const PcgWaits& waits, cudaStream_t s) {
     const long long L4 = L / 4;
     const int most = dsa_mgs_blocks();
     const auto blocks = [&](int k4) { return (L4 + (long long)k4 * kMgsT - 1) / ((long long)k4 * kMgsT); };
     float* vn = V + (long long)(j + 1) * stride;
     // small vectors: few blocks, whose meetings cost less; then every SM with the fewest elements per thread
-    if (blocks(1) <= most) return mgs_k<1>((int)blocks(1), V, stride, j, w, L4, vn, col, meet_mem, s);
+    if (blocks(1) <= most) return mgs_k<1>((int)blocks(1), V, stride, j, w, L4, vn, col, meet_mem, out, waits, s);
     switch (blocks(1) <= 8LL * most ? (int)((blocks(1) + most - 1) / most) : 0) {
-        case 2: return mgs_k<2>(most, V, stride, j, w, L4, vn, col, meet_mem, s);
-        case 3: return mgs_k<3>(most, V, stride, j, w, L4, vn, col, meet_mem, s);
-        case 4: return mgs_k<4>(most, V, stride, j, w, L4, vn, col, meet_mem, s);
+        case 2: return mgs_k<2>(most, V, stride, j, w, L4, vn, col, meet_mem, out, waits, s);
+        case 3: return mgs_k<3>(most, V, stride, j, w, L4, vn, col, meet_mem, out, waits, s);
+        case 4: return mgs_k<4>(most, V, stride, j, w, L4, vn, col, meet_mem, out, waits, s);
         case 5:
-        case 6: return mgs_k<6>(most, V, stride, j, w, L4, vn, col, meet_mem, s);
+        case 6: return mgs_k<6>(most, V, stride, j, w, L4, vn, col, meet_mem, out, waits, s);
         case 7:
-        case 8: return mgs_k<8>(most, V, stride, j, w, L4, vn, col, meet_mem, s);
+        case 8: return mgs_k<8>(most, V, stride, j, w, L4, vn, col, meet_mem, out, waits, s);
     }
-    return mgs_k<0>(most, V, stride, j, w, L4, vn, col, meet_mem, s);
+    return mgs_k<0>(most, V, stride, j, w, L4, vn, col, meet_mem, out, waits, s);
 }
 
 cudaError_t launch_dsa_update(float* e, const float* Z, long long stride, int m, const double* y, long long L,

@@ -47,9 +47,10 @@ bool dsa_prec_streams(int n);
 
 // Modified Gram-Schmidt of w against V[0..j] (vectors of L floats, `stride`
 // apart), in one launch: col[k] = V_k.w, w -= col[k] V_k, col[j + 1] = |w|,
-// V[j + 1] = w / |w|.  meet_mem: pcg_meet_bytes(dsa_mgs_blocks()).
+// V[j + 1] = w / |w|.  meet_mem: pcg_meet_bytes(dsa_mgs_blocks()); out->gave_up
+// says that a wait ran out.
 cudaError_t launch_dsa_mgs(float* V, long long stride, int j, float* w, long long L, double* col, void* meet_mem,
-                           cudaStream_t s);
+                           PcgOut* out, const PcgWaits& waits, cudaStream_t s);
 int dsa_mgs_blocks();
 // e += sum_k y[k] Z_k, k < m
 cudaError_t launch_dsa_update(float* e, const float* Z, long long stride, int m, const double* y, long long L,

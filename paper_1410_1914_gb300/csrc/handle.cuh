@@ -86,7 +86,7 @@ struct cl_lbm {
     double* src = nullptr;     // per-cell source per step (cl_lbm_set_source), NULL: none
     double src_sum = 0.0;      // sum of the sources over active cells (enters the flux balance)
     double *kscale_buf = nullptr, *src_buf = nullptr;  // their storage, allocated on first use
-    long long wait_limit = 0;  // bounded device waits of the step kernel (0: default)
+    long long wait_limit = 0;  // bounded device waits of the step kernel and the steady solves (0: default)
     int never_arrive = 0;      // test hook (cl_lbm_set_wait_test)
 
     int cur = 0;

@@ -37,19 +37,40 @@ namespace cl {
 struct PcgOut {
     double rr, rr0;  // r.r at the end and at the start
     int iters;
-    int bad;  // 0 converged or out of iterations; 1 breakdown or non-finite; 2 nothing to solve; 3 a wait ran out
+    int bad;  // 0 converged or out of iterations; 1 breakdown or non-finite; 2 nothing to solve
+    // Set by a block whose wait ran out, of any kernel of the call (the Gram-Schmidt too), and never cleared: a block
+    // may give up a meeting that the others still make, and then only this word says that its share is missing.
+    unsigned gave_up;
 };
 
-// Words the blocks of a grid meet through (device, zeroed before the launch).
+// Words the blocks of a grid meet through.
 struct PcgMeet {
     double* part;       // [2][3][blocks] partial sums
-    unsigned* counter;  // arrivals, then an abort word
+    unsigned* counter;  // arrivals (zeroed before the launch)
+    unsigned* gave_up;  // PcgOut::gave_up
+    long long limit;    // SM clocks a block waits
+    int never_arrive;   // test hook (cl_lbm_set_wait_test): 1: no meeting comes about; 2: the last block waits for one
+                        // arrival too many at its last meeting of a Gram-Schmidt
 };
-inline size_t pcg_meet_bytes(int blocks) { return sizeof(double) * 6 * (size_t)blocks + 2 * sizeof(unsigned); }
-inline PcgMeet pcg_meet(void* p, int blocks) {
+inline size_t pcg_meet_bytes(int blocks) { return sizeof(double) * 6 * (size_t)blocks + sizeof(unsigned); }
+
+constexpr long long kPcgWaitClocks = 1LL << 32;  // about 2 s of SM clock
+
+// How long the blocks of a call wait, from the handle's test settings (0: the default).
+struct PcgWaits {
+    long long limit = kPcgWaitClocks;
+    int never_arrive = 0;
+    PcgWaits() = default;
+    PcgWaits(long long limit_clocks, int never) : limit(limit_clocks > 0 ? limit_clocks : kPcgWaitClocks), never_arrive(never) {}
+};
+
+inline PcgMeet pcg_meet(void* p, int blocks, PcgOut* out, const PcgWaits& w) {
     PcgMeet m;
     m.part = (double*)p;
     m.counter = (unsigned*)(m.part + 6 * (size_t)blocks);
+    m.gave_up = &out->gave_up;
+    m.limit = w.limit;
+    m.never_arrive = w.never_arrive;
     return m;
 }
 
@@ -66,31 +87,32 @@ struct PcgArgs {
     PcgMeet meet;
     void* meet_mem;     // pcg_meet_bytes(meet_blocks)
     int meet_blocks;
-    PcgOut* out;
+    PcgWaits waits;
+    PcgOut* out;  // zeroed once per call
 };
 
 constexpr int kPcgMaxCluster = 16;
-constexpr long long kPcgWaitClocks = 1LL << 32;  // about 2 s of SM clock
 
 // All blocks of a cooperative launch.
 struct PcgGrid {
     unsigned target = 0;
-    // everything the blocks wrote is visible to all; false when the wait ran out
-    __device__ __forceinline__ bool meet(const PcgMeet& m) {
+    // everything the blocks wrote is visible to all; false when the wait ran out (last: of a Gram-Schmidt, for the hook)
+    __device__ __forceinline__ bool meet(const PcgMeet& m, bool last = false) {
         bool ok = true;
         __syncthreads();
         if (gridDim.x == 1) return true;
         if (threadIdx.x == 0) {
             target += gridDim.x;
+            const unsigned extra = m.never_arrive == 1 || (m.never_arrive == 2 && last && blockIdx.x == gridDim.x - 1);
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(m.counter) : "memory");
             const long long t0 = clock64();
             for (int polls = 1;; ++polls) {
                 unsigned v;
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(m.counter) : "memory");
-                if (v >= target) break;
-                if ((polls & 1023) == 0) {  // another block's abort, or this wait's own bound
-                    if (clock64() - t0 > kPcgWaitClocks) atomicExch(m.counter + 1, 1u);
-                    if (*(volatile unsigned*)(m.counter + 1)) { ok = false; break; }
+                if (v >= target + extra) break;
+                if ((polls & 1023) == 0) {  // another block's giving up, or this wait's own bound
+                    if (clock64() - t0 > m.limit) atomicExch(m.gave_up, 1u);
+                    if (*(volatile unsigned*)m.gave_up) { ok = false; break; }
                 }
             }
         }
@@ -252,9 +274,7 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
     // the scalars are the last warp's: with few cells a block it has none, and forms the reciprocals of the next
     // iteration's ratios while the others update
     constexpr int kLead = NT - 32;
-    PcgOut o;
-    o.iters = o.bad = 0;
-    o.rr = o.rr0 = 0.0;
+    PcgOut o = {};
     T inv_gamma = T(0), inv_alpha = T(0);
     bool met = true;
     for (bool start = true;; start = false) {
@@ -309,9 +329,13 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
             a.u[i] = d * rn;
         });
     }
-    if (!met) o.bad = 3;
     each([&](int k, int i) { op.done(i, X(k, i)); });
-    if (blockIdx.x == 0 && tid == kLead) *a.out = o;
+    if (blockIdx.x == 0 && tid == kLead) {  // gave_up is the waits'
+        a.out->rr = o.rr;
+        a.out->rr0 = o.rr0;
+        a.out->iters = o.iters;
+        a.out->bad = o.bad;
+    }
 }
 
 // SMs of the current device
@@ -352,7 +376,7 @@ cudaError_t pcg_launch_grid(const Op& op, PcgArgs<T> a, int blocks, cudaStream_t
     if ((K > 0 && a.chunk > K * NT) || blocks > a.meet_blocks) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(a.meet_mem, 0, pcg_meet_bytes(blocks), s);
     if (e != cudaSuccess) return e;
-    a.meet = pcg_meet(a.meet_mem, blocks);
+    a.meet = pcg_meet(a.meet_mem, blocks, a.out, a.waits);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(NT);

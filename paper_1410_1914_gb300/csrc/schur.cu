@@ -544,8 +544,7 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
         CK(mem.get(&dy, m));
         double* dnorm = hv + 2 * (size_t)(m + 1);
         // z = L_D^{-1} v to cg_tol (diagonal-preconditioned CG, FP64)
-        PcgArgs<double> cg;
-        memset(&cg, 0, sizeof(cg));
+        PcgArgs<double> cg = {};
         cg.n = n;
         cg.tol2 = cg_tol * cg_tol;
         cg.max_iters = 100000;
@@ -562,6 +561,8 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
         CK(mem.get(&meet_mem, (long long)pcg_meet_bytes(cg.meet_blocks)));
         cg.meet_mem = meet_mem;
         CK(mem.get(&cg.out, 1));
+        CK(cudaMemsetAsync(cg.out, 0, sizeof(PcgOut), s));
+        cg.waits = PcgWaits(h->wait_limit, h->never_arrive);
         FvOp op;
         op.n = n;
         op.nb = d.nb;
@@ -625,11 +626,11 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
                 CK(cudaMemcpyAsync(&po, cg.out, sizeof(po), cudaMemcpyDeviceToHost, s));
                 CK(cudaMemcpyAsync(hh.data(), hv, sizeof(double) * (2 * (size_t)(j + 1) + 1), cudaMemcpyDeviceToHost, s));
                 CK(cudaStreamSynchronize(s));
-                if (po.bad == 1) { set_msg_txt("inner conjugate gradients broke down"); return CL_ERR_DIVERGED; }
-                if (po.bad == 3) {
+                if (po.gave_up) {
                     set_msg_txt("a wait of the steady solve's blocks for one another ran out");
                     return CL_ERR_TIMEOUT;
                 }
+                if (po.bad == 1) { set_msg_txt("inner conjugate gradients broke down"); return CL_ERR_DIVERGED; }
                 inf.inner_iterations += po.iters;
                 for (int k = 0; k <= j; ++k) hcol[k] = hh[k] + hh[j + 1 + k];
                 const double hn = hh[2 * (size_t)(j + 1)];
