@@ -1135,9 +1135,11 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
         CKS(sc.get((void**)&d.omega, sizeof(float) * n));
         CK(launch_dsa_number(m7, m19, N, scan, d.inv, d.list, h->s));
         CK(q19 ? launch_dsa_links19(d, a19, h->s) : launch_dsa_links7(d, a7, h->s));
-        // V (kM + 1) and Z (kM) of the GMRES cycle, w, e and c: one allocation, pads zero
+        // V (kM + 1) and Z (kM) of the GMRES cycle, w, e and c: one allocation, pads zero.  The Gram-Schmidt reads
+        // float4s (Lc is a multiple of 32), whatever the alignment of the caller's allocator.
         float* vecs = nullptr;
-        CKS(sc.get((void**)&vecs, sizeof(float) * (size_t)Lc * (2 * kM + 4)));
+        CKS(sc.get((void**)&vecs, sizeof(float) * (size_t)Lc * (2 * kM + 4) + 16));
+        vecs = (float*)(((uintptr_t)vecs + 15) & ~(uintptr_t)15);
         CK(cudaMemsetAsync(vecs, 0, sizeof(float) * (size_t)Lc * (2 * kM + 4), h->s));
         float* V = vecs;
         float* Z = V + (size_t)Lc * (kM + 1);
