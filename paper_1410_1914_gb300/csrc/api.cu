@@ -679,7 +679,10 @@ cl_status cl_lbm_create(cl_handle* out, const cl_params* p) {
         const long long NP = h->NP19;
         if (h->q19s) {
             for (int b = 0; b < 2; ++b) {
-                if ((st = dalloc_n(h, &h->st19[b].hl, NP)) != CL_OK) return fail(st);
+                // read as float4s (two cells), whatever the alignment of the caller's allocator
+                void* hl = nullptr;
+                if ((st = dalloc(h, &hl, sizeof(float2) * (size_t)NP + 16)) != CL_OK) return fail(st);
+                h->st19[b].hl = (float2*)(((uintptr_t)hl + 15) & ~(uintptr_t)15);
                 if ((st = dalloc(h, &h->st19[b].d, (size_t)h->el * 18 * NP)) != CL_OK) return fail(st);
             }
         } else {

@@ -53,3 +53,8 @@ def _same(storage, lattice, go, shape=(12, 13, 41)):
 @pytest.mark.parametrize("lattice", ["d3q7", "d3q19"])
 def test_krylov_solve_with_buffers_of_eight_byte_alignment(cuda_lib, lattice):
     _same("fp32pop", lattice, lambda s: s.solve_krylov_dsa(tol=1e-7, max_iter=400, max_steps=20))
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16dev"])
+def test_d3q19_step_with_buffers_of_eight_byte_alignment(cuda_lib, storage):
+    _same(storage, "d3q19", lambda s: s.solve_budget(40))
