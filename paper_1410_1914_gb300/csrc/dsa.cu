@@ -286,7 +286,8 @@ struct LapOp {
 // ----------------------------------------------------------- Gram-Schmidt
 // s + e += a b with the rounding errors of the product and of the sum kept
 // (Dot2 of Ogita, Rump and Oishi, SIAM J. Sci. Comput. 26 (2005) 1955): the
-// result is as if formed in twice the working precision.  FP64 runs at 1/64
+// result is as if formed in twice the working precision.  V is normalised, so
+// the products stay inside the f32 range.  FP64 runs at 1/64
 // of the FP32 rate on this GPU, and a product of two f32 in FP64 takes three
 // FP64 instructions (two conversions and the FMA).
 __device__ __forceinline__ void dot2(float a, float b, float& s, float& e) {
@@ -599,13 +600,13 @@ cudaError_t launch_dsa_add64(const DsaCells& d, const float* e, double sign, lon
 // ------------------------------------------------- vectors of one cycle's start
 namespace {
 
+// Products in FP64: these vectors are residuals in the caller's unit of concentration (any magnitude below 1e30), whose
+// squares leave the f32 range.  A few calls per correction, 14 us at 2.8 M elements.
 __global__ void __launch_bounds__(kDT) k_dot(const float* __restrict__ x, const float* __restrict__ y, long long L,
                                              double* __restrict__ part) {
-    float s = 0.f, e = 0.f;
+    double acc[1] = {0.0};
     for (long long i = blockIdx.x * (long long)kDT + threadIdx.x; i < L; i += (long long)gridDim.x * kDT)
-        dot2(x[i], y[i], s, e);
-    warp_dot2(s, e);
-    double acc[1] = {(threadIdx.x & 31) == 0 ? (double)s + (double)e : 0.0};
+        acc[0] = fma((double)x[i], (double)y[i], acc[0]);
     block_sum_store<1>(acc, part + 2 * blockIdx.x);
 }
 
