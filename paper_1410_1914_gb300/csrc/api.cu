@@ -600,6 +600,9 @@ cl_status cl_lbm_create(cl_handle* out, const cl_params* p) {
     // the population kernels switch to 64-bit element offsets once 32 bits
     // no longer hold every offset; this override takes that path on any box
     if (const char* e = getenv("CL_LBM_WIDE_INDEX")) h->wide = atoi(e) != 0;
+    // the small systems of the steady solves take one cluster where the device places it, else the grid; this override
+    // takes the grid on any device
+    if (const char* e = getenv("CL_LBM_NO_CLUSTER")) h->no_cluster = atoi(e) != 0;
     h->el = p->storage == CL_STORE_FP16DEV ? 2 : 4;
     h->s = (cudaStream_t)p->cuda_stream;
     memset(&h->info, 0, sizeof(h->info));
@@ -1165,6 +1168,7 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
         CKS(sc.get((void**)&cg.out, sizeof(PcgOut)));
         CK(cudaMemsetAsync(cg.out, 0, sizeof(PcgOut), h->s));
         cg.waits = PcgWaits(h->wait_limit, h->never_arrive);
+        cg.no_cluster = h->no_cluster;
         double *x64 = nullptr, *y64 = nullptr, *part = nullptr, *dcol = nullptr, *dnrm = nullptr, *dy = nullptr;
         KryScalars* ks = nullptr;
         CKS(sc.get((void**)&x64, sizeof(double) * (size_t)L));

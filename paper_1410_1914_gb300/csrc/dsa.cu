@@ -485,7 +485,10 @@ cudaError_t prec_q(const DsaCells& d, const float* v, float* z, const PcgArgs<fl
     const LapOp<Q> op = lap_op<Q>(d, v, z);
     const int sms = device_sms();
     const auto blocks = [&](int k) { return (d.n + k * kCgT - 1) / (k * kCgT); };
-    if (blocks(2) <= kPcgMaxCluster) return pcg_launch_cluster<float, LapOp<Q>, 2, kCgT>(op, a, blocks(2), s);
+    if (blocks(2) <= kPcgMaxCluster) {
+        const cudaError_t e = pcg_launch_cluster<float, LapOp<Q>, 2, kCgT>(op, a, blocks(2), s);
+        if (e != cudaErrorLaunchOutOfResources) return e;
+    }
     if (blocks(2) <= sms) return pcg_launch_grid<float, LapOp<Q>, 2, kCgT>(op, a, blocks(2), s);
     switch (blocks(1) <= 8 * sms ? (blocks(1) + sms - 1) / sms : 0) {  // every SM, the fewest cells per thread
         case 3: return pcg_launch_grid<float, LapOp<Q>, 3, kCgT>(op, a, sms, s);

@@ -88,6 +88,7 @@ struct PcgArgs {
     void* meet_mem;     // pcg_meet_bytes(meet_blocks)
     int meet_blocks;
     PcgWaits waits;
+    int no_cluster;  // take the grid whatever the size
     PcgOut* out;  // zeroed once per call
 };
 
@@ -346,13 +347,15 @@ inline int device_sms() {
     return nsm;
 }
 
+// cudaErrorLaunchOutOfResources, with no error left behind: the device (or the part of it that this context may use)
+// cannot place such a cluster, and the caller takes the grid.
 template <class T, class Op, int K, int NT>
 cudaError_t pcg_launch_cluster(const Op& op, PcgArgs<T> a, int blocks, cudaStream_t s) {
     a.chunk = (a.n + blocks - 1) / blocks;
     if (a.chunk > K * NT) return cudaErrorInvalidValue;
+    if (a.no_cluster) return cudaErrorLaunchOutOfResources;
     auto kern = k_pcg<T, Op, K, NT, PcgCluster>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(NT);
@@ -364,9 +367,11 @@ cudaError_t pcg_launch_cluster(const Op& op, PcgArgs<T> a, int blocks, cudaStrea
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int fit = 0;
-    e = cudaOccupancyMaxActiveClusters(&fit, kern, &cfg);
-    if (e == cudaSuccess && fit < 1) e = cudaErrorLaunchOutOfResources;
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&fit, kern, &cfg);
+    if (e != cudaSuccess || fit < 1) {
+        cudaGetLastError();
+        return cudaErrorLaunchOutOfResources;
+    }
     return cudaLaunchKernelEx(&cfg, kern, op, a);
 }
 

@@ -310,10 +310,14 @@ bool prec_streams64(int n) { return (n + kCgT64 - 1) / kCgT64 > 8 * device_sms()
 cudaError_t prec64(const FvOp& op, const PcgArgs<double>& a, cudaStream_t s) {
     const int sms = device_sms(), n = op.n;
     const auto blocks = [&](int k) { return (n + k * kCgT64 - 1) / (k * kCgT64); };
-    if (blocks(1) <= kPcgMaxCluster)
+    if (blocks(2) <= kPcgMaxCluster) {
         // the whole cluster, however few the cells
-        return pcg_launch_cluster<double, FvOp, 1, kCgT64>(op, a, std::min(kPcgMaxCluster, (n + 31) / 32), s);
-    if (blocks(2) <= kPcgMaxCluster) return pcg_launch_cluster<double, FvOp, 2, kCgT64>(op, a, kPcgMaxCluster, s);
+        const cudaError_t e =
+            blocks(1) <= kPcgMaxCluster
+                ? pcg_launch_cluster<double, FvOp, 1, kCgT64>(op, a, std::min(kPcgMaxCluster, (n + 31) / 32), s)
+                : pcg_launch_cluster<double, FvOp, 2, kCgT64>(op, a, kPcgMaxCluster, s);
+        if (e != cudaErrorLaunchOutOfResources) return e;
+    }
     if (blocks(1) <= sms) return pcg_launch_grid<double, FvOp, 1, kCgT64>(op, a, std::min(sms, (n + 63) / 64), s);
     switch (blocks(1) <= 8 * sms ? (blocks(1) + sms - 1) / sms : 0) {
         case 2: return pcg_launch_grid<double, FvOp, 2, kCgT64>(op, a, sms, s);
@@ -563,6 +567,7 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
         CK(mem.get(&cg.out, 1));
         CK(cudaMemsetAsync(cg.out, 0, sizeof(PcgOut), s));
         cg.waits = PcgWaits(h->wait_limit, h->never_arrive);
+        cg.no_cluster = h->no_cluster;
         FvOp op;
         op.n = n;
         op.nb = d.nb;
