@@ -16,6 +16,7 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <stdlib.h>
 
 #include <mutex>
 
@@ -326,14 +327,14 @@ static bool vec8(const void* p, int C, int stride, int off) {
 
 static cudaError_t launch_bias_grad(const __nv_bfloat16* dout, long long M, int C, int stride, int off, float* db,
                                     cudaStream_t s) {
-    // at least two voxels per thread of the cluster (27,648 voxels: 3 us, 8 with one block per channel); fewer take
-    // one block per channel 2 to 6 us
-    if (C < 8 || M < 2 * kBgRanks * kBgThreads || !vec8(dout, C, stride, off)) {
+    const auto per_channel = [&] {
         k_bias_grad<<<C, 256, 0, s>>>(dout, M, stride, off, db);
         return cudaGetLastError();
-    }
+    };
+    // at least two voxels per thread of the cluster (27,648 voxels: 3 us, 8 with one block per channel); fewer take
+    // one block per channel 2 to 6 us
+    if (C < 8 || M < 2 * kBgRanks * kBgThreads || !vec8(dout, C, stride, off)) return per_channel();
     cudaError_t e = cudaFuncSetAttribute(k_bias_grad8, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kBgRanks, C / 8);
     cfg.blockDim = dim3(kBgThreads);
@@ -344,6 +345,13 @@ static cudaError_t launch_bias_grad(const __nv_bfloat16* dout, long long M, int 
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
+    int fit = 0;
+    const char* off_env = getenv("CL_LBM_NO_CLUSTER");  // the way of a device that places no such cluster, on any device
+    if (e == cudaSuccess && !(off_env && atoi(off_env))) e = cudaOccupancyMaxActiveClusters(&fit, k_bias_grad8, &cfg);
+    if (e != cudaSuccess || fit < 1) {
+        cudaGetLastError();
+        return per_channel();
+    }
     return cudaLaunchKernelEx(&cfg, k_bias_grad8, dout, M, stride, off, db);
 }
 

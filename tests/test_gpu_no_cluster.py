@@ -1,6 +1,7 @@
-"""The steady solves of small systems where no cluster of their size can be
-placed: CL_LBM_NO_CLUSTER=1 takes the grid's route at every size, which must
-reach what the cluster's reaches."""
+"""Calls that take a cluster of 16 blocks, where no such cluster can be placed
+(CL_LBM_NO_CLUSTER=1 takes that way on any device): the steady solves of small
+systems on the grid must reach what the cluster's route reaches, and the bias
+gradient is summed by one block per channel."""
 import numpy as np
 import pytest
 
@@ -36,3 +37,16 @@ def test_small_systems_on_the_grid(cuda_lib, monkeypatch, kind, lattice, edge):
     else:               # residuals of 1e-10: fields to the rounding of f32
         assert abs(a[0] - b[0]) <= 2
         np.testing.assert_allclose(a[2], b[2], rtol=0, atol=4 * 6e-8)
+
+
+def test_bias_gradient_without_a_cluster(cuda_lib, monkeypatch):
+    import torch
+
+    from paper_1410_1914_gb300 import warmstart as W
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    dy = torch.randint(-3, 4, (20000, 24), device="cuda", generator=gen).to(torch.bfloat16)
+    db = torch.full((16,), 7.0, device="cuda")
+    monkeypatch.setenv("CL_LBM_NO_CLUSTER", "1")
+    W._call("cl_nn_bias_grad", W._p(dy), 20000, 16, 24, 8, W._p(db), None)
+    torch.cuda.synchronize()
+    assert torch.equal(db.double(), dy[:, 8:].double().sum(0))   # whole numbers below 2^24: exact in any order
