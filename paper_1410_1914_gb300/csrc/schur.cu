@@ -342,6 +342,22 @@ __global__ void __launch_bounds__(kSB) k_mdot(const double* __restrict__ V, int 
     block_sum_store<1>(acc, part + (long long)blockIdx.y * gridDim.x + blockIdx.x);
 }
 
+// part[0][j] += the other chunks' parts, in order: one thread per vector, its loads in flight together
+__global__ void __launch_bounds__(32) k_mdot_sum(double* __restrict__ part, int m, int chunks) {
+    const int j = blockIdx.x * 32 + threadIdx.x;
+    if (j >= m) return;
+    double h = part[j];
+#pragma unroll 8
+    for (int k = 1; k < chunks; ++k) h += part[(long long)k * m + j];
+    part[j] = h;
+}
+
+// Up to this many chunks every block of k_msub adds them up itself, which saves a launch; beyond, blocks times chunks
+// grows as the square of the cells.  Added up once, 60 iterations from the start (Pt layers, ms an iteration): 29 k
+// cells 0.395 (four chunks, by every block), 50 k 0.581 to 0.551, 118 k 1.10 to 0.90, 943 k 19.4 to 6.9, 1.84 M 61.3
+// to 13.8.
+constexpr int kFoldChunks = 4;
+
 // w -= sum_j h[j] V_j with h[j] = sum over chunks of part[chunk][j]: blocks of 32 cells, the vectors shared out over
 // 8 warps.  hout gets h (block 0); nrm (nullable): this block's part of |w|^2.
 __global__ void __launch_bounds__(kSB) k_msub(const double* __restrict__ V, int n, int m, int chunks,
@@ -620,8 +636,9 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
                 // classical Gram-Schmidt, twice; |w| and the next vector
                 for (int pass = 0; pass < 2; ++pass) {
                     k_mdot<<<dim3(j + 1, chunks), kSB, 0, s>>>(V, n, w, part);
-                    k_msub<<<parts, kSB, 0, s>>>(V, n, j + 1, chunks, part, w, hv + (size_t)pass * (j + 1),
-                                                 pass ? nrm : nullptr);
+                    if (chunks > kFoldChunks) k_mdot_sum<<<(j + 32) / 32, 32, 0, s>>>(part, j + 1, chunks);
+                    k_msub<<<parts, kSB, 0, s>>>(V, n, j + 1, chunks > kFoldChunks ? 1 : chunks, part, w,
+                                                 hv + (size_t)pass * (j + 1), pass ? nrm : nullptr);
                 }
                 double* hn_dev = hv + 2 * (size_t)(j + 1);
                 k_norm_fin<<<1, kSB, 0, s>>>(nrm, parts, hn_dev);
