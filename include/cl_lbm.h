@@ -340,9 +340,11 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
      tol:      stop when |F(C) - C| falls to tol times |F(0)| (the right-hand
                side; a warm start close to the answer stops at once).
      max_iter: GMRES iterations (applications of F) in all.
-     restart:  Krylov vectors kept; the call allocates 2 * restart + 8
-               FP64 cell fields (restart 1000 at 32^3: 0.5 GB), freed
-               before returning.
+     restart:  Krylov vectors kept; the call allocates, per active cell, 2 *
+               restart + 28 FP64 values (five more above 300 k active cells
+               or with restart < 4), seven more per run of open faces along
+               an axis, and half a value per cell of the box (restart 1000
+               at 32^3, porosity 0.45: 0.24 GB), freed before returning.
      cg_tol:   relative residual of each preconditioner solve, in (0, 1);
                1e-3 is enough (at 24^3 and 33x33x32 the outer count is the
                same as with 1e-10, the inner work less than half).

@@ -68,10 +68,11 @@ struct SchurArgs {
     double* om64;   // [n] omega in FP64
     double* G;      // [6][n] conductance of each link (0 where closed)
     double* dinv;   // [n] 1 / diagonal of the finite-volume operator
-    Run* runs;      // [3][n]
+    Run* runs;      // by axis, from run_base on
+    long long run_base[3];
     int* ord;       // [3][n] the cells of each axis run by run, and
     double2* dso;   // [3][n] their 1 - omega and omega w
-    int* n_runs;    // [3] runs, then [3] cells listed
+    int* n_runs;    // [3] runs, then [3] cells listed, then [3] cells that may start one
 };
 
 __device__ __forceinline__ double cat_factor(const SchurArgs& a, int c) {
@@ -119,6 +120,27 @@ __device__ __forceinline__ void end_rule(const SchurArgs& a, int to, bool minus,
     }
 }
 
+// whether cell i may start a run of axis ax: its - face is closed, or it is the cell of coordinate 0 of a y or z line
+__device__ __forceinline__ bool may_start(const SchurArgs& a, int ax, int i) {
+    if (a.nb[(long long)(2 * ax + 1) * a.n + i] < 0) return true;
+    if (ax == 0) return false;
+    const int c = a.list[i];
+    return (ax == 1 ? (c / a.nx) % a.ny : c / (a.nx * a.ny)) == 0;
+}
+
+// how many runs there can be, which the allocation follows: a few per hundred cells in open boxes
+__global__ void __launch_bounds__(kSB) k_schur_count(SchurArgs a) {
+    int cnt[3] = {0, 0, 0};
+    for (int i = blockIdx.x * kSB + threadIdx.x; i < a.n; i += gridDim.x * kSB)
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) cnt[ax] += may_start(a, ax, i);
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        const int t = __reduce_add_sync(0xffffffffu, cnt[ax]);
+        if ((threadIdx.x & 31) == 0 && t) atomicAdd(a.n_runs + 6 + ax, t);
+    }
+}
+
 // The runs of axis blockIdx.y, in any order (runs do not share cells): each cell whose - face is closed starts one;
 // a y or z line without a closed face is a loop, recorded by its cell of coordinate 0.
 __global__ void __launch_bounds__(kSB) k_schur_runs(SchurArgs a) {
@@ -126,13 +148,9 @@ __global__ void __launch_bounds__(kSB) k_schur_runs(SchurArgs a) {
     const int* __restrict__ fwd = a.nb + (long long)(2 * ax) * a.n;
     const int* __restrict__ bwd = a.nb + (long long)(2 * ax + 1) * a.n;
     for (int i = blockIdx.x * kSB + threadIdx.x; i < a.n; i += gridDim.x * kSB) {
+        if (!may_start(a, ax, i)) continue;
         Run r;
         const bool start = bwd[i] < 0;
-        if (!start) {
-            if (ax == 0) continue;
-            const int c = a.list[i];
-            if ((ax == 1 ? (c / a.nx) % a.ny : c / (a.nx * a.ny)) != 0) continue;
-        }
         int len = 1, last = i, t = fwd[i];
         r.al = 1.0 - a.om64[i];
         for (; t >= 0 && t != i; t = fwd[t]) {
@@ -157,7 +175,7 @@ __global__ void __launch_bounds__(kSB) k_schur_runs(SchurArgs a) {
             a.ord[at + k] = u;
             a.dso[at + k] = make_double2(1.0 - a.om64[u], a.om64[u] * kWa);
         }
-        a.runs[(long long)ax * a.n + atomicAdd(a.n_runs + ax, 1)] = r;
+        a.runs[a.run_base[ax] + atomicAdd(a.n_runs + ax, 1)] = r;
     }
 }
 
@@ -180,7 +198,7 @@ __global__ void __launch_bounds__(kWalkT) k_walk(SchurArgs a, const double* __re
     const int nr = a.n_runs[ax];
     const bool src = !homog && a.src;
     for (int q = blockIdx.x * kWalkT + threadIdx.x; q < nr; q += gridDim.x * kWalkT) {
-        const Run r = a.runs[(long long)ax * n + q];
+        const Run r = a.runs[a.run_base[ax] + q];
         const bool loop = r.len < 0;
         const int len = loop ? -r.len : r.len;
         const int* __restrict__ ord = a.ord + (long long)ax * n + r.pos;
@@ -536,18 +554,23 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
         CK(mem.get(&a.om64, n));
         CK(mem.get(&a.G, 6LL * n));
         CK(mem.get(&a.dinv, n));
-        CK(mem.get(&a.runs, 3LL * n));
         CK(mem.get(&a.ord, 3LL * n));
         CK(mem.get(&a.dso, 3LL * n));
-        CK(mem.get(&a.n_runs, 6));
-        CK(cudaMemsetAsync(a.n_runs, 0, 6 * sizeof(int), s));
+        CK(mem.get(&a.n_runs, 9));
+        CK(cudaMemsetAsync(a.n_runs, 0, 9 * sizeof(int), s));
         const int nb = std::min((n + kSB - 1) / kSB, 152 * 8);
+        k_schur_count<<<nb, kSB, 0, s>>>(a);
         k_schur_setup<<<nb, kSB, 0, s>>>(a);
+        CK(cudaGetLastError());
+        int n_runs[3];  // at most
+        CK(cudaMemcpyAsync(n_runs, a.n_runs + 6, sizeof(n_runs), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        a.run_base[0] = 0;
+        a.run_base[1] = n_runs[0];
+        a.run_base[2] = (long long)n_runs[0] + n_runs[1];
+        CK(mem.get(&a.runs, (long long)n_runs[0] + n_runs[1] + n_runs[2]));
         k_schur_runs<<<dim3(nb, 3), kSB, 0, s>>>(a);
         CK(cudaGetLastError());
-        int n_runs[3];
-        CK(cudaMemcpyAsync(n_runs, a.n_runs, sizeof(n_runs), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
         const int most_runs = std::max(1, std::max(n_runs[0], std::max(n_runs[1], n_runs[2])));
         const dim3 walk_grid(std::min((most_runs + kWalkT - 1) / kWalkT, 152 * 64), 3);
         double *V = nullptr, *Z = nullptr, *x = nullptr, *w = nullptr, *T = nullptr, *part = nullptr, *nrm = nullptr;
@@ -698,8 +721,8 @@ extern "C" cl_status cl_lbm_solve_steady_lines(cl_handle h, double tol, int max_
             if (rn <= tol * r0) result = CL_OK;
         }
         // the state: post-collision populations of the steady field, and its fluxes in FP64
-        double* flux = nullptr;
-        CK(mem.get(&flux, 5LL * n));
+        double* flux = V;  // the basis is done with
+        if (m < 4) CK(mem.get(&flux, 5LL * n));
         CK(cudaMemsetAsync(flux, 0, sizeof(double) * 5 * (size_t)n, s));
         k_walk<true><<<walk_grid, kWalkT, 0, s>>>(a, x, T, 0, h->pop[h->cur], N, flux);
         k_walk_fin<true><<<nb, kSB, 0, s>>>(a, x, T, 0, 0, w, h->pop[h->cur]);
