@@ -910,7 +910,7 @@ struct PopPlaneOp {
         const float* h = t.h;
         const float C = ((h[0] + h[1]) + (h[2] + h[3])) + ((h[4] + h[5]) + h[6]);
         if (a.src) acc.v[0] += (double)C - a.src[t.c];  // the concentration before the last collision's source
-        else acc.add_c(C, 0.f);
+        else f3_add(acc.c, C);
         acc.n += 1;
         const unsigned rb = (t.m >> kReactShift) & 0x3fu;
         if (!rb) return;
@@ -922,7 +922,7 @@ struct PopPlaneOp {
         } else {
 #pragma unroll
             for (int d = 0; d < 6; ++d)
-                if (rb & (1u << d)) acc.add_r(t.h[d + 1], 0.f);
+                if (rb & (1u << d)) f3_add(acc.r, t.h[d + 1]);
         }
     }
     __device__ __forceinline__ double inflow(int row) const {

@@ -116,11 +116,6 @@ struct StoreF16 {
 };
 
 // s + e = a + b exactly (Knuth)
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
 
 // p += hi + lo, p.y keeping what the additions to p.x lose
 __device__ __forceinline__ void pair_add(float2& p, float hi, float lo) {
@@ -1031,7 +1026,8 @@ struct StatePlaneOp {
     }
     __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
         if (!(t.m & kActiveBit)) return;
-        acc.add_c(t.hi, t.lo);
+        f3_add(acc.c, t.hi);
+        f3_add(acc.c, t.lo);
         acc.n += 1;
         const unsigned rb = (t.m >> kReactShift) & 0x3fu;
         if (rb) {
@@ -1041,8 +1037,9 @@ struct StatePlaneOp {
 #pragma unroll
             for (int i = 0; i < 6; ++i)
                 if (rb & (1u << i)) {  // w C + d: the weight is a power of two
-                    acc.add_r(kW1 * t.hi, kW1 * t.lo);
-                    acc.add_r(dv[i], 0.f);
+                    f3_add(acc.r, kW1 * t.hi);
+                    f3_add(acc.r, kW1 * t.lo);
+                    f3_add(acc.r, dv[i]);
                 }
         }
     }

@@ -7,13 +7,14 @@
 // read as they lie, a block sums a share of the rows, and a second kernel
 // adds the shares in order (the sums repeat bit by bit).
 //
-// FP64 issues at 1/64 of the FP32 rate, so the sums over a share's rows run in pairs
-// of floats with the rounding errors kept (two-sum; as good as 46 bits) that are
-// added in FP64 once per kPlaneFlush rows.
+// FP64 issues at 1/64 of the FP32 rate, so the sums over a share's rows run in triples
+// of floats (F3) that are added in FP64 once per kPlaneFlush rows.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include "device_util.cuh"
 
 namespace cl {
 
@@ -21,23 +22,15 @@ constexpr int kPlaneFlush = 16;
 
 struct PlaneAcc {
     double v[5];
-    float cs, ce;  // running sum of C and what its roundings lost
-    float rs, re;  // the same for the consumption, before the sink's factor
+    F3 c;  // running sum of C
+    F3 r;  // of the consumption, before the sink's factor
     unsigned n;
-    static __device__ __forceinline__ void add(float& s, float& e, float hi, float lo) {
-        const float t = __fadd_rn(s, hi);
-        const float z = __fsub_rn(t, s);
-        e = __fadd_rn(e, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(hi, z)), lo));
-        s = t;
-    }
-    __device__ __forceinline__ void add_c(float hi, float lo) { add(cs, ce, hi, lo); }
-    __device__ __forceinline__ void add_r(float hi, float lo) { add(rs, re, hi, lo); }
 };
 
 // Op: load(x, row) reads what a cell needs, without a condition, so that kRows rows are in flight; use(item, acc)
 // adds it.  inflow(row), outflow(row): the parts of the planes x = 0 and x = L, summed with one row per thread: as a
 // condition among the rows their FP64 instructions were predicated off but issued in every one, and were the time of
-// the kernel.  sink(): the factor of the consumption gathered in add_r.
+// the kernel.  sink(): the factor of the consumption gathered in PlaneAcc::r.
 template <class Op>
 __global__ void __launch_bounds__(256) k_plane_part(Op op, int nx, int rows, int share, double* __restrict__ part) {
     __shared__ double sh[8][5][32];
@@ -53,7 +46,7 @@ __global__ void __launch_bounds__(256) k_plane_part(Op op, int nx, int rows, int
     constexpr int U = Op::kRows;
     static_assert(kPlaneFlush % U == 0, "whole groups of rows between flushes");
     for (int b = r0 + warp; b < r1; b += 8 * kPlaneFlush) {
-        a.cs = a.ce = a.rs = a.re = 0.f;
+        a.c = a.r = F3{0.f, 0.f, 0.f};
         if (x < nx)
             for (int g = 0; g < kPlaneFlush && b + 8 * g < r1; g += U) {
                 typename Op::Item it[U];
@@ -63,9 +56,8 @@ __global__ void __launch_bounds__(256) k_plane_part(Op op, int nx, int rows, int
                 for (int u = 0; u < U; ++u)
                     if (b + 8 * (g + u) < r1) op.use(it[u], a);
             }
-        // past an overflow the errors are inf - inf: the sum alone then says what happened
-        a.v[0] += (double)a.cs + (isfinite(a.ce) ? (double)a.ce : 0.0);
-        if (__any_sync(0xffffffffu, a.rs != 0.f)) a.v[2] += sink * ((double)a.rs + (isfinite(a.re) ? (double)a.re : 0.0));
+        a.v[0] += f3_get(a.c);
+        if (__any_sync(0xffffffffu, a.r.a != 0.f || a.r.b != 0.f)) a.v[2] += sink * f3_get(a.r);
     }
     a.v[1] += (double)a.n;
     if (threadIdx.x < 2) edge[threadIdx.x] = 0.0;

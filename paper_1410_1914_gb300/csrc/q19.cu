@@ -336,13 +336,13 @@ struct Pop19PlaneOp {
     __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
         if (!(t.m & kQ19Active)) return;
 #pragma unroll
-        for (int i = 0; i < 19; ++i) acc.add_c(t.h[i], 0.f);
+        for (int i = 0; i < 19; ++i) f3_add(acc.c, t.h[i]);
         acc.n += 1;
         if (!(t.m & kQ19HasReact)) return;
         const uint32_t rb = a.react[t.c];
 #pragma unroll
         for (int i = 1; i < 19; ++i)
-            if (rb & (1u << (i - 1))) acc.add_r(t.h[i], 0.f);
+            if (rb & (1u << (i - 1))) f3_add(acc.r, t.h[i]);
     }
     __device__ __forceinline__ double inflow(int row) const {
         const long long c = (long long)a.px * row;

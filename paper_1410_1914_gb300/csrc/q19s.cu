@@ -408,14 +408,16 @@ struct State19PlaneOp {
     }
     __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
         if (!(t.m & kQ19Active)) return;
-        acc.add_c(t.hl.x, t.hl.y);
+        f3_add(acc.c, t.hl.x);
+        f3_add(acc.c, t.hl.y);
         acc.n += 1;
         if (!(t.m & kQ19HasReact)) return;
         for (unsigned left = a.react[t.p]; left; left &= left - 1) {  // g*_i = a_i C + d_i of the catalytic links
             const int i = __ffs(left);
-            const float w = s19_w(i), h = w * t.hl.x;
-            acc.add_r(h, fmaf(w, t.hl.x, -h) + w * t.hl.y);
-            acc.add_r(d(i, t.p), 0.f);
+            const float w = s19_w(i);
+            f3_add_product(acc.r, w, t.hl.x);
+            f3_add_product(acc.r, w, t.hl.y);
+            f3_add(acc.r, d(i, t.p));
         }
     }
     // 2 (a_i C_bc - g*_i) over the open links through the plane (sgn -1: x = 0, which take in; +1: x = L)
