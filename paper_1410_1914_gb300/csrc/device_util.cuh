@@ -58,16 +58,22 @@ __device__ __forceinline__ void f3_add(F3& s, float x) {
     two_sum(s.b, e, s.b, e);
     s.c = __fadd_rn(s.c, e);
 }
+// a term that is small beside the others (the low word of one), as exact for half the instructions
+__device__ __forceinline__ void f3_add_low(F3& s, float x) {
+    float e;
+    two_sum(s.b, x, s.b, e);
+    s.c = __fadd_rn(s.c, e);
+}
 __device__ __forceinline__ void f3_add(F3& s, const F3& o) {
     f3_add(s, o.a);
-    f3_add(s, o.b);
+    f3_add_low(s, o.b);
     s.c = __fadd_rn(s.c, o.c);
 }
 // w v, the rounding error of the product included
 __device__ __forceinline__ void f3_add_product(F3& s, float w, float v) {
     const float p = __fmul_rn(w, v);
     f3_add(s, p);
-    f3_add(s, __fmaf_rn(w, v, -p));
+    f3_add_low(s, __fmaf_rn(w, v, -p));
 }
 // the sum in FP64; past an overflow the errors are inf - inf, and the sum alone says what happened
 __device__ __forceinline__ double f3_get(const F3& s) {

@@ -115,16 +115,6 @@ struct StoreF16 {
     static __device__ __forceinline__ T st(float v, float s) { return __float2half_rn(v * s); }
 };
 
-// s + e = a + b exactly (Knuth)
-
-// p += hi + lo, p.y keeping what the additions to p.x lose
-__device__ __forceinline__ void pair_add(float2& p, float hi, float lo) {
-    const float t = __fadd_rn(p.x, hi);
-    const float z = __fsub_rn(t, p.x);
-    p.y = __fadd_rn(p.y, __fadd_rn(__fadd_rn(__fsub_rn(p.x, __fsub_rn(t, z)), __fsub_rn(hi, z)), lo));
-    p.x = t;
-}
-
 // ------------------------------------------------------- shared layout
 template <class S, int RW>
 struct SlotLayout {
@@ -225,7 +215,7 @@ template <class S, bool REDUCE>
 __device__ __forceinline__ void pair_update(const MarchArgs& a, uint32_t ma, uint32_t mb, F2 om, F2 hx, F2 lxs,
                                             const F2 (&dds)[6], const F2 (&nh)[6], const F2 (&nls)[6],
                                             const F2 (&nds)[6], int x, F2& hnew, F2& lnew_s, F2 (&dns)[6],
-                                            float2 (&rp)[3], float (&rs)[4], float2& csnap) {
+                                            F3 (&rp)[3], float (&rs)[4], float2& csnap) {
     constexpr bool HALF = sizeof(typename S::T) == 2;
     const float s_lo = HALF ? a.s_lo : 1.0f, s_d = HALF ? a.s_d : 1.0f, inv_d = HALF ? a.inv_d : 1.0f;
     const F2 inv_lo2 = f2(a.inv_lo, a.inv_lo);  // FP16 state
@@ -283,8 +273,8 @@ __device__ __forceinline__ void pair_update(const MarchArgs& a, uint32_t ma, uin
     for (int i = 0; i < 6; ++i) dns[i] = f2_fma(om1, av[i], mt);  // (1 - omega)(a_i - w dC)
     if (REDUCE) {
         // Fluxes and reaction (boundary and catalytic cells only: the stopping rule resolves their changes
-        // down to 1e-9) in pairs of floats with the rounding errors kept, summed in FP64 by the block; the
-        // per-cell diagnostics in per-thread FP32 partials.  In FP64 these conditions were predicated off in
+        // down to 1e-9) in triples of floats (F3; every term is exact, w and the scales are powers of two),
+        // summed in FP64 by the block; the per-cell diagnostics in per-thread FP32 partials.  In FP64 these conditions were predicated off in
         // most lanes but issued in every one, at 1/64 of the FP32 rate: the reducing step took 0.40 ms at
         // 256^3 and 2.7 ms on the 400^3 NPMC layer, against 0.12 and 0.44 ms of a plain one.
         const float2 hn = f2_get(hnew), ln = f2_get(lnew);
@@ -303,21 +293,26 @@ __device__ __forceinline__ void pair_update(const MarchArgs& a, uint32_t ma, uin
             float s, err;
             if (k == 0 && in_a && a.bc_in == CL_BC_DIRICHLET) {
                 two_sum(a.c_in, -hk, s, err);
-                pair_add(rp[0], 2.0f * w * s, 2.0f * w * (err - lk));
-                pair_add(rp[0], -2.0f * dev(1), 0.f);
+                f3_add(rp[0], 2.0f * w * s);
+                f3_add_low(rp[0], 2.0f * w * err);
+                f3_add_low(rp[0], -2.0f * w * lk);
+                f3_add(rp[0], -2.0f * dev(1));
             }
             if ((k == 0 ? out_a : out_b) && a.bc_out == CL_BC_DIRICHLET) {
                 two_sum(hk, -a.c_out, s, err);
-                pair_add(rp[1], 2.0f * w * s, 2.0f * w * (err + lk));
-                pair_add(rp[1], 2.0f * dev(0), 0.f);
+                f3_add(rp[1], 2.0f * w * s);
+                f3_add_low(rp[1], 2.0f * w * err);
+                f3_add_low(rp[1], 2.0f * w * lk);
+                f3_add(rp[1], 2.0f * dev(0));
             }
             const unsigned rb = ((k == 0 ? ma : mb) >> kReactShift) & 0x3fu;
             if (rb) {
 #pragma unroll
                 for (int q = 0; q < 6; ++q)
-                    if (rb & (1u << q)) {  // w C + delta, the weight a power of two
-                        pair_add(rp[2], w * hk, w * lk);
-                        pair_add(rp[2], dev(q), 0.f);
+                    if (rb & (1u << q)) {  // w C + delta
+                        f3_add(rp[2], w * hk);
+                        f3_add_low(rp[2], w * lk);
+                        f3_add(rp[2], dev(q));
                     }
             }
             const float Cf = hk + lk;  // the f32 rounding of the double-float C
@@ -441,9 +436,9 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
     }
     // ---------------------------------------------------------- consumers
     float rs[4] = {0.f, 0.f, 0.f, 0.f};  // FP32 partials of sum C, sum |dC|, sum |C|, non-finite
-    float2 rp[3];                        // J_in, J_out, and R before the sink's factor
+    F3 rp[3];                            // J_in, J_out, and R before the sink's factor
 #pragma unroll
-    for (int i = 0; i < 3; ++i) rp[i] = make_float2(0.f, 0.f);
+    for (int i = 0; i < 3; ++i) rp[i] = F3{0.f, 0.f, 0.f};
     const int xl = tx & (LPR - 1);        // lane within its tile row
     const int row = ty * RW + tx / LPR;   // tile row of this lane
     const int xa = x0 + 2 * xl;  // this lane's cells: xa, xa + 1
@@ -563,9 +558,9 @@ __device__ __forceinline__ bool march_item(const MarchMaps* maps, const MarchArg
     }
     if (ok) release(nplanes - 1);  // plane ze, read only as a z+1 neighbour
     if (REDUCE) {
-        rv[RED_JIN] += (double)rp[0].x + (double)rp[0].y;
-        rv[RED_JOUT] += (double)rp[1].x + (double)rp[1].y;
-        rv[RED_R] += a.rsink_d * ((double)rp[2].x + (double)rp[2].y);
+        rv[RED_JIN] += f3_get(rp[0]);
+        rv[RED_JOUT] += f3_get(rp[1]);
+        rv[RED_R] += a.rsink_d * f3_get(rp[2]);
         rv[RED_SUMC] += (double)rs[0];
         rv[RED_DC] += (double)rs[1];
         rv[RED_ABSC] += (double)rs[2];
@@ -1027,7 +1022,7 @@ struct StatePlaneOp {
     __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
         if (!(t.m & kActiveBit)) return;
         f3_add(acc.c, t.hi);
-        f3_add(acc.c, t.lo);
+        f3_add_low(acc.c, t.lo);
         acc.n += 1;
         const unsigned rb = (t.m >> kReactShift) & 0x3fu;
         if (rb) {
@@ -1038,7 +1033,7 @@ struct StatePlaneOp {
             for (int i = 0; i < 6; ++i)
                 if (rb & (1u << i)) {  // w C + d: the weight is a power of two
                     f3_add(acc.r, kW1 * t.hi);
-                    f3_add(acc.r, kW1 * t.lo);
+                    f3_add_low(acc.r, kW1 * t.lo);
                     f3_add(acc.r, dv[i]);
                 }
         }

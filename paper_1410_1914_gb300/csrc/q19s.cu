@@ -409,7 +409,7 @@ struct State19PlaneOp {
     __device__ __forceinline__ void use(const Item& t, PlaneAcc& acc) const {
         if (!(t.m & kQ19Active)) return;
         f3_add(acc.c, t.hl.x);
-        f3_add(acc.c, t.hl.y);
+        f3_add_low(acc.c, t.hl.y);
         acc.n += 1;
         if (!(t.m & kQ19HasReact)) return;
         for (unsigned left = a.react[t.p]; left; left &= left - 1) {  // g*_i = a_i C + d_i of the catalytic links
