@@ -187,6 +187,12 @@ Q19Args make_args19(cl_lbm* h) {
     a.c_out = (float)h->p.c_out;
     a.c_in_d = h->p.c_in;
     a.c_out_d = h->p.c_out;
+    const auto rest = [](double c) {
+        const double d = c - (double)(float)c;
+        return make_float2((float)d, (float)(d - (double)(float)d));
+    };
+    a.c_in_rest = rest(h->p.c_in);
+    a.c_out_rest = rest(h->p.c_out);
     a.bc_in = h->p.bc_in;
     a.bc_out = h->p.bc_out;
     a.Csnap = h->Csnap;

@@ -75,6 +75,12 @@ __device__ __forceinline__ void f3_add_product(F3& s, float w, float v) {
     f3_add(s, p);
     f3_add_low(s, __fmaf_rn(w, v, -p));
 }
+// the same for a small term v
+__device__ __forceinline__ void f3_add_product_low(F3& s, float w, float v) {
+    const float p = __fmul_rn(w, v);
+    f3_add_low(s, p);
+    s.c = __fadd_rn(s.c, __fmaf_rn(w, v, -p));
+}
 // the sum in FP64; past an overflow the errors are inf - inf, and the sum alone says what happened
 __device__ __forceinline__ double f3_get(const F3& s) {
     const double lost = (double)s.b + (double)s.c;

@@ -75,6 +75,7 @@ struct Q19Args {
     double rsink_d;
     float c_in, c_out;
     double c_in_d, c_out_d;
+    float2 c_in_rest, c_out_rest;  // c_in_d - c_in as two floats, the first the larger (reducing step)
     int bc_in, bc_out;
     float* Csnap;         // padded (reduction)
     double* partials;     // [blocks][RED_N] (reduction)

@@ -47,6 +47,13 @@ __host__ __device__ constexpr int s19_link(int cx, int cy, int cz) {
         if (s19_cx(i) == cx && s19_cy(i) == cy && s19_cz(i) == cz) return i;
     return 0;
 }
+// bits i - 1 of the links whose x component is cx
+__host__ __device__ constexpr uint32_t s19_links(int cx) {
+    uint32_t m = 0;
+    for (int i = 1; i < 19; ++i)
+        if (s19_cx(i) == cx) m |= 1u << (i - 1);
+    return m;
+}
 __host__ __device__ constexpr float s19_w(int i) {
     return i == 0 ? 1.f / 3.f : (i <= 6 ? 1.f / 18.f : 1.f / 36.f);
 }
@@ -70,17 +77,10 @@ __device__ __forceinline__ I dev_at(I c) {
     return (c >> 5) * (I)(18 * 32) + (c & (I)31);
 }
 
-// s + e = a + b exactly (Knuth's two-sum)
-__device__ __forceinline__ void two_sum19(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
 // (hi, lo) + d, renormalised
 __device__ __forceinline__ void df_add19(float hi, float lo, float d, float& ho, float& lo_out) {
     float s, e;
-    two_sum19(hi, d, s, e);
+    two_sum(hi, d, s, e);
     e += lo;
     ho = s + e;
     lo_out = e - (ho - s);
@@ -103,9 +103,11 @@ __device__ __forceinline__ void df_add19(float hi, float lo, float d, float& ho,
 // Bound by issue and by the latency of the loads: 128^3 Pt layer, FP16 state,
 // 78 us a step with a cell per lane and plane-by-plane deviations, 49 us;
 // FP32 state 72, 56 us.
-// The reducing step keeps its sums in floats -- pairs of them (hi, lo) for the
-// fluxes and the reaction -- down to the warp and in FP64 from there: one FP64
-// lane per cell took 515 us at 128^3, 75 us now.
+// The reducing step keeps its sums in triples of floats (F3) down to the warp
+// and in FP64 from there: one FP64 lane per cell took 515 us at 128^3 (FP16
+// state), 87 us now; the same sums in pairs of floats and f32 took 75 us, with
+// the residual off by 1e-9.  Four blocks on an SM: its 139 registers left three
+// (100 us).
 constexpr int kS19T = 128;
 constexpr int kS19Cells = 2 * kS19T;
 
@@ -124,14 +126,6 @@ __device__ __forceinline__ void st_pair(__half* p, float a, float b) {
     *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b);
 }
 
-// p += hi + lo, p.y keeping what the additions to p.x lose
-__device__ __forceinline__ void pair_add19(float2& p, float hi, float lo) {
-    float s, e;
-    two_sum19(p.x, hi, s, e);
-    p.x = s;
-    p.y = __fadd_rn(p.y, __fadd_rn(e, lo));
-}
-
 // w (hi + lo) as a pair
 __device__ __forceinline__ float2 scaled19(float w, float hi, float lo) {
     const float h = __fmul_rn(w, hi);
@@ -139,7 +133,7 @@ __device__ __forceinline__ float2 scaled19(float w, float hi, float lo) {
 }
 
 template <class S, bool REDUCE, int LX, class I>  // LX lanes to a row
-__global__ void __launch_bounds__(kS19T) k_step19s(Q19State src, Q19State dst, Q19Args a) {
+__global__ void __launch_bounds__(kS19T, REDUCE ? 4 : 0) k_step19s(Q19State src, Q19State dst, Q19Args a) {
     using T = typename S::T;
     constexpr bool HALF = sizeof(T) == 2;
     const int x = (blockIdx.x * LX + threadIdx.x % LX) * 2;
@@ -159,10 +153,10 @@ __global__ void __launch_bounds__(kS19T) k_step19s(Q19State src, Q19State dst, Q
     const float s_d = HALF ? a.s_d : 1.f, inv_d = HALF ? a.inv_d : 1.f;
     const float2* __restrict__ shl = src.hl;
     const T* __restrict__ sd = reinterpret_cast<const T*>(src.d);
-    float2 rp[3];                        // J_in, J_out, and R before the sink's factor
-    float rs[4] = {0.f, 0.f, 0.f, 0.f};  // sum C, sum |dC|, sum |C|, non-finite
-#pragma unroll
-    for (int i = 0; i < 3; ++i) rp[i] = make_float2(0.f, 0.f);
+    constexpr F3 kNone = {0.f, 0.f, 0.f};
+    F3 jin = kNone, jout = kNone, r = kNone;                 // through the end planes; R before the sink's factor
+    F3 sum_c = kNone, sum_dc = kNone, sum_abs = kNone;       // C, |dC|, |C|
+    bool bad[2] = {false, false};                            // not finite
     if (st_d) {
         float hn[2], ln[2];
         const I plane = (I)px * (I)ny;
@@ -280,77 +274,103 @@ __global__ void __launch_bounds__(kS19T) k_step19s(Q19State src, Q19State dst, Q
         }
         if (st_hl) *reinterpret_cast<float4*>(dst.hl + c) = make_float4(hn[0], ln[0], hn[1], ln[1]);
         if (REDUCE) {
+            float Cf[2], dc[2], de[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                if (!on[k]) continue;
-                const bool inlet = x + k == 0, outlet = x + k == nx - 1;
-                const uint32_t rb = rbits[k];
-                if (inlet || outlet || rb) {
-#pragma unroll
-                    for (int i = 1; i < 19; ++i) {
-                        const bool wall = (m[k] >> (i - 1)) & 1u;
-                        const float w = s19_w(i), d = (k == 0 ? dn[i - 1].x : dn[i - 1].y) * inv_d;  // g*_i = w C + d
-                        if (s19_cx(i) < 0 && inlet && !wall && a.bc_in == CL_BC_DIRICHLET) {
-                            float s, e;
-                            two_sum19(a.c_in, -hn[k], s, e);
-                            e += (float)(a.c_in_d - (double)a.c_in);
-                            const float2 f = scaled19(2.0f * w, s, e - ln[k]);
-                            pair_add19(rp[0], f.x, f.y);
-                            pair_add19(rp[0], -2.0f * d, 0.f);
-                        }
-                        if (s19_cx(i) > 0 && outlet && !wall && a.bc_out == CL_BC_DIRICHLET) {
-                            float s, e;
-                            two_sum19(hn[k], -a.c_out, s, e);
-                            e -= (float)(a.c_out_d - (double)a.c_out);
-                            const float2 f = scaled19(2.0f * w, s, e + ln[k]);
-                            pair_add19(rp[1], f.x, f.y);
-                            pair_add19(rp[1], 2.0f * d, 0.f);
-                        }
-                        if (rb & (1u << (i - 1))) {
-                            const float2 f = scaled19(w, hn[k], ln[k]);
-                            pair_add19(rp[2], f.x, f.y);
-                            pair_add19(rp[2], d, 0.f);
-                        }
-                    }
+                Cf[k] = on[k] ? hn[k] + ln[k] : 0.f;
+                two_sum(Cf[k], on[k] ? (k == 0 ? -snap.x : -snap.y) : 0.f, dc[k], de[k]);
+                if (dc[k] < 0.f) {
+                    dc[k] = -dc[k];
+                    de[k] = -de[k];
                 }
-                const float Cf = hn[k] + ln[k];
-                rs[0] += Cf;
-                rs[1] += fabsf(Cf - (k == 0 ? snap.x : snap.y));
-                rs[2] += fabsf(Cf);
-                if (!isfinite(hn[k])) rs[3] += 1.0f;
+                bad[k] = !isfinite(hn[k]);
             }
+            // sum += n / 36 (c - C) of cell k, c being three floats: the equilibrium parts of its links, axis links
+            // counted twice
+            auto equilibrium = [&](F3& sum, float n, float c, const float2& rest, float hi, float lo) {
+                const float w = n * s19_w(7), we = fmaf(n, s19_w(7), -w);
+                float s, e;
+                two_sum(c, -hi, s, e);
+                f3_add_product(sum, w, s);
+                f3_add_product_low(sum, we, s);
+                f3_add_product_low(sum, w, e);
+                f3_add_product_low(sum, w, rest.x);
+                f3_add_product_low(sum, w, -lo);
+                sum.c = fmaf(we, (e + rest.x) - lo, fmaf(w, rest.y, sum.c));
+            };
+            auto count = [](uint32_t links) { return (float)(__popc(links) + __popc(links & 0x3fu)); };
+            // the inlet is cell 0 of a pair, the outlet either; 2 (w c - g*_i) and 2 (g*_i - w c) over their open links
+            if (x == 0 && on[0] && a.bc_in == CL_BC_DIRICHLET) {
+                const uint32_t open = ~m[0] & s19_links(-1);
+                equilibrium(jin, 2.0f * count(open), a.c_in, a.c_in_rest, hn[0], ln[0]);
+#pragma unroll
+                for (int i = 1; i < 19; ++i)
+                    if (s19_cx(i) < 0 && ((open >> (i - 1)) & 1u)) f3_add(jin, -2.0f * (dn[i - 1].x * inv_d));
+            }
+            const int ko = (nx - 1) & 1;
+            if (x == nx - 1 - ko && (ko ? on[1] : on[0]) && a.bc_out == CL_BC_DIRICHLET) {
+                const uint32_t open = ~(ko ? m[1] : m[0]) & s19_links(1);
+                equilibrium(jout, -2.0f * count(open), a.c_out, a.c_out_rest, ko ? hn[1] : hn[0], ko ? ln[1] : ln[0]);
+#pragma unroll
+                for (int i = 1; i < 19; ++i)
+                    if (s19_cx(i) > 0 && ((open >> (i - 1)) & 1u))
+                        f3_add(jout, 2.0f * ((ko ? dn[i - 1].y : dn[i - 1].x) * inv_d));
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint32_t rb = on[k] ? rbits[k] & ((1u << 18) - 1u) : 0u;  // g*_i = w C + d of the catalytic links
+                if (rb == 0u) continue;
+                equilibrium(r, -count(rb), 0.f, make_float2(0.f, 0.f), hn[k], ln[k]);
+#pragma unroll
+                for (int i = 1; i < 19; ++i)
+                    if ((rb >> (i - 1)) & 1u) f3_add(r, (k == 0 ? dn[i - 1].x : dn[i - 1].y) * inv_d);
+            }
+            two_sum(Cf[0], Cf[1], sum_c.a, sum_c.b);
+            two_sum(fabsf(Cf[0]), fabsf(Cf[1]), sum_abs.a, sum_abs.b);
+            two_sum(dc[0], dc[1], sum_dc.a, sum_dc.b);
+            f3_add_low(sum_dc, de[0]);
+            f3_add_low(sum_dc, de[1]);
         }
         if (REDUCE) {
-            if (m[0] & kQ19Active) snap.x = hn[0] + ln[0];
-            if (m[1] & kQ19Active) snap.y = hn[1] + ln[1];
+            if (on[0]) snap.x = hn[0] + ln[0];
+            if (on[1]) snap.y = hn[1] + ln[1];
             *reinterpret_cast<float2*>(a.Csnap + c) = snap;
         }
     }
     if (REDUCE) {
+        // Four sums over the warp in six additions: half of the lanes go on with two of them, then a quarter with one.
+        auto other = [](const F3& v, int o) {
+            return F3{__shfl_xor_sync(0xffffffffu, v.a, o), __shfl_xor_sync(0xffffffffu, v.b, o),
+                      __shfl_xor_sync(0xffffffffu, v.c, o)};
+        };
+        const bool hi16 = lane & 16u, hi8 = lane & 8u;
+        F3 v0 = hi16 ? sum_abs : sum_c, v1 = hi16 ? r : sum_dc;
+        f3_add(v0, other(hi16 ? sum_c : sum_abs, 16));
+        f3_add(v1, other(hi16 ? sum_dc : r, 16));
+        F3 v = hi8 ? v1 : v0;
+        f3_add(v, other(hi8 ? v0 : v1, 8));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-                pair_add19(rp[k], __shfl_xor_sync(0xffffffffu, rp[k].x, o), __shfl_xor_sync(0xffffffffu, rp[k].y, o));
-#pragma unroll
-            for (int k = 0; k < 4; ++k) rs[k] += __shfl_xor_sync(0xffffffffu, rs[k], o);
-        }
-        __shared__ float2 part[kS19T / 32][RED_N];
-        if (lane == 0) {
-            float2* q = part[threadIdx.x >> 5];
-            q[RED_JIN] = rp[0];
-            q[RED_JOUT] = rp[1];
-            q[RED_R] = rp[2];
-            q[RED_SUMC] = make_float2(rs[0], 0.f);
-            q[RED_DC] = make_float2(rs[1], 0.f);
-            q[RED_ABSC] = make_float2(rs[2], 0.f);
-            q[RED_NONFINITE] = make_float2(rs[3], 0.f);
-        }
+        for (int o = 4; o > 0; o >>= 1) f3_add(v, other(v, o));
+        const unsigned nbad = __popc(__ballot_sync(0xffffffffu, bad[0])) + __popc(__ballot_sync(0xffffffffu, bad[1]));
+        __shared__ F3 part[kS19T / 32][4];           // sum C, sum |dC|, sum |C|, R
+        __shared__ F3 ends[2][kS19T / LX];           // the rows' cells of the end planes: one lane each
+        __shared__ unsigned part_bad[kS19T / 32];
+        if ((lane & 7u) == 0) part[threadIdx.x >> 5][lane >> 3] = v;
+        if (lane == 0) part_bad[threadIdx.x >> 5] = nbad;
+        const int row = threadIdx.x / LX, out_lane = (nx - 1) / 2 - blockIdx.x * LX;
+        if (threadIdx.x % LX == 0) ends[0][row] = jin;
+        if (threadIdx.x % LX == (out_lane >= 0 && out_lane < LX ? out_lane : 0)) ends[1][row] = jout;
         __syncthreads();
         if (threadIdx.x < RED_N) {
             double v = 0.0;
-            for (int w = 0; w < kS19T / 32; ++w)
-                v += (double)part[w][threadIdx.x].x + (double)part[w][threadIdx.x].y;
+            if (threadIdx.x == RED_JIN || threadIdx.x == RED_JOUT) {
+                for (int q = 0; q < kS19T / LX; ++q) v += f3_get(ends[threadIdx.x == RED_JOUT][q]);
+            } else if (threadIdx.x == RED_NONFINITE) {
+                for (int w = 0; w < kS19T / 32; ++w) v += (double)part_bad[w];
+            } else {
+                const int k = threadIdx.x == RED_SUMC ? 0 : (threadIdx.x == RED_DC ? 1 : (threadIdx.x == RED_ABSC ? 2 : 3));
+                for (int w = 0; w < kS19T / 32; ++w) v += f3_get(part[w][k]);
+            }
             if (threadIdx.x == RED_R) v *= a.rsink_d;
             const long long blk = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
             a.partials[blk * RED_N + threadIdx.x] = v;
@@ -416,7 +436,7 @@ struct State19PlaneOp {
             const int i = __ffs(left);
             const float w = s19_w(i);
             f3_add_product(acc.r, w, t.hl.x);
-            f3_add_product(acc.r, w, t.hl.y);
+            f3_add_product_low(acc.r, w, t.hl.y);
             f3_add(acc.r, d(i, t.p));
         }
     }
@@ -460,13 +480,13 @@ __global__ void __launch_bounds__(256) k_out19s(Q19State st, Q19Args a, float* _
             const float d = act ? S::ld(dp[(i - 1) * 32]) * (HALF ? a.inv_d : 1.f) : 0.f;
             const float2 f = scaled19(s19_w(i), hl.x, hl.y);
             float t, e;
-            two_sum19(f.x, d, t, e);
+            two_sum(f.x, d, t, e);
             gout[i * N + c] = t + (e + f.y);
             s += d;
         }
         const float2 f = scaled19(s19_w(0), hl.x, hl.y);
         float t, e;
-        two_sum19(f.x, -s, t, e);
+        two_sum(f.x, -s, t, e);
         gout[c] = t + (e + f.y);
     }
 }
