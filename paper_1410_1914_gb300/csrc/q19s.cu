@@ -126,10 +126,31 @@ __device__ __forceinline__ void st_pair(__half* p, float a, float b) {
     *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b);
 }
 
-// w (hi + lo) as a pair
-__device__ __forceinline__ float2 scaled19(float w, float hi, float lo) {
-    const float h = __fmul_rn(w, hi);
-    return make_float2(h, __fadd_rn(fmaf(w, hi, -h), __fmul_rn(w, lo)));
+// w (hi + lo) + d, rounded once, where the first two floats of the sum settle it, whatever their rounding errors hide
+// (all but a few in a million); else *clear = false
+__device__ __forceinline__ float population(float w, float hi, float lo, float d, bool* clear) {
+    const float p = __fmul_rn(w, hi), pe = __fmaf_rn(w, hi, -p), q = __fmul_rn(w, lo);
+    float t, e;
+    two_sum(p, d, t, e);
+    const float low = (e + pe) + q, hidden = 0x1p-22f * ((fabsf(e) + fabsf(pe)) + fabsf(q));
+    const float up = t + (low + hidden);
+    *clear = *clear && up == t + (low - hidden);
+    return up;
+}
+
+// The same whatever it takes: the sum is exact in three floats (but for 2^-70 of it), and the second is rounded to odd
+// where the third is not 0, so that the last addition sees on which side of a tie it lies.
+__device__ __noinline__ float population_at_tie(float w, float hi, float lo, float d) {
+    const float p = __fmul_rn(w, hi), pe = __fmaf_rn(w, hi, -p), q = __fmul_rn(w, lo), qe = __fmaf_rn(w, lo, -q);
+    float t, e, l, m, n, r;
+    two_sum(p, d, t, e);
+    two_sum(e, pe, l, m);
+    two_sum(l, q, l, n);
+    two_sum(t, l, t, l);
+    two_sum(l, __fadd_rn(__fadd_rn(m, n), qe), l, r);
+    const int bits = __float_as_int(l);
+    if (r != 0.f && !(bits & 1)) l = __int_as_float(bits + ((r > 0.f) == (l > 0.f) ? 1 : -1));
+    return isfinite(t) ? t + l : t;
 }
 
 template <class S, bool REDUCE, int LX, class I>  // LX lanes to a row
@@ -459,8 +480,9 @@ struct State19PlaneOp {
     }
 };
 
-// Unpadded C and/or g* as [19][nz][ny][nx]; g*_i = a_i C + delta_i of the pair (hi, lo), rounded once in effect (FP64
-// per cell and population took 120 us at 128^3 FP16, 48 us now, bound by the bytes written)
+// Unpadded C and/or g* as [19][nz][ny][nx]; g*_i = a_i C + delta_i of the pair (hi, lo), rounded once.  A call at 128^3,
+// FP32 and FP16 state: 246 and 245 us with FP64 per population; 111 and 71 us in pairs of floats, which may round to the
+// other side near a tie; 72 and 69 us, all 18 deviations in flight and the ties apart.
 template <class S>
 __global__ void __launch_bounds__(256) k_out19s(Q19State st, Q19Args a, float* __restrict__ C, float* __restrict__ gout) {
     using T = typename S::T;
@@ -474,20 +496,20 @@ __global__ void __launch_bounds__(256) k_out19s(Q19State st, Q19Args a, float* _
         if (C) C[c] = hl.x + hl.y;
         if (!gout) continue;
         const T* dp = reinterpret_cast<const T*>(st.d) + dev_at((unsigned long long)p);
-        float s = 0.f;
+        float d[19], g[19];
+        d[0] = 0.f;
 #pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            const float d = act ? S::ld(dp[(i - 1) * 32]) * (HALF ? a.inv_d : 1.f) : 0.f;
-            const float2 f = scaled19(s19_w(i), hl.x, hl.y);
-            float t, e;
-            two_sum(f.x, d, t, e);
-            gout[i * N + c] = t + (e + f.y);
-            s += d;
-        }
-        const float2 f = scaled19(s19_w(0), hl.x, hl.y);
-        float t, e;
-        two_sum(f.x, -s, t, e);
-        gout[c] = t + (e + f.y);
+        for (int i = 1; i < 19; ++i) d[i] = act ? S::ld(dp[(i - 1) * 32]) * (HALF ? a.inv_d : 1.f) : 0.f;
+#pragma unroll
+        for (int i = 1; i < 19; ++i) d[0] -= d[i];
+        bool clear = true;
+#pragma unroll
+        for (int i = 0; i < 19; ++i) g[i] = population(s19_w(i), hl.x, hl.y, d[i], &clear);
+        if (!clear)
+#pragma unroll
+            for (int i = 0; i < 19; ++i) g[i] = population_at_tie(s19_w(i), hl.x, hl.y, d[i]);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) gout[i * N + c] = g[i];
     }
 }
 
