@@ -32,6 +32,7 @@
 // left is instruction issue: a warp walks on until the last of its 1024 cells
 // has met a wall, 27 steps a way on average where a run is 8.
 #include "chords.cuh"
+#include "device_util.cuh"
 
 #include <math.h>
 
@@ -232,14 +233,6 @@ __device__ __forceinline__ void add_dir(const uint32_t* __restrict__ B, const ui
     add_planes(S, C);
     count_runs<EX, EY, EZ, false>(B, Ad, b, ey, ez, wx, y, z, pore & ~full, 0, C);
     add_planes(S, C);
-}
-
-// 1 / a from the f32 reciprocal r (24 bits) and one third-order step, r (1 + e + e^2) with e = 1 - a r: what is left
-// out is e^3, below 2^-69.  a is a finite positive normal number well inside the f32 range.
-__device__ __forceinline__ double recip(double a) {
-    const double r = (double)__frcp_rn((float)a);
-    const double e = fma(-a, r, 1.0);
-    return fma(r, fma(e, e, e), r);
 }
 
 // D of every cell, and the whole-number sums over the pore cells: tot[0..2] axis, face- and body-diagonal runs,

@@ -87,6 +87,14 @@ __device__ __forceinline__ double f3_get(const F3& s) {
     return isfinite(s.a) ? (double)s.a + lost : (double)s.a;
 }
 
+// 1 / a from the f32 reciprocal r (24 bits) and one third-order step, r (1 + e + e^2) with e = 1 - a r: what is left
+// out is e^3, below 2^-69.  a is a finite positive normal number well inside the f32 range.
+__device__ __forceinline__ double recip(double a) {
+    const double r = (double)__frcp_rn((float)a);
+    const double e = fma(-a, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
 template <int NV>
 __device__ __forceinline__ void warp_sum(double (&v)[NV]) {
 #pragma unroll

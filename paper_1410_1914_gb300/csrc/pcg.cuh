@@ -22,15 +22,22 @@
 // memory but have every block read every other's word while it is awaited:
 // 8.9 and 14.1 us.
 // The sums are formed in a fixed order, so that every block sees the same
-// scalars, takes the same branches, and a solve repeats bit by bit.  One
-// thread of each block turns the sums into alpha and beta: FP64 runs at 1/64
-// of the FP32 rate here, and the two divisions done by every thread cost
-// more than the rest of the iteration (9.4 us an iteration with 512 threads
-// a block, 14.7 us with 1024).
+// scalars, takes the same branches, and a solve repeats bit by bit.  The
+// scalars are FP64, also where the vectors are f32: the threads' f32 sums are
+// added without rounding errors (F3) and converted by the three warps that add
+// up the block.  One thread of each block turns the sums into alpha and beta:
+// FP64 runs at 1/64 of the FP32 rate here, and the two divisions done by every
+// thread cost more than the rest of the iteration (9.4 us an iteration with 512
+// threads a block, 14.7 us with 1024).  Against f32 scalars and f32 sums of a
+// warp, a solve at 96^3 (4003 iterations) takes 51.1 ms instead of 49.5.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include <type_traits>
+
+#include "device_util.cuh"
 
 namespace cl {
 
@@ -171,7 +178,8 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
     constexpr int NW = NT / 32;
     constexpr bool kKeep = K > 0 && K * sizeof(typename Op::Row) <= 192;  // rows stay in registers too
     static_assert(NW % 2 == 0 && NW >= 4, "an even number of warps");
-    __shared__ double sh[3][sizeof(T) == 8 ? NT : NW];
+    using Part = std::conditional_t<sizeof(T) == 8, double, F3>;
+    __shared__ Part sh[3][sizeof(T) == 8 ? NT : NW];
     __shared__ double box[3][kPcgMaxCluster];
     __shared__ double tot[3];
     __shared__ T s_al, s_be;  // alpha, beta of the next iteration
@@ -223,17 +231,20 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
             sh[1][tid] = g1;
             sh[2][tid] = g2;
         } else {
+            // the threads' f32 sums are added without a rounding error (F3) and turned into FP64 by the three warps that
+            // add up the block: half of the lanes go on with g2, a quarter each with g0 and g1
+            const bool hi16 = lane & 16, hi8 = lane & 8;
+            const float x0 = __shfl_xor_sync(0xffffffffu, hi16 ? g0 : g2, 16), x1 = __shfl_xor_sync(0xffffffffu, g1, 16);
+            float s0, e0, s1, e1;
+            two_sum(hi16 ? g2 : g0, x0, s0, e0);
+            two_sum(hi16 ? T(0) : g1, hi16 ? T(0) : x1, s1, e1);
+            F3 v = {hi8 ? s1 : s0, hi8 ? e1 : e0, 0.f};
+            f3_add(v, F3{__shfl_xor_sync(0xffffffffu, hi8 ? s0 : s1, 8), __shfl_xor_sync(0xffffffffu, hi8 ? e0 : e1, 8), 0.f});
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                g0 += __shfl_xor_sync(0xffffffffu, g0, o);
-                g1 += __shfl_xor_sync(0xffffffffu, g1, o);
-                g2 += __shfl_xor_sync(0xffffffffu, g2, o);
-            }
-            if (lane == 0) {
-                sh[0][warp] = (double)g0;
-                sh[1][warp] = (double)g1;
-                sh[2][warp] = (double)g2;
-            }
+            for (int o = 4; o > 0; o >>= 1)
+                f3_add(v, F3{__shfl_xor_sync(0xffffffffu, v.a, o), __shfl_xor_sync(0xffffffffu, v.b, o),
+                             __shfl_xor_sync(0xffffffffu, v.c, o)});
+            if ((lane & 7) == 0 && lane < 24) sh[lane >> 3][warp] = v;
         }
         __syncthreads();
         if (warp < 3) {
@@ -247,7 +258,7 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
                 }
                 v += v2;
             } else {
-                v = lane < NW ? sh[warp][lane] : 0.0;
+                v = lane < NW ? f3_get(sh[warp][lane]) : 0.0;
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -272,51 +283,61 @@ __global__ void __launch_bounds__(NT, 1) k_pcg(Op op, PcgArgs<T> a) {
         R(k, i) = b;
         a.u[i] = d * b;
     });
-    // the scalars are the last warp's: with few cells a block it has none, and forms the reciprocals of the next
-    // iteration's ratios while the others update
+    // the scalars are the last warp's: with few cells a block it has none
     constexpr int kLead = NT - 32;
     PcgOut o = {};
-    T inv_gamma = T(0), inv_alpha = T(0);
+    // Scalars in FP64 for either type.  What lies between a meeting and the next update is a chain of FP64 latencies: with
+    // f32 vectors, whose iterations are short, the two divisions go through f32 reciprocals (recip) side by side.
+    double inv_gamma = 0.0, inv_alpha = 0.0, stop = 0.0;
     bool met = true;
     for (bool start = true;; start = false) {
         met = apply();
         if (!met) break;
-        T gn_t = T(0), alpha = T(0);
+        double gamma = 0.0, alpha = 0.0;
+        bool formed = false;  // the reciprocals of this iteration
         if (tid == kLead) {
             const double gn = tot[0], delta = tot[1], rr = tot[2];
             int go = 1;
-            T be = T(0);
-            gn_t = (T)gn;
+            double be = 0.0;
+            gamma = gn;
             o.rr = rr;
-            if (start) o.rr0 = rr;
-            else ++o.iters;
+            if (start) {
+                o.rr0 = rr;
+                stop = a.tol2 * rr;
+            } else {
+                ++o.iters;
+            }
             if (!isfinite(gn) || !isfinite(rr) || !isfinite(delta)) { o.bad = 1; go = 0; }
             else if (rr == 0.0 || gn == 0.0) { o.bad = start ? 2 : 0; go = 0; }
-            else if ((!start && rr <= a.tol2 * o.rr0) || o.iters >= a.max_iters) go = 0;
+            else if ((!start && rr <= stop) || o.iters >= a.max_iters) go = 0;
             else {
-                // ratios in the vectors' own type
-                T den = (T)delta;
-                if (!start) {
-                    be = gn_t * inv_gamma;
-                    den -= be * gn_t * inv_alpha;
+                be = gn * inv_gamma;
+                double den = delta - be * gn * inv_alpha;
+                const auto clear = [](float v) { return v > 1e-30f && v < 1e30f; };  // recip's range
+                if (sizeof(T) == 4 && clear((float)den) && clear((float)gn)) {
+                    inv_gamma = recip(gn);
+                    alpha = gn * recip(den);
+                    inv_alpha = den * inv_gamma;
+                    formed = true;
+                } else {
+                    if (!(den > 0.0)) {  // rounding has spoilt the recurrence: start it again from this residual
+                        den = delta;
+                        be = 0.0;
+                    }
+                    if (!(den > 0.0) || !(gn > 0.0)) { o.bad = 1; go = 0; }
+                    else alpha = gn / den;
                 }
-                if (!(den > T(0))) {  // rounding has spoilt the recurrence: start it again from this residual
-                    den = (T)delta;
-                    be = T(0);
-                }
-                if (!(den > T(0)) || !(gn > 0.0)) { o.bad = 1; go = 0; }
-                else alpha = gn_t / den;
             }
-            s_al = alpha;
-            s_be = be;
+            s_al = (T)alpha;
+            s_be = (T)be;
             s_go = go;
         }
         __syncthreads();
         if (!s_go) break;
         const T al = s_al, be = s_be;
-        if (tid == kLead) {
-            inv_gamma = T(1) / gn_t;
-            inv_alpha = T(1) / alpha;
+        if (tid == kLead && !formed) {  // while the others update
+            inv_gamma = 1.0 / gamma;
+            inv_alpha = 1.0 / alpha;
         }
         each([&](int k, int i) {
             const T d = D(k, i), r = R(k, i);
