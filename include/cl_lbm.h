@@ -307,7 +307,7 @@ cl_status cl_lbm_solve_krylov(cl_handle h, double tol, int max_iter, long long m
    stalls.
    Each GMRES cycle (at most 10 per correction) restarts from the true
    residual.  Refinement, stopping and certification as in
-   cl_lbm_solve_krylov.
+   cl_lbm_solve_krylov; the correction that is to reach tol goes to 4e-4.
      iterations:       nullable; GMRES iterations (step applications).
      inner_iterations: nullable; conjugate-gradient iterations in all.
    Needs CL_STORAGE_FP32POP, else CL_ERR_STATE.  Allocates 64 f32

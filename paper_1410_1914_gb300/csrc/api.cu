@@ -1119,6 +1119,7 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
     constexpr int kMaxCycles = 10;   // cycles per correction
     constexpr int kMaxCg = 4000;     // CG iterations per preconditioner application
     const double kCgTol = 1e-1;      // relative residual of the inner CG solve (see dsa.cuh)
+    const double kLastTol = 4e-4;    // of the correction that is to reach tol, instead of kKryInnerTol (see dsa.cuh)
     int iters = 0;
     long long cg_total = 0;
     {
@@ -1284,7 +1285,8 @@ cl_status cl_lbm_solve_krylov_dsa(cl_handle h, double tol, int max_iter, long lo
             if (hs.rr <= tol2 * rr0 || iters >= max_iter || !(hs.rr < 0.25 * rr_prev)) break;
             rr_prev = hs.rr;
             CK(launch_dsa_gather(d, cfull, N, c, h->s));
-            CKS(correct(kKryInnerTol));
+            const bool last = hs.rr * kKryInnerTol * kKryInnerTol <= tol2 * rr0;
+            CKS(correct(last ? kLastTol : kKryInnerTol));
             CK(launch_dsa_add64(d, e, 1.0, N, x64, h->s));
         }
         CK(launch_kry_to32(x64, x, L, nblk, h->s));

@@ -39,8 +39,12 @@ cudaError_t launch_dsa_links19(const DsaCells& d, const Q19Args& a, cudaStream_t
 // w = (I - A) z, A the step with zero boundary values and no source
 cudaError_t launch_dsa_apply(const DsaCells& d, const float* z, float* w, cudaStream_t s);
 // z = v + w_i eps, L eps = sum_i v_i (conjugate gradients until r.r is tol2 of its start).  The caller asks
-// for 1e-1: on Knudsen and reactive layers of 24^3 to 96^3 that takes 57 to 120 outer iterations against 58
-// to 119 at 1e-2, half the inner ones (6354 against 10570 at 96^3), and gives the same field to 2e-7.
+// for 1e-1: bulk, Knudsen and reactive layers of 24^3 to 160^3 (D3Q7) and 24^3 to 110^3 (D3Q19) take 16 to 139 outer
+// iterations against 15 to 135 at 1e-2, with 40 to 80 % of the inner ones (4003 against 10323 at 96^3, 9261 against
+// 12406 at 128^3).  What a correction leaves behind then has more of the slow modes, whose error is the largest for a
+// residual: at the same residual the field was off by 4.5e-9 of itself (40 layers of 24^3 to 96^3, solved to 1e-8,
+// geometric mean) against 2.7e-9 at 1e-2.  So the last correction goes on to 4e-4 instead of 1e-3: 2.4e-9, for 6 % of
+// the time (the looser inner solves save 35 %).
 cudaError_t launch_dsa_prec(const DsaCells& d, const float* v, float* z, PcgArgs<float> a, cudaStream_t s);
 // whether the CG of n cells keeps its vectors in memory (PcgArgs x .. w)
 bool dsa_prec_streams(int n);
