@@ -12,8 +12,9 @@
 //                        8 x 16 block of output voxels; the 10 x 18 x 3 input
 //                        halo is staged once per channel chunk and every tap
 //                        is a shifted descriptor into it; weights stream.
-//   k_conv3d_tc          forward with one gather per tap and voxel; used
-//                        where a halo tile does not fit.
+//   k_conv3d_tc          forward with one gather per tap and voxel; taken
+//                        where batch x planes is above 65535, the other two's
+//                        grid limit.
 //   k_conv3d_wgrad_tc    weight gradient: per voxel block the input tile and
 //                        the halo of 16 output-gradient channels are staged
 //                        once and serve all 27 taps, whose accumulators stay in
