@@ -294,10 +294,8 @@ __device__ __forceinline__ void dot2(float a, float b, float& s, float& e) {
     // rounded as written: a contraction to FMA would break the error terms
     const float p = __fmul_rn(a, b);
     const float pe = __fmaf_rn(a, b, -p);
-    const float t = __fadd_rn(s, p);
-    const float z = __fsub_rn(t, s);
-    const float se = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
-    s = t;
+    float se;
+    two_sum(s, p, s, se);
     e = __fadd_rn(e, __fadd_rn(pe, se));
 }
 
@@ -306,10 +304,9 @@ __device__ __forceinline__ void warp_dot2(float& s, float& e) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const float a = __shfl_xor_sync(0xffffffffu, s, o), b = __shfl_xor_sync(0xffffffffu, e, o);
-        const float t = __fadd_rn(s, a);
-        const float z = __fsub_rn(t, s);
-        e = __fadd_rn(__fadd_rn(e, b), __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(a, z)));
-        s = t;
+        float se;
+        two_sum(s, a, s, se);
+        e = __fadd_rn(__fadd_rn(e, b), se);
     }
 }
 

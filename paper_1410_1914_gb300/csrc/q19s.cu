@@ -109,7 +109,6 @@ __device__ __forceinline__ void df_add19(float hi, float lo, float d, float& ho,
 // the residual off by 1e-9.  Four blocks on an SM: its 139 registers left three
 // (100 us).
 constexpr int kS19T = 128;
-constexpr int kS19Cells = 2 * kS19T;
 
 template <class S>
 __device__ __forceinline__ float2 ld_pair(const typename S::T* p);
@@ -160,7 +159,6 @@ __global__ void __launch_bounds__(kS19T, REDUCE ? 4 : 0) k_step19s(Q19State src,
     const int x = (blockIdx.x * LX + threadIdx.x % LX) * 2;
     const int y = blockIdx.y * (kS19T / LX) + threadIdx.x / LX, z = blockIdx.z;
     const int nx = a.nx, ny = a.ny, nz = a.nz, px = a.px;
-    const I NP = (I)a.NP;
     const I c = (I)x + (I)px * ((I)y + (I)ny * (I)z);  // even: px is a multiple of 32
     const bool in_row = x < px && y < ny;
     const uint2 mm = in_row ? *reinterpret_cast<const uint2*>(a.mask + c) : make_uint2(0u, 0u);
