@@ -128,7 +128,8 @@ __device__ __forceinline__ bool may_start(const SchurArgs& a, int ax, int i) {
     return (ax == 1 ? (c / a.nx) % a.ny : c / (a.nx * a.ny)) == 0;
 }
 
-// how many runs there can be, which the allocation follows: a few per hundred cells in open boxes
+// how many runs there can be, which the allocation follows (a run record is 56 bytes; one for every cell and axis was
+// more than the operator)
 __global__ void __launch_bounds__(kSB) k_schur_count(SchurArgs a) {
     int cnt[3] = {0, 0, 0};
     for (int i = blockIdx.x * kSB + threadIdx.x; i < a.n; i += gridDim.x * kSB)
